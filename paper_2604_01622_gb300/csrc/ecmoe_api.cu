@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <cstring>
 #include <cstdarg>
+#include <type_traits>
 
 #include <nvtx3/nvToolsExt.h>
 
@@ -26,7 +27,7 @@ struct ec_ctx {
   size_t ws_bytes = 0;
   // workspace offsets (bytes)
   size_t o_status, o_goff, o_kg, o_koff, o_ST, o_S, o_idx, o_gate, o_slot, o_H, o_A, o_B, o_U,
-      o_O, o_dO, o_dA, o_dB, o_dgate, o_dZ, o_dZb, o_wrpad, o_f32a, o_f32b, o_dXr, o_part, total;
+      o_O, o_dO, o_dA, o_dB, o_dgate, o_dZ, o_dZb, o_wrpad, o_dXr, o_part, total;
   int wr_splits = 1;   // split-K factor of dWr = X^T dZ
   int dg_parts = 1;    // partial sums per gate gradient (tensor-core dU epilogue)
   size_t o_dgsum = 0;  // the gate gradients summed over their partials
@@ -156,7 +157,7 @@ void layout(ec_ctx* c) {
   c->o_idx = take(P * 4);
   c->o_gate = take(P * 4);
   c->o_slot = take(N * E * 4);
-  c->o_H = take(P * d * es);
+  c->o_H = take(use_tc(c) ? P * d * es : 0);   // fp32: rows are gathered from X by the GEMMs
   c->o_A = take(P * F * es);
   c->o_B = take(P * F * es);
   c->o_U = take(P * F * es);
@@ -182,11 +183,6 @@ void layout(ec_ctx* c) {
   c->o_dBsh = take(N * Fs * es);
   // the shared FFN's dWd as two split-K halves (tensor cores; see ffn_backward)
   c->o_shpart = take(use_tc(c) && Fs ? 2 * Fs * d * 4 : 0);
-  // fp32 scratch: SIMT GEMM outputs (fp32 path) and router logits / router dX part
-  const size_t big = std::max(std::max(P * F, P * d), std::max(N * Fs, Fs ? N * d : 0));
-  const size_t f32n = use_tc(c) ? N * E : std::max(big, N * E);
-  c->o_f32a = take(f32n * 4);
-  c->o_f32b = take((use_tc(c) ? 0 : big) * 4);
   c->o_dXr = take(N * d * es);   // the router's part of dX, in the layer dtype
   c->o_colsum = take((size_t)std::max(colsum_scratch_floats((int)N, (int)E),
                                        router_bwd_scratch_floats((int)N, (int)E)) * 4);
@@ -197,7 +193,8 @@ void layout(ec_ctx* c) {
       if (N % s == 0 && N / s >= 256) { c->wr_splits = s; break; }
     c->o_part = take((size_t)2 * c->wr_splits * d * c->Ep * 4);
   } else {
-    c->wr_splits = (int)std::max<size_t>(1, std::min<size_t>(64, N / 512));
+    // one split per 64 tokens (at most 64): X^T dZ has only d*E outputs for the whole GPU
+    c->wr_splits = (int)std::max<size_t>(1, std::min<size_t>(64, N / 64));
     c->o_part = take((size_t)c->wr_splits * d * E * 4);
   }
   c->total = o;
@@ -258,20 +255,21 @@ ec_status upload_groups(ec_ctx* c) {
   return EC_OK;
 }
 
-// ---------------------------------------------------------------- SIMT GEMM helpers
-// Batched over experts: C[e] = A[e] . B[e] (+ beta C[e]).
-SimtGemmArgs sg(const void* A, int64_t a_bs, int64_t a_ms, int64_t a_ks, const void* B,
-                int64_t b_bs, int64_t b_ks, int64_t b_ns, float* C, int64_t c_bs, int64_t c_ms,
-                int M, int N, int K, int batch, float beta = 0.f) {
+// ---------------------------------------------------------------- SIMT GEMM helper
+// One fp32 product over a batch: operand and output pointers with their batch strides and the
+// stride of the dimension that is not contiguous (a_kfast / b_kfast: contiguous along K).
+SimtGemmArgs sg(const float* A, int64_t a_bs, int64_t a_ld, bool a_kfast, const float* B,
+                int64_t b_bs, int64_t b_ld, bool b_kfast, float* C, int64_t c_bs, int64_t c_ld,
+                int M, int N, int K, int batch) {
   SimtGemmArgs a;
-  a.A = A; a.a_bs = a_bs; a.a_ms = a_ms; a.a_ks = a_ks;
-  a.B = B; a.b_bs = b_bs; a.b_ks = b_ks; a.b_ns = b_ns;
-  a.C = C; a.c_bs = c_bs; a.c_ms = c_ms;
-  a.M = M; a.N = N; a.K = K; a.batch = batch; a.splits = 1; a.c_split = 0; a.beta = beta;
+  a.A = A; a.a_bs = a_bs; a.a_ld = a_ld; a.a_kfast = a_kfast;
+  a.B = B; a.b_bs = b_bs; a.b_ld = b_ld; a.b_kfast = b_kfast;
+  a.C = C; a.c_bs = c_bs; a.c_ld = c_ld;
+  a.M = M; a.N = N; a.K = K; a.batch = batch;
   return a;
 }
 
-EType et(const ec_ctx* c) { return c->dtype == EC_BF16 ? EType::BF16 : EType::F32; }
+const float* f32p(const void* p) { return static_cast<const float*>(p); }
 
 // The router weights as the tensor cores read them, [d][Ep] bf16: Wr itself when E is a
 // multiple of 64, else the zero-padded copy the forward pass made.
@@ -298,10 +296,8 @@ ec_status run_route(ec_ctx* c, const void* X, const void* Wr, const float* br, c
               tc_router_softmax(X, Wr, at<void>(c, c->o_wrpad), br, S, ST, slot, N, d, E,
                                 at<int>(c, c->o_status), st));
   } else {
-    float* Z = at<float>(c, c->o_f32a);
-    EC_KERNEL("router_gemm", nz,
-              launch_simt_gemm(sg(X, 0, d, 1, Wr, 0, E, 1, Z, 0, E, N, E, d, 1), et(c), et(c), st));
-    EC_KERNEL("router_softmax", nz, launch_softmax_rows(Z, br, S, ST, slot, N, E, st));
+    EC_KERNEL("router_gemm_softmax", nz,
+              launch_router_f32(f32p(X), f32p(Wr), br, S, ST, slot, N, d, E, st));
   }
   EC_KERNEL("topk", 1,
             launch_topk(ST, N, E, c->G, at<int>(c, c->o_goff), at<int>(c, c->o_kg),
@@ -335,33 +331,29 @@ const FfnNames kRouted = {"gemm_gate_up_swiglu", "gemm_down", "gemm_dgrad_up_swi
 const FfnNames kShared = {"shared_gate_up_swiglu", "shared_down", "shared_dgrad_up_swiglu",
                           "shared_dgrad_h", "shared_wgrad"};
 
-// On the tensor-core path `gate` (per row, or NULL) scales U, so O rows come out gated.
+// Tensor cores: H holds the rows; `gate` (per row, or NULL) scales U, so O rows come out gated.
+// fp32: row m of expert e is row idx[e*M + m] of H (idx NULL: row m), gathered by the GEMM.
 template <typename T>
-ec_status ffn_forward(ec_ctx* c, const FfnNames& nm, const T* H, const void* Wg, const void* Wu,
-                      const void* Wd, T* A, T* B, T* U, T* O, int E, int M, int F,
+ec_status ffn_forward(ec_ctx* c, const FfnNames& nm, const T* H, const int* idx, const void* Wg,
+                      const void* Wu, const void* Wd, T* A, T* B, T* U, T* O, int E, int M, int F,
                       cudaStream_t st, const float* gate = nullptr) {
   const int d = c->d;
   const int64_t P = (int64_t)E * M;
   if (P == 0) return EC_OK;
-  int* status = at<int>(c, c->o_status);
-  if (use_tc(c)) {
+  if constexpr (std::is_same<T, bf16>::value) {
+    int* status = at<int>(c, c->o_status);
     EC_KERNEL(nm.up, 1,
               tc_expert_up(H, Wg, Wu, A, B, U, E, M, d, F, status, st, nullptr, gate, c->tiles));
     EC_KERNEL(nm.down, 1, tc_expert_down(U, Wd, O, E, M, d, F, status, st, nullptr, c->tiles));
   } else {
-    float* Ag = at<float>(c, c->o_f32a);
-    float* Bu = at<float>(c, c->o_f32b);
     const int64_t hs = (int64_t)M * d, ws = (int64_t)d * F, os = (int64_t)M * F;
-    EC_KERNEL(nm.up, 1,
-              launch_simt_gemm(sg(H, hs, d, 1, Wg, ws, F, 1, Ag, os, F, M, F, d, E), et(c), et(c), st));
-    EC_KERNEL(nm.up, 1,
-              launch_simt_gemm(sg(H, hs, d, 1, Wu, ws, F, 1, Bu, os, F, M, F, d, E), et(c), et(c), st));
-    EC_KERNEL("swiglu", 1, launch_swiglu_fwd_ew<T>(Ag, Bu, A, B, U, P * F, st));
-    float* O32 = at<float>(c, c->o_f32a);
+    SimtGemmArgs up = sg(H, idx ? 0 : hs, d, true, f32p(Wg), ws, F, false, A, os, F, M, F, d, E);
+    up.idx = idx; up.idx_bs = M;
+    up.B2 = f32p(Wu); up.C2 = B; up.C3 = U;
+    EC_KERNEL(nm.up, 1, launch_simt_gemm(up, st));
     EC_KERNEL(nm.down, 1,
-              launch_simt_gemm(sg(U, os, F, 1, Wd, (int64_t)F * d, d, 1, O32, hs, d, M, d, F, E),
-                               et(c), et(c), st));
-    EC_KERNEL("convert_o", 1, launch_convert<T>(O32, O, P * d, st));
+              launch_simt_gemm(sg(U, os, F, true, f32p(Wd), ws, d, false, O, hs, d, M, d, F, E),
+                               st));
   }
   return EC_OK;
 }
@@ -371,13 +363,15 @@ ec_status ffn_forward(ec_ctx* c, const FfnNames& nm, const T* H, const void* Wg,
 // On the tensor-core path with `gate`, dO holds the ungated rows dY[idx] and U the gated
 // ones (as ffn_forward wrote them): dU = gate * dO.Wd^T, dWd = U^T.dO, and the gate
 // gradients <dO.Wd^T, silu(A) B> land in dgate_part (c->dg_parts partials, stride E*M).
+// fp32: H is gathered through idx as in ffn_forward.
 // dwd_split: optional scratch of 2*F*d floats for the single-FFN case (E = 1, the shared
 // experts), whose dWd = U^T.dO has few output tiles for the whole GPU and a K loop over all
 // M rows: the rows are split into two halves computed as two batch entries at once and
 // summed in order afterwards.
 template <typename T>
-ec_status ffn_backward(ec_ctx* c, const FfnNames& nm, const T* dO, const T* H, const T* A,
-                       const T* B, const T* U, const void* Wg, const void* Wu, const void* Wd,
+ec_status ffn_backward(ec_ctx* c, const FfnNames& nm, const T* dO, const T* H, const int* idx,
+                       const T* A, const T* B, const T* U, const void* Wg, const void* Wu,
+                       const void* Wd,
                        T* dA, T* dB, T* dH, float* dWg, float* dWu, float* dWd, int E, int M, int F,
                        cudaStream_t st, const float* gate = nullptr, float* dgate_part = nullptr,
                        float* dwd_split = nullptr) {
@@ -389,8 +383,8 @@ ec_status ffn_backward(ec_ctx* c, const FfnNames& nm, const T* dO, const T* H, c
     EC_CUDA(cudaMemsetAsync(dWd, 0, (size_t)E * d * F * 4, st), "zero dWd");
     return EC_OK;
   }
-  int* status = at<int>(c, c->o_status);
-  if (use_tc(c)) {
+  if constexpr (std::is_same<T, bf16>::value) {
+    int* status = at<int>(c, c->o_status);
     EC_KERNEL(nm.dgrad_up, 1,
               tc_expert_dgrad_up(dO, Wd, A, B, dA, dB, E, M, d, F, status, st, nullptr, gate,
                                  dgate_part, P, c->tiles));
@@ -412,32 +406,23 @@ ec_status ffn_backward(ec_ctx* c, const FfnNames& nm, const T* dO, const T* H, c
                                 c->tiles));
     }
   } else {
-    float* dU32 = at<float>(c, c->o_f32a);
-    float* dH32 = at<float>(c, c->o_f32b);
     const int64_t hs = (int64_t)M * d, fs = (int64_t)M * F, wgs = (int64_t)d * F;
-    // dU = dO . Wd^T : B[k=i][n=j] = Wd[j][i]
-    EC_KERNEL(nm.dgrad_up, 1,
-              launch_simt_gemm(sg(dO, hs, d, 1, Wd, (int64_t)F * d, 1, d, dU32, fs, F, M, F, d, E),
-                               et(c), et(c), st));
-    EC_KERNEL("swiglu_bwd", 1, launch_swiglu_bwd_ew<T>(dU32, A, B, dA, dB, P * F, st));
+    // dU = dO . Wd^T (B[k=i][n=j] = Wd[j][i]), its SwiGLU backward in the epilogue
+    SimtGemmArgs du = sg(dO, hs, d, true, f32p(Wd), wgs, d, true, dA, fs, F, M, F, d, E);
+    du.C2 = dB; du.E1 = A; du.E2 = B;
+    EC_KERNEL(nm.dgrad_up, 1, launch_simt_gemm(du, st));
     // dH = dA . Wg^T + dB . Wu^T
-    EC_KERNEL(nm.dgrad_h, 1,
-              launch_simt_gemm(sg(dA, fs, F, 1, Wg, wgs, 1, F, dH32, hs, d, M, d, F, E),
-                               et(c), et(c), st));
-    EC_KERNEL(nm.dgrad_h, 1,
-              launch_simt_gemm(sg(dB, fs, F, 1, Wu, wgs, 1, F, dH32, hs, d, M, d, F, E, 1.f),
-                               et(c), et(c), st));
-    EC_KERNEL("convert_dh", 1, launch_convert<T>(dH32, dH, P * d, st));
+    SimtGemmArgs dh = sg(dA, fs, F, true, f32p(Wg), wgs, F, true, dH, hs, d, M, d, F, E);
+    dh.segs = 2; dh.A2 = dB; dh.B2 = f32p(Wu);
+    EC_KERNEL(nm.dgrad_h, 1, launch_simt_gemm(dh, st));
     // dWd = U^T dO ; dWg = H^T dA ; dWu = H^T dB   (A[m][k] = U[k][m])
     EC_KERNEL(nm.wgrad, 1,
-              launch_simt_gemm(sg(U, fs, 1, F, dO, hs, d, 1, dWd, (int64_t)F * d, d, F, d, M, E),
-                               et(c), et(c), st));
-    EC_KERNEL(nm.wgrad, 1,
-              launch_simt_gemm(sg(H, hs, 1, d, dA, fs, F, 1, dWg, wgs, F, d, F, M, E),
-                               et(c), et(c), st));
-    EC_KERNEL(nm.wgrad, 1,
-              launch_simt_gemm(sg(H, hs, 1, d, dB, fs, F, 1, dWu, wgs, F, d, F, M, E),
-                               et(c), et(c), st));
+              launch_simt_gemm(sg(U, fs, F, false, dO, hs, d, false, dWd, wgs, d, F, d, M, E),
+                               st));
+    SimtGemmArgs dw = sg(H, idx ? 0 : hs, d, false, dA, fs, F, false, dWg, wgs, F, d, F, M, E);
+    dw.idx = idx; dw.idx_bs = M;
+    dw.B2 = dB; dw.C2 = dWu;
+    EC_KERNEL(nm.wgrad, 1, launch_simt_gemm(dw, st));
   }
   return EC_OK;
 }
@@ -459,12 +444,11 @@ ec_status run_forward(ec_ctx* c, const void* X, const void* Wg, const void* Wu, 
   const int64_t P = (int64_t)E * M;
   const int pz = P > 0;
   const T* Xt = static_cast<const T*>(X);
-  T* H = at<T>(c, c->o_H);
   T* O = at<T>(c, c->o_O);
   const T* Osh = nullptr;
   if (Fs > 0) {
     T* o = at<T>(c, c->o_Osh);
-    EC_TRY(ffn_forward<T>(c, kShared, Xt, Wgs, Wus, Wds, at<T>(c, c->o_Ash), at<T>(c, c->o_Bsh),
+    EC_TRY(ffn_forward<T>(c, kShared, Xt, nullptr, Wgs, Wus, Wds, at<T>(c, c->o_Ash), at<T>(c, c->o_Bsh),
                           at<T>(c, c->o_Ush), o, 1, N, Fs, st));
     Osh = o;
   }
@@ -473,9 +457,15 @@ ec_status run_forward(ec_ctx* c, const void* X, const void* Wg, const void* Wu, 
   // tensor cores: the gate is applied in the gate/up epilogue (O rows come out gated)
   const bool fused_gate = use_tc(c);
   // token-major: each X row is read once and written to the rows of the experts that chose it
-  EC_KERNEL("gather", N > 0 && pz,
-            launch_scatter_rows<T>(Xt, at<int>(c, c->o_slot), H, N, E, M, d, st));
-  EC_TRY(ffn_forward<T>(c, kRouted, H, Wg, Wu, Wd, at<T>(c, c->o_A), at<T>(c, c->o_B),
+  // (fp32: the GEMMs gather the rows themselves)
+  const T* H = Xt;
+  if constexpr (std::is_same<T, bf16>::value) {
+    T* h = at<T>(c, c->o_H);
+    EC_KERNEL("gather", N > 0 && pz,
+              launch_scatter_rows<T>(Xt, at<int>(c, c->o_slot), h, N, E, M, d, st));
+    H = h;
+  }
+  EC_TRY(ffn_forward<T>(c, kRouted, H, idx, Wg, Wu, Wd, at<T>(c, c->o_A), at<T>(c, c->o_B),
                         at<T>(c, c->o_U), O, E, M, F, st, fused_gate ? gate : nullptr));
   EC_KERNEL("combine", N > 0,
             launch_combine<T>(O, fused_gate ? nullptr : gate, at<int>(c, c->o_slot),
@@ -503,16 +493,17 @@ ec_status run_backward(ec_ctx* c, const void* dY, void* dX, float* dWr, float* d
   const float* gate = at<float>(c, c->o_gate);
   const int* slot = at<int>(c, c->o_slot);
 
-  if (use_tc(c)) {
+  if constexpr (std::is_same<T, bf16>::value) {
     // dO holds dY[idx] ungated; the dU epilogue applies the gate and forms dgate
     EC_KERNEL("gather_dy", N > 0 && pz, launch_scatter_rows<T>(dYt, slot, dO, N, E, M, d, st));
-    EC_TRY(ffn_backward<T>(c, kRouted, dO, at<T>(c, c->o_H), at<T>(c, c->o_A), at<T>(c, c->o_B),
-                           at<T>(c, c->o_U), c->Wg, c->Wu, c->Wd, at<T>(c, c->o_dA),
-                           at<T>(c, c->o_dB), dH, dWg, dWu, dWd, E, M, F, st, gate, dgate));
+    EC_TRY(ffn_backward<T>(c, kRouted, dO, at<T>(c, c->o_H), idx, at<T>(c, c->o_A),
+                           at<T>(c, c->o_B), at<T>(c, c->o_U), c->Wg, c->Wu, c->Wd,
+                           at<T>(c, c->o_dA), at<T>(c, c->o_dB), dH, dWg, dWu, dWd, E, M, F, st,
+                           gate, dgate));
   } else {
     EC_KERNEL("bwd_gather_scale", pz,
               launch_bwd_gather_scale<T>(dYt, O, idx, gate, dO, dgate, P, d, st));
-    EC_TRY(ffn_backward<T>(c, kRouted, dO, at<T>(c, c->o_H), at<T>(c, c->o_A), at<T>(c, c->o_B),
+    EC_TRY(ffn_backward<T>(c, kRouted, dO, f32p(c->X), idx, at<T>(c, c->o_A), at<T>(c, c->o_B),
                            at<T>(c, c->o_U), c->Wg, c->Wu, c->Wd, at<T>(c, c->o_dA),
                            at<T>(c, c->o_dB), dH, dWg, dWu, dWd, E, M, F, st));
   }
@@ -520,7 +511,7 @@ ec_status run_backward(ec_ctx* c, const void* dY, void* dX, float* dWr, float* d
   if (Fs > 0) {
     // shared experts: dO is dY itself (no gate), the input gradient goes into the dX scatter
     T* dh = at<T>(c, c->o_Osh);
-    EC_TRY(ffn_backward<T>(c, kShared, dYt, static_cast<const T*>(c->X), at<T>(c, c->o_Ash),
+    EC_TRY(ffn_backward<T>(c, kShared, dYt, static_cast<const T*>(c->X), nullptr, at<T>(c, c->o_Ash),
                            at<T>(c, c->o_Bsh), at<T>(c, c->o_Ush), c->Wgs, c->Wus, c->Wds,
                            at<T>(c, c->o_dAsh), at<T>(c, c->o_dBsh), dh, dWgs, dWus, dWds, 1, N,
                            Fs, st, nullptr, nullptr,
@@ -565,16 +556,15 @@ ec_status run_backward(ec_ctx* c, const void* dY, void* dX, float* dWr, float* d
     else
       EC_KERNEL("softmax_bwd", nz, launch_softmax_bwd(S, slot, dgate, dZ, nullptr, N, E, E, M, st));
     EC_KERNEL("router_dgrad_gemm", nz,
-              launch_simt_gemm(sg(dZ, 0, E, 1, c->Wr, 0, 1, E, reinterpret_cast<float*>(dXr), 0, d,
-                                  N, d, E, 1),
-                               EType::F32,
-                               et(c), st));
+              launch_simt_gemm(sg(dZ, 0, E, true, f32p(c->Wr), 0, E, true,
+                                  reinterpret_cast<float*>(dXr), 0, d, N, d, E, 1),
+                               st));
     EC_KERNEL("dx_combine", nz,
               launch_dx_combine<T>(dH, slot, dXr, res, dHsh, static_cast<T*>(dX), N, E, M, d, st));
-    SimtGemmArgs a = sg(c->X, 0, 1, d, dZ, 0, E, 1, part, 0, E, d, E, N, 1);
+    SimtGemmArgs a = sg(f32p(c->X), 0, d, false, dZ, 0, E, false, part, 0, E, d, E, N, 1);
     a.splits = c->wr_splits;
     a.c_split = (int64_t)d * E;
-    EC_KERNEL("router_wgrad_gemm", 1, launch_simt_gemm(a, et(c), EType::F32, st));
+    EC_KERNEL("router_wgrad_gemm", 1, launch_simt_gemm(a, st));
     EC_KERNEL("router_wgrad_reduce", 1,
               launch_reduce_splits(part, dWr, (int64_t)d * E, c->wr_splits, st));
   }

@@ -1,94 +1,539 @@
-// Batched fp32 CUDA-core GEMM with arbitrary operand strides.
+// Batched fp32 CUDA-core GEMMs of the fp32 path (tensor-core TF32 would miss its 1e-4 bound).
 //
-// Serves the fp32 path of the layer (where tensor-core TF32 would miss a 1e-4 relative
-// error bound) and the small router-gradient products dZ.Wr^T and X^T.dZ. Tiles of
-// 64x64 outputs, 16-deep K slices staged in shared memory, 4x4 outputs per thread; each
-// operand tile is loaded along whichever of its two dimensions is contiguous.
+// C[b] = A[b] . B[b], one output tile per CTA. Both operands may be contiguous along K or
+// along their other dimension; k-slices are fetched with 16-byte loads one slice ahead into
+// registers, stored k-major into one of two shared buffers (one barrier per slice), and each
+// thread accumulates a TM x TN block in column pairs (one paired FMA per two products). Every
+// output is one chain of fused multiply-adds in ascending k, so the tile shape does not change
+// a bit of the result.
+//
+// What bounds it: the FMA pipes. With 8 x 8 outputs per thread they are busy 69% of an SM's
+// active cycles (ncu; the most frequent stall is the pipe itself), and 40-46 TFLOP/s come out of
+// the 75 that the pipes allow, the rest lost to the last wave and the edge tiles. The scalar
+// 4 x 4 kernel with 4-byte loads before it ran 22 TFLOP/s on the same shapes (16 experts of 1000
+// rows, d 500, d_ff 364). The row gather of H = X[idx], the SwiGLU and its derivative, and the
+// second product of dH are part of the same launches, so no intermediate is written that a
+// later kernel only reads back: that layer's step 2820 -> 1424 us, a 256-token layer's (24
+// kernels, now 15) 195 -> 89-96 us.
 #include "common.cuh"
 #include "kernels.h"
 
 namespace ecmoe {
 
 namespace {
-constexpr int BM = 64, BN = 64, BK = 16;
 
-template <typename T>
-__device__ __forceinline__ float ld(const void* p, int64_t i) {
-  return to_f32(reinterpret_cast<const T*>(p)[i]);
+enum SimtEpi : int {
+  SIMT_PLAIN = 0,       // C
+  SIMT_DUAL = 1,        // column halves: C = A.B, C2 = A.B2
+  SIMT_SWIGLU_FWD = 2,  // column halves a = A.B, b = A.B2: C = a, C2 = b, C3 = silu(a) b
+  SIMT_SWIGLU_BWD = 3   // acc = dU, with E1 = A, E2 = B: C = dA, C2 = dB
+};
+
+__device__ __forceinline__ uint64_t pair2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void split2(uint64_t r, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(r));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
 }
 
-template <typename TA, typename TB>
-__global__ void __launch_bounds__(256) simt_gemm_kernel(SimtGemmArgs p) {
-  __shared__ float As[BK][BM + 4];
-  __shared__ float Bs[BK][BN + 4];
-  const int tid = threadIdx.x;
-  const int bz = blockIdx.z;
-  const int b = bz / p.splits, s = bz % p.splits;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  const int kchunk = (p.K + p.splits - 1) / p.splits;
-  const int kb = s * kchunk, ke = min(p.K, kb + kchunk);
-  const int64_t a_off = (int64_t)b * p.a_bs, b_off = (int64_t)b * p.b_bs;
-  const bool a_kfast = p.a_ks == 1, b_nfast = p.b_ns == 1;
-  const int ty = tid >> 4, tx = tid & 15;
-  float acc[4][4] = {};
-  for (int k0 = kb; k0 < ke; k0 += BK) {
+// Four elements of a chunk whose contiguous dimension is at `i` of `n`: one 16-byte load when
+// `vec` (n, the stride and the base are multiples of 16 bytes, so a chunk is in or out whole).
+__device__ __forceinline__ void load4(float (&v)[4], const float* p, int i, int n, bool vec) {
+  if (vec) {
+    const float4 q = i < n ? __ldg(reinterpret_cast<const float4*>(p)) : make_float4(0, 0, 0, 0);
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+  } else {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int l = tid + i * 256;
-      int mm, kk;
-      if (a_kfast) { kk = l % BK; mm = l / BK; } else { mm = l % BM; kk = l / BM; }
-      const int gm = m0 + mm, gk = k0 + kk;
-      As[kk][mm] = (gm < p.M && gk < ke) ? ld<TA>(p.A, a_off + gm * p.a_ms + gk * p.a_ks) : 0.f;
-      int nn, kk2;
-      if (b_nfast) { nn = l % BN; kk2 = l / BN; } else { kk2 = l % BK; nn = l / BK; }
-      const int gn = n0 + nn, gk2 = k0 + kk2;
-      Bs[kk2][nn] = (gn < p.N && gk2 < ke) ? ld<TB>(p.B, b_off + gk2 * p.b_ks + gn * p.b_ns) : 0.f;
+    for (int j = 0; j < 4; ++j) v[j] = i + j < n ? __ldg(p + j) : 0.f;
+  }
+}
+
+// G consecutive values at dst (vec: 4 * G bytes aligned and wholly inside), else guarded.
+template <int G>
+__device__ __forceinline__ void store_group(float* dst, const float* v, int n, int N, bool vec) {
+  if (vec) {
+    if (n < N) {
+      if constexpr (G == 4) *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+      else *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
     }
-    __syncthreads();
+  } else {
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float av[4], bv[4];
+    for (int j = 0; j < G; ++j)
+      if (n + j < N) dst[j] = v[j];
+  }
+}
+
+// A_K / B_K: the operand is contiguous along k. Thread (ty, tx) of TY x TX owns rows in RG
+// groups of RW and columns in CG groups of CW, spread evenly over the tile (so with two B
+// operands, each half of the tile's columns, it holds the same columns of both products).
+template <int BM, int BN, int BK, int TM, int TN, int MINB, bool A_K, bool B_K, int EPI>
+__global__ void __launch_bounds__(BM / TM * (BN / TN), MINB) simt_gemm_kernel(const SimtGemmArgs p) {
+  constexpr int TX = BN / TN, TY = BM / TM, NT = TX * TY;
+  constexpr bool DUAL = EPI == SIMT_DUAL || EPI == SIMT_SWIGLU_FWD;
+  constexpr int RW = TM >= 4 ? 4 : 2, RG = TM / RW;   // rows per group, groups per thread
+  constexpr int CW = TN >= 8 ? 4 : 2, CG = TN / CW;   // columns per group, groups per thread
+  constexpr int KQ = BK / 4;
+  constexpr int LDA = BM + 4, LDB = BN + 4;
+  constexpr int NA = BM * BK / 4 / NT, NB = BN * BK / 4 / NT;   // 16-byte chunks per thread
+  static_assert(NA * NT * 4 == BM * BK && NB * NT * 4 == BN * BK, "chunks divide evenly");
+  static_assert(KQ % 2 == 0 && BM % 16 == 0 && BN % 16 == 0 && TX % 8 == 0 && TY % 4 == 0 &&
+                CG % 2 == 0, "chunk and thread maps");
+  __shared__ __align__(16) float As[2][BK][LDA];
+  __shared__ __align__(16) float Bs[2][BK][LDB];
+  // a warp covers 4 x 8 threads of the block, so its 16-byte reads of Bs touch one 128-byte line
+  // and those of As four addresses
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ty = warp / (TX / 8) * 4 + (lane >> 3), tx = warp % (TX / 8) * 8 + (lane & 7);
+  const int b = blockIdx.z / p.splits, sp = blockIdx.z % p.splits;
+  const int m0 = blockIdx.y * BM;
+  const int n0 = blockIdx.x * (DUAL ? BN / 2 : BN);
+  const int kb = sp * p.kchunk, ke = min(p.K, kb + p.kchunk);
+  const int ksl = (ke - kb + BK - 1) / BK;            // k-slices of one product
+  const int nsl = p.segs * ksl;
+  const int* idx = p.idx ? p.idx + (int64_t)b * p.idx_bs : nullptr;
+  const float* A0 = p.A + (int64_t)b * p.a_bs;
+  const float* A1 = p.A2 + (int64_t)b * p.a_bs;
+  const float* B0 = p.B + (int64_t)b * p.b_bs;
+  const float* B1 = p.B2 + (int64_t)b * p.b_bs;
+  const bool va = p.vec_a, vb = p.vec_b;
+
+  // Chunk c of an operand contiguous along k: a warp takes 16 rows x 2 chunks, so its loads use
+  // whole 32-byte sectors and its transposed 4-byte stores fall into 32 different banks
+  // (rows of 4 LDA floats are 16 banks apart).
+  auto ck = [](int c) { return ((c & 1) + 2 * ((c >> 5) % (KQ / 2))) * 4; };
+  auto cm = [](int c) { return (c >> 5) / (KQ / 2) * 16 + ((c & 31) >> 1); };
+
+  // A rows of this thread's chunks (gathered through idx where given): fixed over the k loop
+  int64_t arow[A_K ? NA : 1];
+  if constexpr (A_K) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) av[i] = As[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) bv[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+    for (int i = 0; i < NA; ++i) {
+      const int gm = m0 + cm(tid + i * NT);
+      arow[i] = gm < p.M ? (int64_t)(idx ? __ldg(idx + gm) : gm) * p.a_ld : -1;
     }
+  }
+  float ra[NA][4], rb[NB][4];
+  auto fetch = [&](int s) {
+    const bool second = s >= ksl;
+    const int k0 = kb + (second ? s - ksl : s) * BK;
+    const float* Ab = second ? A1 : A0;
+    const float* Bb = second && !DUAL ? B1 : B0;
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+      const int c = tid + i * NT;
+      if constexpr (A_K) {
+        const int gk = k0 + ck(c);
+        load4(ra[i], Ab + arow[i] + gk, arow[i] >= 0 ? gk : ke, ke, va);
+      } else {
+        const int gk = k0 + c / (BM / 4), gm = m0 + (c % (BM / 4)) * 4;
+        const bool ok = gk < ke;
+        const int64_t r = ok ? (idx ? __ldg(idx + gk) : gk) : 0;
+        load4(ra[i], Ab + r * p.a_ld + gm, ok ? gm : p.M, p.M, va);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      const int c = tid + i * NT;
+      const int nn = B_K ? cm(c) : (c % (BN / 4)) * 4;   // column of the tile
+      const bool h1 = DUAL && nn >= BN / 2;
+      const float* Bp = h1 ? B1 : Bb;
+      const int gn = n0 + (h1 ? nn - BN / 2 : nn);
+      if constexpr (B_K) {
+        const int gk = k0 + ck(c);
+        load4(rb[i], Bp + (int64_t)gn * p.b_ld + gk, gn < p.N ? gk : ke, ke, vb);
+      } else {
+        const int gk = k0 + c / (BN / 4);
+        load4(rb[i], Bp + (int64_t)gk * p.b_ld + gn, gk < ke ? gn : p.N, p.N, vb);
+      }
+    }
+  };
+  auto put = [&](int buf) {
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+      const int c = tid + i * NT;
+      if constexpr (A_K) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) As[buf][ck(c) + j][cm(c)] = ra[i][j];
+      } else {
+        *reinterpret_cast<float4*>(&As[buf][c / (BM / 4)][(c % (BM / 4)) * 4]) =
+            make_float4(ra[i][0], ra[i][1], ra[i][2], ra[i][3]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      const int c = tid + i * NT;
+      if constexpr (B_K) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) Bs[buf][ck(c) + j][cm(c)] = rb[i][j];
+      } else {
+        *reinterpret_cast<float4*>(&Bs[buf][c / (BN / 4)][(c % (BN / 4)) * 4]) =
+            make_float4(rb[i][0], rb[i][1], rb[i][2], rb[i][3]);
+      }
+    }
+  };
+
+  float* C = p.C + (int64_t)b * p.c_bs + (int64_t)sp * p.c_split;
+  float* C2 = (EPI == SIMT_PLAIN) ? nullptr : p.C2 + (int64_t)b * p.c_bs;
+  float* C3 = (EPI == SIMT_SWIGLU_FWD) ? p.C3 + (int64_t)b * p.c_bs : nullptr;
+  auto row_of = [&](int i) { return m0 + (i / RW) * (BM / RG) + ty * RW + i % RW; };
+  // column group h (of CG; of a dual tile, of the CG / 2 in each half)
+  auto col_of = [&](int h) { return n0 + h * (BN / CG) + tx * CW; };
+
+  uint64_t acc[TM][TN / 2];
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0ull;
+
+  if (nsl > 0) {
+    fetch(0);
+    put(0);
+  }
+  __syncthreads();
+  for (int s = 0; s < nsl; ++s) {
+    const int buf = s & 1;
+    if (s + 1 < nsl) fetch(s + 1);
+    if (EPI == SIMT_PLAIN && s == ksl && s > 0) {
+      // the first product is complete: it waits in C (this thread's own elements) and the
+      // second one starts from zero, so the two are rounded and added as separate sums
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const int gm = row_of(i);
+        float v[TN];
+#pragma unroll
+        for (int j = 0; j < TN / 2; ++j) {
+          split2(acc[i][j], v[2 * j], v[2 * j + 1]);
+          acc[i][j] = 0ull;
+        }
+        if (gm < p.M)
+#pragma unroll
+          for (int h = 0; h < CG; ++h)
+            store_group<CW>(C + (int64_t)gm * p.c_ld + col_of(h), v + h * CW, col_of(h), p.N,
+                            p.vec_c);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < BK; ++k) {
+      float a[TM];
+      uint64_t bb[TN / 2];
+#pragma unroll
+      for (int g = 0; g < RG; ++g) {
+        const float* src = &As[buf][k][g * (BM / RG) + ty * RW];
+        if constexpr (RW == 4) {
+          const float4 q = *reinterpret_cast<const float4*>(src);
+          a[g * RW] = q.x; a[g * RW + 1] = q.y; a[g * RW + 2] = q.z; a[g * RW + 3] = q.w;
+        } else {
+          const float2 q = *reinterpret_cast<const float2*>(src);
+          a[g * RW] = q.x; a[g * RW + 1] = q.y;
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < CG; ++h) {
+        const float* src = &Bs[buf][k][h * (BN / CG) + tx * CW];
+        if constexpr (CW == 4) {
+          const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(src);
+          bb[2 * h] = q.x;
+          bb[2 * h + 1] = q.y;
+        } else {
+          bb[h] = *reinterpret_cast<const unsigned long long*>(src);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const uint64_t aa = pair2(a[i], a[i]);
+#pragma unroll
+        for (int j = 0; j < TN / 2; ++j) acc[i][j] = fma2(aa, bb[j], acc[i][j]);
+      }
+    }
+    // the other buffer was last read before the previous slice's barrier
+    if (s + 1 < nsl) put(buf ^ 1);
     __syncthreads();
   }
-  float* C = p.C + (int64_t)b * p.c_bs + (p.splits > 1 ? (int64_t)s * p.c_split : 0);
+
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int gm = m0 + ty * 4 + i;
+  for (int i = 0; i < TM; ++i) {
+    const int gm = row_of(i);
     if (gm >= p.M) continue;
+    float v[TN];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gn = n0 + tx * 4 + j;
-      if (gn >= p.N) continue;
-      float v = acc[i][j];
-      float* c = C + (int64_t)gm * p.c_ms + gn;
-      if (p.splits == 1 && p.beta != 0.f) v += p.beta * *c;
-      *c = v;
+    for (int j = 0; j < TN / 2; ++j) split2(acc[i][j], v[2 * j], v[2 * j + 1]);
+    const int64_t ro = (int64_t)gm * p.c_ld;
+    if constexpr (EPI == SIMT_PLAIN) {
+#pragma unroll
+      for (int h = 0; h < CG; ++h) {
+        const int n = col_of(h);
+        if (p.segs == 2)
+#pragma unroll
+          for (int j = 0; j < CW; ++j)
+            if (n + j < p.N) v[h * CW + j] += C[ro + n + j];
+        store_group<CW>(C + ro + n, v + h * CW, n, p.N, p.vec_c);
+      }
+    } else if constexpr (DUAL) {
+#pragma unroll
+      for (int h = 0; h < CG / 2; ++h) {
+        const int n = col_of(h);
+        const float* x = v + h * CW;
+        const float* y = v + (CG / 2 + h) * CW;
+        store_group<CW>(C + ro + n, x, n, p.N, p.vec_c);
+        store_group<CW>(C2 + ro + n, y, n, p.N, p.vec_c);
+        if constexpr (EPI == SIMT_SWIGLU_FWD) {
+          float u[CW];
+#pragma unroll
+          for (int j = 0; j < CW; ++j) u[j] = x[j] * sigmoidf_(x[j]) * y[j];
+          store_group<CW>(C3 + ro + n, u, n, p.N, p.vec_c);
+        }
+      }
+    } else {
+      const float* E1 = p.E1 + (int64_t)b * p.c_bs + ro;
+      const float* E2 = p.E2 + (int64_t)b * p.c_bs + ro;
+#pragma unroll
+      for (int h = 0; h < CG; ++h) {
+        const int n = col_of(h);
+        float da[CW], db[CW];
+#pragma unroll
+        for (int j = 0; j < CW; ++j) {
+          const float aj = n + j < p.N ? __ldg(E1 + n + j) : 0.f;
+          const float bj = n + j < p.N ? __ldg(E2 + n + j) : 0.f;
+          const float du = v[h * CW + j], sg = sigmoidf_(aj);
+          da[j] = du * bj * sg * (1.0f + aj * (1.0f - sg));
+          db[j] = du * aj * sg;
+        }
+        store_group<CW>(C + ro + n, da, n, p.N, p.vec_c);
+        store_group<CW>(C2 + ro + n, db, n, p.N, p.vec_c);
+      }
     }
   }
+}
+
+int simt_sms() {
+  static int n = 0;
+  if (!n) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (n <= 0) n = 1;
+  }
+  return n;
+}
+
+template <int BM, int BN, int BK, int TM, int TN, int MINB, bool A_K, bool B_K, int EPI>
+cudaError_t go(const SimtGemmArgs& a, cudaStream_t st) {
+  constexpr bool DUAL = EPI == SIMT_DUAL || EPI == SIMT_SWIGLU_FWD;
+  constexpr int cols = DUAL ? BN / 2 : BN;
+  const dim3 grid((a.N + cols - 1) / cols, (a.M + BM - 1) / BM, a.batch * a.splits);
+  simt_gemm_kernel<BM, BN, BK, TM, TN, MINB, A_K, B_K, EPI>
+      <<<grid, BM / TM * (BN / TN), 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+// Tile shape: the one whose busiest SM has the least work, tiles per SM (rounded up) times the
+// tile's outputs times its measured cost per output against 128 x 128 (the shapes below, on
+// 16 problems of M 1000 and M 96, N 364 and 500, K 364 to 1000: 64 x 128 1.02-1.12, 64 x 64
+// 1.14, 32 x 32 2.1-2.4; 16 x 8 outputs per thread were slower in every shape). It takes 64 x 128
+// where 128 x 128 leaves a nearly empty last wave (1000 x 500 x 364: 129 against 141 us) and
+// the small tiles for a few rows per expert (96 x 500 x 364: 27 against 43 us).
+template <bool A_K, bool B_K, int EPI>
+cudaError_t pick(const SimtGemmArgs& a, cudaStream_t st) {
+  constexpr int half = (EPI == SIMT_DUAL || EPI == SIMT_SWIGLU_FWD) ? 2 : 1;
+  const int64_t sms = simt_sms();
+  auto cost = [&](int bm, int bn, double per_output) {
+    const int64_t tiles = (int64_t)((a.M + bm - 1) / bm) * (((int64_t)a.N * half + bn - 1) / bn) *
+                          a.batch * a.splits;
+    return (double)((tiles + sms - 1) / sms) * bm * bn * per_output;
+  };
+  const double c[4] = {cost(128, 128, 1.0), cost(64, 128, 1.06), cost(64, 64, 1.14),
+                       cost(32, 32, 2.2)};
+  int best = 0;
+  for (int i = 1; i < 4; ++i)
+    if (c[i] < c[best]) best = i;
+  switch (best) {
+    case 0: return go<128, 128, 16, 8, 8, 2, A_K, B_K, EPI>(a, st);
+    case 1: return go<64, 128, 16, 8, 8, 4, A_K, B_K, EPI>(a, st);
+    case 2: return go<64, 64, 16, 8, 4, 4, A_K, B_K, EPI>(a, st);
+  }
+  return go<32, 32, 32, 2, 4, 4, A_K, B_K, EPI>(a, st);
+}
+
+bool vec_ok(const void* p, int64_t bs, int64_t ld, int contiguous) {
+  return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && bs % 4 == 0 && ld % 4 == 0 &&
+         contiguous % 4 == 0;
+}
+
+}  // namespace
+
+cudaError_t launch_simt_gemm(SimtGemmArgs a, cudaStream_t st) {
+  if (a.M == 0 || a.N == 0 || a.batch == 0) return cudaSuccess;
+  const bool second_a = a.segs == 2;
+  if (!a.A2) a.A2 = a.A;
+  if (!a.B2) a.B2 = a.B;
+  // split boundaries are multiples of 4, so a chunk of four k never crosses one
+  a.kchunk = a.splits > 1 ? ((a.K + a.splits - 1) / a.splits + 3) / 4 * 4 : a.K;
+  a.vec_a = vec_ok(a.A, a.a_bs, a.a_ld, a.a_kfast ? a.K : a.M) &&
+            (!second_a || vec_ok(a.A2, a.a_bs, a.a_ld, a.a_kfast ? a.K : a.M));
+  a.vec_b = vec_ok(a.B, a.b_bs, a.b_ld, a.b_kfast ? a.K : a.N) &&
+            vec_ok(a.B2, a.b_bs, a.b_ld, a.b_kfast ? a.K : a.N);
+  a.vec_c = vec_ok(a.C, a.c_bs, a.c_ld, a.N) && a.c_split % 4 == 0 &&
+            (!a.C2 || vec_ok(a.C2, a.c_bs, a.c_ld, a.N)) &&
+            (!a.C3 || vec_ok(a.C3, a.c_bs, a.c_ld, a.N));
+  if (a.C3) return pick<true, false, SIMT_SWIGLU_FWD>(a, st);
+  if (a.E1) return pick<true, true, SIMT_SWIGLU_BWD>(a, st);
+  if (a.C2) return pick<false, false, SIMT_DUAL>(a, st);
+  if (a.a_kfast)
+    return a.b_kfast ? pick<true, true, SIMT_PLAIN>(a, st) : pick<true, false, SIMT_PLAIN>(a, st);
+  return pick<false, false, SIMT_PLAIN>(a, st);
+}
+
+// ------------------------------------------------------------------ router
+// Scores of 32 tokens per CTA: logits X.Wr as one FMA chain per (token, expert) in ascending
+// k, kept in shared memory (never written to global), then the row softmax, S, S^T and the
+// slot map's -1.
+namespace {
+constexpr int RBM = 32, RBK = 64;
+
+template <int BN, int TM, int TN>
+__global__ void __launch_bounds__(RBM / TM * (BN / TN))
+router_f32_kernel(const float* __restrict__ X, const float* __restrict__ Wr,
+                  const float* __restrict__ br, float* __restrict__ S, float* __restrict__ ST,
+                  int* __restrict__ slot, int N, int d, int E, bool vx, bool vw) {
+  constexpr int TX = BN / TN, TY = RBM / TM, NT = TX * TY;
+  constexpr int LDA = RBM + 4, LDB = BN + 4;
+  constexpr int NA = RBM * RBK / 4 / NT, NB = BN * RBK / 4 / NT;
+  static_assert(NA * NT * 4 == RBM * RBK && NB * NT * 4 == BN * RBK, "chunks divide evenly");
+  extern __shared__ float4 sh4[];
+  float* As = reinterpret_cast<float*>(sh4);     // [2][RBK][LDA]
+  float* Bs = As + 2 * RBK * LDA;                // [2][RBK][LDB]
+  float* tile = Bs + 2 * RBK * LDB;              // [RBM][E+1] logits, then scores
+  const int tid = threadIdx.x, ty = tid / TX, tx = tid % TX;
+  const int warp = tid >> 5, lane = tid & 31, nw = NT / 32;
+  const int t0 = blockIdx.x * RBM;
+  const int nsl = (d + RBK - 1) / RBK;
+  float ra[NA][4], rb[NB][4];
+  for (int n0 = 0; n0 < E; n0 += BN) {
+    auto fetch = [&](int s) {
+#pragma unroll
+      for (int i = 0; i < NA; ++i) {
+        const int c = tid + i * NT, t = t0 + c / (RBK / 4), k = s * RBK + (c % (RBK / 4)) * 4;
+        load4(ra[i], X + (int64_t)t * d + k, t < N ? k : d, d, vx);
+      }
+#pragma unroll
+      for (int i = 0; i < NB; ++i) {
+        const int c = tid + i * NT, k = s * RBK + c / (BN / 4), n = n0 + (c % (BN / 4)) * 4;
+        load4(rb[i], Wr + (int64_t)k * E + n, k < d ? n : E, E, vw);
+      }
+    };
+    auto put = [&](int buf) {
+#pragma unroll
+      for (int i = 0; i < NA; ++i) {
+        const int c = tid + i * NT;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          As[(buf * RBK + (c % (RBK / 4)) * 4 + j) * LDA + c / (RBK / 4)] = ra[i][j];
+      }
+#pragma unroll
+      for (int i = 0; i < NB; ++i) {
+        const int c = tid + i * NT;
+        *reinterpret_cast<float4*>(Bs + (buf * RBK + c / (BN / 4)) * LDB + (c % (BN / 4)) * 4) =
+            make_float4(rb[i][0], rb[i][1], rb[i][2], rb[i][3]);
+      }
+    };
+    float acc[TM][TN];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+    fetch(0);
+    put(0);
+    __syncthreads();
+    for (int s = 0; s < nsl; ++s) {
+      const int buf = s & 1;
+      if (s + 1 < nsl) fetch(s + 1);
+#pragma unroll 16
+      for (int k = 0; k < RBK; ++k) {
+        float a[TM], w[TN];
+#pragma unroll
+        for (int i = 0; i < TM; ++i) a[i] = As[(buf * RBK + k) * LDA + ty * TM + i];
+#pragma unroll
+        for (int j = 0; j < TN; ++j) w[j] = Bs[(buf * RBK + k) * LDB + tx * TN + j];
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+          for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i], w[j], acc[i][j]);
+      }
+      if (s + 1 < nsl) put(buf ^ 1);
+      __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        const int e = n0 + tx * TN + j;
+        if (e < E) tile[(ty * TM + i) * (E + 1) + e] = acc[i][j];
+      }
+  }
+  __syncthreads();
+  for (int r = warp; r < RBM; r += nw) {
+    const int t = t0 + r;
+    if (t >= N) break;
+    float* row = tile + r * (E + 1);
+    float mx = -INFINITY;
+    for (int e = lane; e < E; e += 32) {
+      const float v = row[e] + (br ? __ldg(br + e) : 0.0f);
+      row[e] = v;
+      mx = fmaxf(mx, v);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    float sum = 0.f;
+    for (int e = lane; e < E; e += 32) {
+      const float q = expf(row[e] - mx);
+      row[e] = q;
+      sum += q;
+    }
+    sum = warp_sum(sum);
+    const float inv = 1.0f / sum;
+    for (int e = lane; e < E; e += 32) {
+      const float q = row[e] * inv;
+      row[e] = q;
+      S[(size_t)t * E + e] = q;
+      slot[(size_t)t * E + e] = -1;
+    }
+  }
+  __syncthreads();
+  for (int e = warp; e < E; e += nw) {
+    const int t = t0 + lane;
+    if (t < N) ST[(size_t)e * N + t] = tile[lane * (E + 1) + e];
+  }
+}
+
+template <int BN, int TM, int TN>
+cudaError_t router_go(const float* X, const float* Wr, const float* br, float* S, float* ST,
+                      int* slot, int N, int d, int E, cudaStream_t st) {
+  auto kern = router_f32_kernel<BN, TM, TN>;
+  const size_t smem =
+      ((size_t)2 * RBK * (RBM + 4 + BN + 4) + (size_t)RBM * (E + 1)) * sizeof(float);
+  if (smem > 48 * 1024) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  kern<<<(N + RBM - 1) / RBM, RBM / TM * (BN / TN), smem, st>>>(
+      X, Wr, br, S, ST, slot, N, d, E, vec_ok(X, 0, d, d), vec_ok(Wr, 0, E, E));
+  return cudaGetLastError();
 }
 }  // namespace
 
-cudaError_t launch_simt_gemm(const SimtGemmArgs& a, EType ta, EType tb, cudaStream_t st) {
-  if (a.M == 0 || a.N == 0 || a.batch == 0) return cudaSuccess;
-  dim3 grid((a.N + BN - 1) / BN, (a.M + BM - 1) / BM, a.batch * a.splits);
-  if (ta == EType::F32 && tb == EType::F32)
-    simt_gemm_kernel<float, float><<<grid, 256, 0, st>>>(a);
-  else if (ta == EType::BF16 && tb == EType::BF16)
-    simt_gemm_kernel<bf16, bf16><<<grid, 256, 0, st>>>(a);
-  else if (ta == EType::F32 && tb == EType::BF16)
-    simt_gemm_kernel<float, bf16><<<grid, 256, 0, st>>>(a);
-  else
-    simt_gemm_kernel<bf16, float><<<grid, 256, 0, st>>>(a);
-  return cudaGetLastError();
+cudaError_t launch_router_f32(const float* X, const float* Wr, const float* br, float* S,
+                              float* ST, int* slot, int N, int d, int E, cudaStream_t st) {
+  if (N == 0) return cudaSuccess;
+  if (E <= 16) return router_go<16, 2, 2>(X, Wr, br, S, ST, slot, N, d, E, st);
+  return router_go<64, 2, 4>(X, Wr, br, S, ST, slot, N, d, E, st);
 }
 
 }  // namespace ecmoe

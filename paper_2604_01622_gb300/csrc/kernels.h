@@ -7,10 +7,10 @@
 namespace ecmoe {
 
 // ---------------------------------------------------------------- router + selection
-// Row softmax of fp32 logits Z [N][E] (+ br) -> S [N][E] and S^T [E][N]; sets the slot map
-// slot [N][E] to -1 (the state launch_topk expects).
-cudaError_t launch_softmax_rows(const float* Z, const float* br, float* S, float* ST, int* slot,
-                                int N, int E, cudaStream_t st);
+// fp32 router: logits X.Wr (+ br) and their row softmax in one kernel, S [N][E] and S^T [E][N];
+// sets the slot map slot [N][E] to -1 (the state launch_topk expects). X [N][d], Wr [d][E].
+cudaError_t launch_router_f32(const float* X, const float* Wr, const float* br, float* S,
+                              float* ST, int* slot, int N, int d, int E, cudaStream_t st);
 // Transpose scores [E][N] -> [N][E] (used when the caller supplies S); sets slot [N][E] to -1.
 cudaError_t launch_transpose_scores(const float* ST, float* S, int* slot, int N, int E,
                                     cudaStream_t st);
@@ -98,30 +98,35 @@ cudaError_t launch_dx_combine(const T* dH, const int* slot, const T* dXr, const 
 cudaError_t launch_colsum(const float* Z, float* out, int N, int E, float* scratch,
                           cudaStream_t st);
 int64_t colsum_scratch_floats(int N, int E);
-template <typename T>
-cudaError_t launch_swiglu_fwd_ew(const float* Ag, const float* Bu, T* A, T* B, T* U, int64_t n,
-                                 cudaStream_t st);
-template <typename T>
-cudaError_t launch_swiglu_bwd_ew(const float* dU, const T* A, const T* B, T* dA, T* dB,
-                                 int64_t n, cudaStream_t st);
-template <typename T>
-cudaError_t launch_convert(const float* in, T* out, int64_t n, cudaStream_t st);
 cudaError_t launch_reduce_splits(const float* part, float* out, int64_t n, int splits,
                                  cudaStream_t st);
 
 // ---------------------------------------------------------------- fp32 SIMT GEMM
-// C[b] (+)= A[b] . B[b] with A logical [M][K], B logical [K][N], C [M][N] fp32 (unit column
-// stride). Element strides per operand; TA/TB are float or bf16.
+// C[b] = A[b].B[b], A logical [M][K], B logical [K][N], C [M][N] (row stride c_ld). Each operand
+// is contiguous along K (kfast: rows of A, columns of B, `ld` apart) or along its other
+// dimension (k rows `ld` apart). With idx, A's rows (kfast) or k rows (else) are gathered:
+// row i is row idx[b*idx_bs + i] of A. Forms, by the pointers given:
+//   segs == 2       C = A.B + A2.B2 (two K loops, each rounded as its own sum)
+//   C2 (no C3, E1)  C = A.B, C2 = A.B2
+//   C3              a = A.B, b = A.B2: C = a, C2 = b, C3 = silu(a) b
+//   E1              dU = A.B with a = E1, b = E2 (layout of C): C = dU b silu'(a), C2 = dU silu(a)
+//   splits > 1      (plain) split s of K writes C + s * c_split
 struct SimtGemmArgs {
-  const void* A; int64_t a_bs, a_ms, a_ks;
-  const void* B; int64_t b_bs, b_ks, b_ns;
-  float* C; int64_t c_bs, c_ms;
-  int M, N, K, batch;
-  int splits;                 // >1: split s writes C + s * c_split (beta ignored)
-  int64_t c_split;
-  float beta;                 // C = A.B + beta*C (splits == 1 only)
+  const float *A = nullptr, *A2 = nullptr;
+  int64_t a_bs = 0, a_ld = 0;
+  const float *B = nullptr, *B2 = nullptr;
+  int64_t b_bs = 0, b_ld = 0;
+  const int* idx = nullptr;
+  int64_t idx_bs = 0;
+  float *C = nullptr, *C2 = nullptr, *C3 = nullptr;
+  const float *E1 = nullptr, *E2 = nullptr;
+  int64_t c_bs = 0, c_ld = 0, c_split = 0;
+  int M = 0, N = 0, K = 0, batch = 1, splits = 1, segs = 1;
+  bool a_kfast = true, b_kfast = false;
+  // set by the launcher
+  int kchunk = 0;
+  bool vec_a = false, vec_b = false, vec_c = false;
 };
-enum class EType { F32, BF16 };
-cudaError_t launch_simt_gemm(const SimtGemmArgs& a, EType ta, EType tb, cudaStream_t st);
+cudaError_t launch_simt_gemm(SimtGemmArgs a, cudaStream_t st);
 
 }  // namespace ecmoe

@@ -677,66 +677,6 @@ cudaError_t launch_colsum(const float* Z, float* out, int N, int E, float* scrat
   return cudaGetLastError();
 }
 
-// ------------------------------------------------------------------ SwiGLU elementwise (SIMT path)
-template <typename T>
-__global__ void swiglu_fwd_ew_kernel(const float* __restrict__ Ag, const float* __restrict__ Bu,
-                                     T* __restrict__ A, T* __restrict__ B, T* __restrict__ U,
-                                     int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const float a = Ag[i], b = Bu[i];
-    A[i] = from_f32<T>(a);
-    B[i] = from_f32<T>(b);
-    U[i] = from_f32<T>(a * sigmoidf_(a) * b);
-  }
-}
-
-template <typename T>
-cudaError_t launch_swiglu_fwd_ew(const float* Ag, const float* Bu, T* A, T* B, T* U, int64_t n,
-                                 cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  const unsigned blocks = grid_for(n, 152 * 64);
-  swiglu_fwd_ew_kernel<T><<<blocks, 256, 0, st>>>(Ag, Bu, A, B, U, n);
-  return cudaGetLastError();
-}
-
-template <typename T>
-__global__ void swiglu_bwd_ew_kernel(const float* __restrict__ dU, const T* __restrict__ A,
-                                     const T* __restrict__ B, T* __restrict__ dA,
-                                     T* __restrict__ dB, int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const float a = to_f32(A[i]), b = to_f32(B[i]), du = dU[i];
-    const float s = sigmoidf_(a);
-    dA[i] = from_f32<T>(du * b * s * (1.0f + a * (1.0f - s)));
-    dB[i] = from_f32<T>(du * a * s);
-  }
-}
-
-template <typename T>
-cudaError_t launch_swiglu_bwd_ew(const float* dU, const T* A, const T* B, T* dA, T* dB,
-                                 int64_t n, cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  const unsigned blocks = grid_for(n, 152 * 64);
-  swiglu_bwd_ew_kernel<T><<<blocks, 256, 0, st>>>(dU, A, B, dA, dB, n);
-  return cudaGetLastError();
-}
-
-template <typename T>
-__global__ void convert_kernel(const float* __restrict__ in, T* __restrict__ out, int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = from_f32<T>(in[i]);
-}
-
-template <typename T>
-cudaError_t launch_convert(const float* in, T* out, int64_t n, cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  const unsigned blocks = grid_for(n, 152 * 64);
-  convert_kernel<T><<<blocks, 256, 0, st>>>(in, out, n);
-  return cudaGetLastError();
-}
-
 __global__ void reduce_splits_kernel(const float* __restrict__ part, float* __restrict__ out,
                                      int64_t n, int splits) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -765,21 +705,20 @@ cudaError_t launch_reduce_splits(const float* part, float* out, int64_t n, int s
 }
 
 #define ECMOE_INST(T)                                                                            \
-  template cudaError_t launch_scatter_rows<T>(const T*, const int*, T*, int, int, int, int,       \
-                                              cudaStream_t);                                      \
-  template cudaError_t launch_zero_pad_rows<T>(const int*, const int*, T*, int, int, cudaStream_t); \
   template cudaError_t launch_combine<T>(const T*, const float*, const int*, const T*, const T*,  \
                                          T*, int, int, int, int, cudaStream_t);                   \
-  template cudaError_t launch_bwd_gather_scale<T>(const T*, const T*, const int*, const float*,   \
-                                                  T*, float*, int64_t, int, cudaStream_t);        \
   template cudaError_t launch_dx_combine<T>(const T*, const int*, const T*, const T*,             \
-                                            const T*, T*, int, int, int, int, cudaStream_t);      \
-  template cudaError_t launch_swiglu_fwd_ew<T>(const float*, const float*, T*, T*, T*, int64_t,   \
-                                               cudaStream_t);                                     \
-  template cudaError_t launch_swiglu_bwd_ew<T>(const float*, const T*, const T*, T*, T*,          \
-                                               int64_t, cudaStream_t);                            \
-  template cudaError_t launch_convert<T>(const float*, T*, int64_t, cudaStream_t);
+                                            const T*, T*, int, int, int, int, cudaStream_t);
 ECMOE_INST(float)
 ECMOE_INST(bf16)
+// the fp32 path gathers rows inside its GEMMs; the bf16 path takes the gate and its gradient
+// into the expert GEMMs' epilogues
+template cudaError_t launch_scatter_rows<bf16>(const bf16*, const int*, bf16*, int, int, int, int,
+                                               cudaStream_t);
+template cudaError_t launch_zero_pad_rows<bf16>(const int*, const int*, bf16*, int, int,
+                                                cudaStream_t);
+template cudaError_t launch_bwd_gather_scale<float>(const float*, const float*, const int*,
+                                                    const float*, float*, float*, int64_t, int,
+                                                    cudaStream_t);
 
 }  // namespace ecmoe

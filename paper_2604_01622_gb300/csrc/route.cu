@@ -1,4 +1,4 @@
-// Router softmax and expert-choice top-k selection (arXiv 2604.01622, Sec. 2.2).
+// Score transpose and expert-choice top-k selection (arXiv 2604.01622, Sec. 2.2).
 //
 // Selection: for every expert e and group g (one sequence, Sec. 5.2) keep the k_g tokens
 // with the largest S[t,e] (Sec. 2.2 TopC; capacity per group, Sec. 4.2). Ties go to the
@@ -10,59 +10,6 @@
 #include "kernels.h"
 
 namespace ecmoe {
-
-// ------------------------------------------------------------------ softmax over experts
-// 32 tokens per CTA; the S^T tile is staged in shared memory so both layouts are written
-// with coalesced stores. The slot map [N][E] (same layout as S) is set to -1 beside S.
-__global__ void softmax_rows_kernel(const float* __restrict__ Z, const float* __restrict__ br,
-                                    float* __restrict__ S, float* __restrict__ ST,
-                                    int* __restrict__ slot, int N, int E) {
-  extern __shared__ float tile[];  // [32][E+1]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const int t0 = blockIdx.x * 32;
-  for (int r = warp; r < 32; r += nw) {
-    const int t = t0 + r;
-    if (t >= N) break;
-    const float* z = Z + (size_t)t * E;
-    float mx = -INFINITY;
-    for (int e = lane; e < E; e += 32) {
-      float v = z[e] + (br ? br[e] : 0.0f);
-      tile[r * (E + 1) + e] = v;
-      mx = fmaxf(mx, v);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    float sum = 0.f;
-    for (int e = lane; e < E; e += 32) {
-      float p = expf(tile[r * (E + 1) + e] - mx);
-      tile[r * (E + 1) + e] = p;
-      sum += p;
-    }
-    sum = warp_sum(sum);
-    const float inv = 1.0f / sum;
-    for (int e = lane; e < E; e += 32) {
-      float p = tile[r * (E + 1) + e] * inv;
-      tile[r * (E + 1) + e] = p;
-      S[(size_t)t * E + e] = p;
-      slot[(size_t)t * E + e] = -1;
-    }
-  }
-  __syncthreads();
-  for (int e = warp; e < E; e += nw) {
-    const int t = t0 + lane;
-    if (t < N) ST[(size_t)e * N + t] = tile[lane * (E + 1) + e];
-  }
-}
-
-cudaError_t launch_softmax_rows(const float* Z, const float* br, float* S, float* ST, int* slot,
-                                int N, int E, cudaStream_t st) {
-  if (N == 0) return cudaSuccess;
-  size_t smem = (size_t)32 * (E + 1) * sizeof(float);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(softmax_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  softmax_rows_kernel<<<(N + 31) / 32, 256, smem, st>>>(Z, br, S, ST, slot, N, E);
-  return cudaGetLastError();
-}
 
 // S = (S^T)^T through a 32 x 32 shared tile; the slot map is set to -1 beside S.
 __global__ void transpose_scores_kernel(const float* __restrict__ ST, float* __restrict__ S,

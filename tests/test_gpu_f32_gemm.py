@@ -1,0 +1,26 @@
+"""The fp32 path's GEMMs at the sizes where a tile shape or a load form changes, against the
+oracle (relative max-norm 1e-4, the fp32 parity bound of the other tests): one shape per tile
+(128 x 128, 64 x 128, 64 x 64, 32 x 32), each with ragged row, column and k edges, an expert
+count that is not a multiple of 4 (scalar loads and stores in the router products), more than 64
+experts (several column tiles of the router kernel) and fewer than 64 tokens (one split of
+X^T dZ)."""
+import pytest
+
+from paper_2604_01622_gb300 import inputs as I
+from tests.test_gpu_parity import _check_layer
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("L,d,E,d_ff,k", [
+    (3000, 260, 24, 132, 700),    # 128 x 128: a 60-row tail, 4 columns past a tile
+    (2000, 260, 16, 132, 260),    # 64 x 128
+    (900, 132, 14, 132, 130),     # 64 x 64, 14 experts
+    (130, 68, 6, 36, 33),         # 32 x 32: one row past a tile
+    (1000, 36, 70, 20, 40),       # 70 experts: two column tiles of the router
+    (40, 516, 5, 4, 7),           # 40 tokens, k loop of 516 = 8 slices and 4; d_ff one chunk
+])
+def test_f32_layer_tile_edges(L, d, E, d_ff, k):
+    w = I.scaled(I.WORKLOADS["tiny_f32"], G=1, L=L, d=d, E=E, d_ff=d_ff, k_base=k, seed=31,
+                 router_bias=True)
+    _check_layer(I.make_inputs(w))
