@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <cstring>
 #include <cstdarg>
+#include <initializer_list>
 #include <type_traits>
 
 #include <nvtx3/nvToolsExt.h>
@@ -22,6 +23,7 @@ using namespace ecmoe;
 struct ec_ctx {
   int N = 0, d = 0, E = 0, F = 0, G = 0, dtype = 0;
   int M_cap = 0, M = 0, max_group = 0;
+  bool goff_aligned = false;   // every group of every score column starts on a 16-byte boundary
   std::vector<int32_t> group_off, k_g, k_off;
   char* ws = nullptr;
   size_t ws_bytes = 0;
@@ -235,6 +237,8 @@ ec_status set_groups(ec_ctx* c, const int32_t* group_off, const int32_t* k_g, bo
     c->group_off.assign(group_off, group_off + G + 1);
     c->M_cap = (int)M;
     c->max_group = maxL;
+    c->goff_aligned = c->N % 4 == 0;
+    for (int g = 0; g < G; ++g) c->goff_aligned = c->goff_aligned && group_off[g] % 4 == 0;
   }
   c->k_g.assign(k_g, k_g + G);
   c->k_off.assign(G + 1, 0);
@@ -278,43 +282,100 @@ const void* router_b(ec_ctx* c) {
 }
 
 // ---------------------------------------------------------------- router + selection
+// Where the selection and the scores of a call go. The kernels write the caller's arrays
+// themselves (`direct`); otherwise they write the workspace and copy_out copies at the end.
+struct RouteOut {
+  int32_t* idx;
+  float* gate;
+  float* S;
+  bool direct;
+};
+
+struct Span {
+  const void* p;
+  size_t n;
+};
+
+// Direct writes happen while the call still reads its inputs (and, in a forward, before Y is
+// written), where copies at the end do not: they need the alignment of the kernels' stores and
+// arrays that overlap neither the inputs and outputs in `others` nor one another.
+bool can_write_direct(const RouteOut& o, size_t P, size_t NE, std::initializer_list<Span> others) {
+  const Span out[3] = {{o.idx, P * 4}, {o.gate, P * 4}, {o.S, NE * 4}};
+  if ((reinterpret_cast<uintptr_t>(o.idx) & 3u) || (reinterpret_cast<uintptr_t>(o.gate) & 3u) ||
+      !aligned16(o.S))
+    return false;
+  auto apart = [](const Span& a, const Span& b) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a.p), y = reinterpret_cast<uintptr_t>(b.p);
+    return !a.p || !b.p || x + a.n <= y || y + b.n <= x;
+  };
+  for (int i = 0; i < 3; ++i) {
+    for (int j = i + 1; j < 3; ++j)
+      if (!apart(out[i], out[j])) return false;
+    for (const Span& s : others)
+      if (!apart(out[i], s)) return false;
+  }
+  return true;
+}
+
+// Scores and selection. `layer`: the call goes on to the experts, which need S token-major, the
+// slot map and the workspace's idx and gate; otherwise (ec_route) only what the caller asked for
+// is written.
 template <typename T>
 ec_status run_route(ec_ctx* c, const void* X, const void* Wr, const float* br, const float* S_in,
-                    cudaStream_t st) {
+                    const RouteOut& out, bool layer, cudaStream_t st) {
   const int N = c->N, E = c->E, d = c->d;
-  float* ST = at<float>(c, c->o_ST);
-  float* S = at<float>(c, c->o_S);
   const int nz = N > 0;
-  // each of the three kernels that write S token-major also sets the slot map to -1, so the
-  // top-k kernel writes only the selected entries
-  int* slot = at<int>(c, c->o_slot);
+  TopkArgs p;
+  p.N = N; p.E = E; p.M = c->M;
+  p.group_off = at<int>(c, c->o_goff); p.k_g = at<int>(c, c->o_kg); p.k_off = at<int>(c, c->o_koff);
+  p.idx = at<int>(c, c->o_idx);
+  p.gate = at<float>(c, c->o_gate);
+  if (layer) {
+    p.slot = at<int>(c, c->o_slot);
+    if (out.direct) { p.idx2 = out.idx; p.gate2 = out.gate; }
+  } else if (out.direct) {
+    p.idx = out.idx;
+    p.gate = out.gate;
+  }
+  float* ST = out.direct && out.S ? out.S : at<float>(c, c->o_ST);
+  float* S = layer ? at<float>(c, c->o_S) : nullptr;
+  // the kernels that write S also set the slot map to -1, so the top-k kernel writes only the
+  // selected entries
   if (S_in) {
-    EC_CUDA(cudaMemcpyAsync(ST, S_in, (size_t)E * N * 4, cudaMemcpyDeviceToDevice, st), "copy S_in");
-    EC_KERNEL("transpose_scores", nz, launch_transpose_scores(ST, S, slot, N, E, st));
-  } else if (use_tc(c)) {
-    EC_KERNEL("router_gemm_softmax", (router_needs_pad(E) ? 2 : 1) * nz,
-              tc_router_softmax(X, Wr, at<void>(c, c->o_wrpad), br, S, ST, slot, N, d, E,
-                                at<int>(c, c->o_status), st));
+    if (out.direct) {
+      p.ST = S_in;
+      p.S_copy = out.S;
+    } else {
+      EC_CUDA(cudaMemcpyAsync(ST, S_in, (size_t)E * N * 4, cudaMemcpyDeviceToDevice, st),
+              "copy S_in");
+      p.ST = ST;
+    }
   } else {
-    EC_KERNEL("router_gemm_softmax", nz,
-              launch_router_f32(f32p(X), f32p(Wr), br, S, ST, slot, N, d, E, st));
+    p.ST = ST;
+    if constexpr (std::is_same<T, bf16>::value)
+      EC_KERNEL("router_gemm_softmax", (router_needs_pad(E) ? 2 : 1) * nz,
+                tc_router_softmax(X, Wr, at<void>(c, c->o_wrpad), br, S, ST, p.slot, N, d, E,
+                                  at<int>(c, c->o_status), st));
+    else
+      EC_KERNEL("router_gemm_softmax", nz,
+                launch_router_f32(f32p(X), f32p(Wr), br, S, ST, p.slot, N, d, E, st));
   }
   EC_KERNEL("topk", 1,
-            launch_topk(ST, N, E, c->G, at<int>(c, c->o_goff), at<int>(c, c->o_kg),
-                        at<int>(c, c->o_koff), c->M, c->max_group, at<int>(c, c->o_idx),
-                        at<float>(c, c->o_gate), slot, st));
+            launch_topk(p, c->G, c->max_group, c->goff_aligned && aligned16(p.ST), st));
   return EC_OK;
 }
 
-ec_status copy_out(ec_ctx* c, int32_t* idx, float* gate, float* S_out, cudaStream_t st) {
+ec_status copy_out(ec_ctx* c, const RouteOut& o, cudaStream_t st) {
+  if (o.direct) return EC_OK;
   const size_t P = (size_t)c->E * c->M;
-  if (idx && P)
-    EC_CUDA(cudaMemcpyAsync(idx, at<int>(c, c->o_idx), P * 4, cudaMemcpyDeviceToDevice, st), "idx out");
-  if (gate && P)
-    EC_CUDA(cudaMemcpyAsync(gate, at<float>(c, c->o_gate), P * 4, cudaMemcpyDeviceToDevice, st),
+  if (o.idx && P)
+    EC_CUDA(cudaMemcpyAsync(o.idx, at<int>(c, c->o_idx), P * 4, cudaMemcpyDeviceToDevice, st),
+            "idx out");
+  if (o.gate && P)
+    EC_CUDA(cudaMemcpyAsync(o.gate, at<float>(c, c->o_gate), P * 4, cudaMemcpyDeviceToDevice, st),
             "gate out");
-  if (S_out)
-    EC_CUDA(cudaMemcpyAsync(S_out, at<float>(c, c->o_ST), (size_t)c->E * c->N * 4,
+  if (o.S)
+    EC_CUDA(cudaMemcpyAsync(o.S, at<float>(c, c->o_ST), (size_t)c->E * c->N * 4,
                             cudaMemcpyDeviceToDevice, st), "S out");
   return EC_OK;
 }
@@ -778,11 +839,17 @@ ec_status ec_route(ec_ctx* c, const void* X, const void* Wr, const float* br, co
     return fail(c, EC_ERR_INVALID_ARG, "inputs must be 16-byte aligned");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   c->have_fwd = false;
-  s = c->dtype == EC_BF16 ? run_route<bf16>(c, X, Wr, br, S_in, st)
-                          : run_route<float>(c, X, Wr, br, S_in, st);
+  const size_t P = (size_t)c->E * c->M, NE = (size_t)c->N * c->E, es = esize(c);
+  RouteOut out{idx, gate, S_out == S_in ? nullptr : S_out, false};
+  out.direct = S_in ? can_write_direct(out, P, NE, {{S_in, NE * 4}})
+                    : can_write_direct(out, P, NE,
+                                       {{X, (size_t)c->N * c->d * es}, {Wr, (size_t)c->d * c->E * es},
+                                        {br, (size_t)c->E * 4}});
+  s = c->dtype == EC_BF16 ? run_route<bf16>(c, X, Wr, br, S_in, out, false, st)
+                          : run_route<float>(c, X, Wr, br, S_in, out, false, st);
   if (s != EC_OK) return s;
   mark(c, "end", st);
-  return copy_out(c, idx, gate, S_out, st);
+  return copy_out(c, out, st);
 }
 
 static ec_status forward_impl(ec_ctx* c, const void* X, const void* Wr, const float* br,
@@ -801,14 +868,21 @@ static ec_status forward_impl(ec_ctx* c, const void* X, const void* Wr, const fl
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   c->have_fwd = false;
   c->Wgs = Wgs; c->Wus = Wus; c->Wds = Wds;
-  s = c->dtype == EC_BF16 ? run_route<bf16>(c, X, Wr, br, nullptr, st)
-                          : run_route<float>(c, X, Wr, br, nullptr, st);
+  const size_t es = esize(c), x = (size_t)c->N * c->d * es, w = (size_t)c->E * c->d * c->F * es,
+               ws = (size_t)c->d * c->Fs * es;
+  RouteOut out{idx, gate, S_out, false};
+  out.direct = can_write_direct(out, (size_t)c->E * c->M, (size_t)c->N * c->E,
+                                {{X, x}, {Wr, (size_t)c->d * c->E * es}, {br, (size_t)c->E * 4},
+                                 {Wg, w}, {Wu, w}, {Wd, w}, {Wgs, ws}, {Wus, ws}, {Wds, ws},
+                                 {Y, x}});
+  s = c->dtype == EC_BF16 ? run_route<bf16>(c, X, Wr, br, nullptr, out, true, st)
+                          : run_route<float>(c, X, Wr, br, nullptr, out, true, st);
   if (s != EC_OK) return s;
   s = c->dtype == EC_BF16 ? run_forward<bf16>(c, X, Wg, Wu, Wd, Wgs, Wus, Wds, Y, st)
                           : run_forward<float>(c, X, Wg, Wu, Wd, Wgs, Wus, Wds, Y, st);
   if (s != EC_OK) return s;
   mark(c, "end", st);
-  s = copy_out(c, idx, gate, S_out, st);
+  s = copy_out(c, out, st);
   if (s != EC_OK) return s;
   c->X = X; c->Wr = Wr; c->br = br; c->Wg = Wg; c->Wu = Wu; c->Wd = Wd;
   c->have_fwd = true;

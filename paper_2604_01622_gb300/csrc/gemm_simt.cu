@@ -501,8 +501,8 @@ router_f32_kernel(const float* __restrict__ X, const float* __restrict__ Wr,
     for (int e = lane; e < E; e += 32) {
       const float q = row[e] * inv;
       row[e] = q;
-      S[(size_t)t * E + e] = q;
-      slot[(size_t)t * E + e] = -1;
+      if (S) S[(size_t)t * E + e] = q;
+      if (slot) slot[(size_t)t * E + e] = -1;
     }
   }
   __syncthreads();

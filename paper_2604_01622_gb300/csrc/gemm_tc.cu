@@ -1163,15 +1163,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
 #pragma unroll
               for (int i = 0; i < 32; ++i) ev[c][i] *= inv;
               if (cg * 32 >= E || !st_any) continue;
-              if (lane == 0) bulk_wait_read<0>();   // the buffer's last store has read it
-              __syncwarp();
-              stage_f32(bS, lane, ev[c]);
-              fence_async_smem();
-              __syncwarp();
-              if (lane == 0) {
-                tma_store_3d(&mO0, smem_u32(bS), cg * 32, srow, 0);
-                bulk_wait_read<0>();
+              if (p.out0) {
+                if (lane == 0) bulk_wait_read<0>();   // the buffer's last store has read it
+                __syncwarp();
+                stage_f32(bS, lane, ev[c]);
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0) tma_store_3d(&mO0, smem_u32(bS), cg * 32, srow, 0);
               }
+              if (lane == 0) bulk_wait_read<0>();
               __syncwarp();
 #pragma unroll
               for (int i = 0; i < 32; ++i)
@@ -1191,12 +1191,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
 #pragma unroll
             for (int i = 0; i < 32; ++i) ev[c][i] *= inv;
             if (row_ok) {
-              float* srow = S + (int64_t)gm * E + c * 32;
+              float* srow = S ? S + (int64_t)gm * E + c * 32 : nullptr;
               int* lrow = slot ? slot + (int64_t)gm * E + c * 32 : nullptr;
               if (vec && c * 32 + 32 <= E) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
-                  reinterpret_cast<float4*>(srow)[j] =
+                  if (srow) reinterpret_cast<float4*>(srow)[j] =
                       make_float4(ev[c][4 * j], ev[c][4 * j + 1], ev[c][4 * j + 2], ev[c][4 * j + 3]);
                 if (lrow)
 #pragma unroll
@@ -1206,7 +1206,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
 #pragma unroll
                 for (int i = 0; i < 32; ++i)
                   if (c * 32 + i < E) {
-                    srow[i] = ev[c][i];
+                    if (srow) srow[i] = ev[c][i];
                     if (lrow) lrow[i] = -1;
                   }
               }
@@ -1253,7 +1253,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
               const int e = c * 32 + i;
               if (e < E && row_ok) {
                 const float pr = __expf(f32(v[i]) + (p.bias ? p.bias[e] : 0.f) - mx) * inv;
-                S[(int64_t)gm * E + e] = pr;
+                if (S) S[(int64_t)gm * E + e] = pr;
                 ST[(int64_t)e * p.M + gm] = pr;
                 if (slot) slot[(int64_t)gm * E + e] = -1;
               }
@@ -1475,8 +1475,9 @@ cudaError_t tc_router_softmax(const void* X, const void* Wr, void* Wr_pad, const
   if (Ep <= 128 && E % 4 == 0 && N % 4 == 0) {
     // S [N][E] and S^T [E][N] leave through TMA stores (row strides of 16-byte multiples)
     CUtensorMap mo0, mo1;
-    TC_TRY(make_out_map(&mo0, S, true, E, N, 1));
     TC_TRY(make_out_map(&mo1, ST, true, N, E, 1));
+    if (S) TC_TRY(make_out_map(&mo0, S, true, E, N, 1));
+    else mo0 = mo1;   // not stored through
     // rows split evenly over the SMs; a 192 KB ring (the main loop streams X at the rate its
     // bytes in flight allow); 8 epilogue warps, two per TMEM lane quarter, each taking half of
     // a row's experts (the epilogue of a CTA's last tile is not hidden behind a main loop)

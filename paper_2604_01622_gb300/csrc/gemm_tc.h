@@ -26,8 +26,8 @@ struct VarRows {
 // policy 2 (and never with variable rows): its epilogue reads A and B per row and cannot
 // drain an accumulator half within the MMAs that cover it.
 
-// Router: Z = X.Wr (+br), S = row softmax over the E experts, written as S [N][E] and
-// S^T [E][N]. X [N][d] bf16, Wr [d][E] bf16. Wr_pad: device scratch of d*round_up(E,64)
+// Router: Z = X.Wr (+br), S = row softmax over the E experts, written as S [N][E] (NULL: not
+// written) and S^T [E][N]. X [N][d] bf16, Wr [d][E] bf16. Wr_pad: device scratch of d*round_up(E,64)
 // bf16 (zero-padded copy of Wr made on the stream when E is not a multiple of 64,
 // router_needs_pad; otherwise Wr itself is read and Wr_pad is untouched). slot_init
 // (nullable): an int [N][E] map set to -1 beside S (the expert-choice slot map before

@@ -7,19 +7,25 @@
 namespace ecmoe {
 
 // ---------------------------------------------------------------- router + selection
-// fp32 router: logits X.Wr (+ br) and their row softmax in one kernel, S [N][E] and S^T [E][N];
-// sets the slot map slot [N][E] to -1 (the state launch_topk expects). X [N][d], Wr [d][E].
+// fp32 router: logits X.Wr (+ br) and their row softmax in one kernel, S [N][E] (NULL: not
+// written) and S^T [E][N]; sets the slot map slot [N][E] (if given) to -1, the state launch_topk
+// expects. X [N][d], Wr [d][E].
 cudaError_t launch_router_f32(const float* X, const float* Wr, const float* br, float* S,
                               float* ST, int* slot, int N, int d, int E, cudaStream_t st);
-// Transpose scores [E][N] -> [N][E] (used when the caller supplies S); sets slot [N][E] to -1.
-cudaError_t launch_transpose_scores(const float* ST, float* S, int* slot, int N, int E,
-                                    cudaStream_t st);
-// Expert-choice top-k per (expert, group) over S^T [E][N]; writes idx/gate [E][M] and, for
-// the selected pairs only, the token->slot map slot [N][E] (= m). The other entries of slot
-// must already hold -1.
-cudaError_t launch_topk(const float* ST, int N, int E, int G, const int* group_off, const int* k_g,
-                        const int* k_off, int M, int max_group, int* idx, float* gate, int* slot,
-                        cudaStream_t st);
+// Expert-choice top-k per (expert, group) over the scores ST [E][N]: idx/gate [E][M], and where
+// given a second copy of both (idx2, gate2), a copy of the scores (S_copy [E][N]) and, for the
+// selected pairs only, the token->slot map slot [N][E] (= m), whose other entries must already
+// hold -1. group_off/k_g/k_off: device tables of the G groups, the longest of max_group tokens;
+// aligned: every column starts on a 16-byte boundary of ST. No output overlaps ST.
+struct TopkArgs {
+  const float* ST = nullptr;
+  int N = 0, E = 0, M = 0;
+  const int *group_off = nullptr, *k_g = nullptr, *k_off = nullptr;
+  int *idx = nullptr, *idx2 = nullptr;
+  float *gate = nullptr, *gate2 = nullptr, *S_copy = nullptr;
+  int* slot = nullptr;
+};
+cudaError_t launch_topk(const TopkArgs& p, int G, int max_group, bool aligned, cudaStream_t st);
 
 // Capacity update from device memory (one CTA): if 0 <= k_new[g] <= L_g for every group and
 // sum k_new == M, writes k_g [G] and its prefix sums k_off [G+1]; otherwise leaves both and

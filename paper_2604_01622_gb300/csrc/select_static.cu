@@ -115,6 +115,7 @@ extern "C" ec_status ec_select_static(const float* S, int32_t N, int32_t E, int3
   int32_t* t_koff = tbl + (2 * G + 1);
   t_koff[0] = 0;
   int max_group = 0;
+  bool aligned = (reinterpret_cast<uintptr_t>(S) & 15u) == 0 && N % 4 == 0;
   for (int g = 0; g < G; ++g) {
     const int L = group_off[g + 1] - group_off[g];
     if (L < 0 || k_g[g] < 0 || k_g[g] > L) return EC_ERR_SHAPE;
@@ -123,6 +124,7 @@ extern "C" ec_status ec_select_static(const float* S, int32_t N, int32_t E, int3
     t_kg[g] = k_g[g];
     t_koff[g + 1] = t_koff[g] + k_g[g];
     if (L > max_group) max_group = L;
+    aligned = aligned && group_off[g] % 4 == 0;
   }
   t_goff[G] = group_off[G];
   const int M = t_koff[G];
@@ -148,8 +150,11 @@ extern "C" ec_status ec_select_static(const float* S, int32_t N, int32_t E, int3
   if (cudaMemcpyAsync(base, tbl, (size_t)(3 * G + 2) * sizeof(int32_t), cudaMemcpyHostToDevice,
                       st) != cudaSuccess)
     return EC_ERR_CUDA;
-  if (ecmoe::launch_topk(S, N, E, G, d_goff, d_kg, d_koff, M, max_group, idx, gate, d_slot, st) !=
-      cudaSuccess)
-    return EC_ERR_CUDA;
+  ecmoe::TopkArgs p;
+  p.ST = S;
+  p.N = N; p.E = E; p.M = M;
+  p.group_off = d_goff; p.k_g = d_kg; p.k_off = d_koff;
+  p.idx = idx; p.gate = gate; p.slot = d_slot;
+  if (ecmoe::launch_topk(p, G, max_group, aligned, st) != cudaSuccess) return EC_ERR_CUDA;
   return EC_OK;
 }
