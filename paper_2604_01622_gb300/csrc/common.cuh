@@ -4,6 +4,10 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <utility>
+
+#include "launch.h"
+
 namespace ecmoe {
 
 // Device status word codes (first word of the workspace).
@@ -54,6 +58,52 @@ __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+// ------------------------------------------------------------------ overlapped launches
+// Small calls launch every kernel with programmatic stream serialisation (LaunchStream::overlap):
+// its CTAs may start while the kernel before it still runs, and each waits in pdl_begin for that
+// kernel's end (and its memory) before it touches global memory. Only what comes before
+// pdl_begin overlaps: the launch itself, barrier and TMEM set-up, tensor-map fetches. The next
+// kernel is let in after the wait, so when a kernel starts, everything before its predecessor has
+// completed. Launched without it, both instructions do nothing.
+// The pointers named in pdl_begin come out of an opaque step behind the wait, so no load through
+// them, read-only loads included, can be moved above it.
+template <typename P>
+__device__ __forceinline__ P* after_wait(P* p) {
+  asm volatile("" : "+l"(p)::"memory");
+  return p;
+}
+template <typename... P>
+__device__ __forceinline__ void pdl_begin(P&... ptrs) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  (([&] { asm volatile("" : "+l"(ptrs)::"memory"); }()), ...);
+}
+
+template <typename... K, typename... A>
+cudaError_t launch_kernel(void (*kern)(K...), dim3 grid, dim3 block, size_t smem, LaunchStream st,
+                          int cluster, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  unsigned n = 0;
+  if (st.overlap) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = (unsigned)cluster;
+    at[n].val.clusterDim.y = 1;
+    at[n++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
 }
 
 // silu(a) = a * sigmoid(a); sigmoid evaluated with the CUDA math library's expf.

@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(BM / TM * (BN / TN), MINB) simt_gemm_kernel(co
   const float* A1 = p.A2 + (int64_t)b * p.a_bs;
   const float* B0 = p.B + (int64_t)b * p.b_bs;
   const float* B1 = p.B2 + (int64_t)b * p.b_bs;
+  pdl_begin(idx, A0, A1, B0, B1);
   const bool va = p.vec_a, vb = p.vec_b;
 
   // Chunk c of an operand contiguous along k: a warp takes 16 rows x 2 chunks, so its loads use
@@ -291,8 +292,8 @@ __global__ void __launch_bounds__(BM / TM * (BN / TN), MINB) simt_gemm_kernel(co
         }
       }
     } else {
-      const float* E1 = p.E1 + (int64_t)b * p.c_bs + ro;
-      const float* E2 = p.E2 + (int64_t)b * p.c_bs + ro;
+      const float* E1 = after_wait(p.E1) + (int64_t)b * p.c_bs + ro;
+      const float* E2 = after_wait(p.E2) + (int64_t)b * p.c_bs + ro;
 #pragma unroll
       for (int h = 0; h < CG; ++h) {
         const int n = col_of(h);
@@ -324,13 +325,12 @@ int simt_sms() {
 }
 
 template <int BM, int BN, int BK, int TM, int TN, int MINB, bool A_K, bool B_K, int EPI>
-cudaError_t go(const SimtGemmArgs& a, cudaStream_t st) {
+cudaError_t go(const SimtGemmArgs& a, LaunchStream st) {
   constexpr bool DUAL = EPI == SIMT_DUAL || EPI == SIMT_SWIGLU_FWD;
   constexpr int cols = DUAL ? BN / 2 : BN;
   const dim3 grid((a.N + cols - 1) / cols, (a.M + BM - 1) / BM, a.batch * a.splits);
-  simt_gemm_kernel<BM, BN, BK, TM, TN, MINB, A_K, B_K, EPI>
-      <<<grid, BM / TM * (BN / TN), 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(simt_gemm_kernel<BM, BN, BK, TM, TN, MINB, A_K, B_K, EPI>, grid,
+                       BM / TM * (BN / TN), 0, st, 1, a);
 }
 
 // Tile shape: the one whose busiest SM has the least work, tiles per SM (rounded up) times the
@@ -340,7 +340,7 @@ cudaError_t go(const SimtGemmArgs& a, cudaStream_t st) {
 // where 128 x 128 leaves a nearly empty last wave (1000 x 500 x 364: 129 against 141 us) and
 // the small tiles for a few rows per expert (96 x 500 x 364: 27 against 43 us).
 template <bool A_K, bool B_K, int EPI>
-cudaError_t pick(const SimtGemmArgs& a, cudaStream_t st) {
+cudaError_t pick(const SimtGemmArgs& a, LaunchStream st) {
   constexpr int half = (EPI == SIMT_DUAL || EPI == SIMT_SWIGLU_FWD) ? 2 : 1;
   const int64_t sms = simt_sms();
   auto cost = [&](int bm, int bn, double per_output) {
@@ -368,7 +368,7 @@ bool vec_ok(const void* p, int64_t bs, int64_t ld, int contiguous) {
 
 }  // namespace
 
-cudaError_t launch_simt_gemm(SimtGemmArgs a, cudaStream_t st) {
+cudaError_t launch_simt_gemm(SimtGemmArgs a, LaunchStream st) {
   if (a.M == 0 || a.N == 0 || a.batch == 0) return cudaSuccess;
   const bool second_a = a.segs == 2;
   if (!a.A2) a.A2 = a.A;
@@ -406,6 +406,7 @@ router_f32_kernel(const float* __restrict__ X, const float* __restrict__ Wr,
   constexpr int LDA = RBM + 4, LDB = BN + 4;
   constexpr int NA = RBM * RBK / 4 / NT, NB = BN * RBK / 4 / NT;
   static_assert(NA * NT * 4 == RBM * RBK && NB * NT * 4 == BN * RBK, "chunks divide evenly");
+  pdl_begin(X, Wr, br);
   extern __shared__ float4 sh4[];
   float* As = reinterpret_cast<float*>(sh4);     // [2][RBK][LDA]
   float* Bs = As + 2 * RBK * LDA;                // [2][RBK][LDB]
@@ -514,7 +515,7 @@ router_f32_kernel(const float* __restrict__ X, const float* __restrict__ Wr,
 
 template <int BN, int TM, int TN>
 cudaError_t router_go(const float* X, const float* Wr, const float* br, float* S, float* ST,
-                      int* slot, int N, int d, int E, cudaStream_t st) {
+                      int* slot, int N, int d, int E, LaunchStream st) {
   auto kern = router_f32_kernel<BN, TM, TN>;
   const size_t smem =
       ((size_t)2 * RBK * (RBM + 4 + BN + 4) + (size_t)RBM * (E + 1)) * sizeof(float);
@@ -523,14 +524,13 @@ cudaError_t router_go(const float* X, const float* Wr, const float* br, float* S
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  kern<<<(N + RBM - 1) / RBM, RBM / TM * (BN / TN), smem, st>>>(
-      X, Wr, br, S, ST, slot, N, d, E, vec_ok(X, 0, d, d), vec_ok(Wr, 0, E, E));
-  return cudaGetLastError();
+  return launch_kernel(kern, (N + RBM - 1) / RBM, RBM / TM * (BN / TN), smem, st, 1, X, Wr, br, S,
+                       ST, slot, N, d, E, vec_ok(X, 0, d, d), vec_ok(Wr, 0, E, E));
 }
 }  // namespace
 
 cudaError_t launch_router_f32(const float* X, const float* Wr, const float* br, float* S,
-                              float* ST, int* slot, int N, int d, int E, cudaStream_t st) {
+                              float* ST, int* slot, int N, int d, int E, LaunchStream st) {
   if (N == 0) return cudaSuccess;
   if (E <= 16) return router_go<16, 2, 2>(X, Wr, br, S, ST, slot, N, d, E, st);
   return router_go<64, 2, 4>(X, Wr, br, S, ST, slot, N, d, E, st);

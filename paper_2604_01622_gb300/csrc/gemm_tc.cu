@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
                const __grid_constant__ CUtensorMap mB0, const __grid_constant__ CUtensorMap mB1,
                const __grid_constant__ CUtensorMap mO0, const __grid_constant__ CUtensorMap mO1,
-               const __grid_constant__ CUtensorMap mO2, const Args p) {
+               const __grid_constant__ CUtensorMap mO2, Args p) {
   constexpr bool WIDE = BN == 512;            // single accumulator handed over in two halves
   constexpr int NH = WIDE ? 2 : 1;            // accumulator segments per tile
   constexpr int SEGW = BN / NH;               // columns per segment = N of one MMA
@@ -544,6 +544,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
   if constexpr (PAIR) cluster_sync();   // the peer's barriers are initialised before use
   tc_fence_after();
   const uint32_t tmem_base = *tmem_holder;
+  pdl_begin(p.in0, p.in1, p.bias, p.vm_tiles, p.vm_count, p.gate);
 
   const int tiles_per_b = p.m_tiles * p.n_tiles;
   const int total = VARM == 1 ? __ldg(p.vm_tiles + p.vm_E) * p.n_tiles : p.batch * tiles_per_b;
@@ -1345,31 +1346,28 @@ template <int BN, bool A_MN, bool B_MN, bool B_SPLIT, bool K_SPLIT, int EPI, int
           int EPW = 8, bool PAIR = false, int VARM = 0>
 cudaError_t launch(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0,
                    const CUtensorMap& b1, const CUtensorMap& o0, const CUtensorMap& o1,
-                   const CUtensorMap& o2, Args p, cudaStream_t st) {
+                   const CUtensorMap& o2, Args p, LaunchStream st) {
   auto kern = tc_gemm_kernel<BN, A_MN, B_MN, B_SPLIT, K_SPLIT, EPI, STAGES, EPW, PAIR, VARM>;
   constexpr uint32_t smem = smem_bytes<BN, STAGES, PAIR, EPW, EPI>();
   static_assert(smem <= 232448, "dynamic shared memory above the 227 KB per-block limit");
   constexpr int threads = 64 + 32 * EPW;
   static bool attr = false;
   static int max_clusters = 0;
-  cudaLaunchAttribute cl[1];
-  cl[0].id = cudaLaunchAttributeClusterDimension;
-  cl[0].val.clusterDim.x = 2;
-  cl[0].val.clusterDim.y = 1;
-  cl[0].val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  if (PAIR) {
-    cfg.attrs = cl;
-    cfg.numAttrs = 1;
-  }
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     if (PAIR) {
+      cudaLaunchAttribute cl[1];
+      cl[0].id = cudaLaunchAttributeClusterDimension;
+      cl[0].val.clusterDim.x = 2;
+      cl[0].val.clusterDim.y = 1;
+      cl[0].val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(2 * sm_count());
+      cfg.blockDim = dim3(threads);
+      cfg.dynamicSmemBytes = smem;
+      cfg.attrs = cl;
+      cfg.numAttrs = 1;
       e = cudaOccupancyMaxActiveClusters(&max_clusters, kern, &cfg);
       if (e != cudaSuccess) return e;
       if (max_clusters <= 0) return cudaErrorNotSupported;
@@ -1388,19 +1386,13 @@ cudaError_t launch(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorM
     p.batch = 1;
     p.n_tiles = 1;
     p.m_tiles = g * (int)((max_rows + BM - 1) / BM);
-    kern<<<g, threads, smem, st>>>(a0, a1, b0, b1, o0, o1, o2, p);
-    return cudaGetLastError();
+    return launch_kernel(kern, g, threads, smem, st, 1, a0, a1, b0, b1, o0, o1, o2, p);
   }
   const int total = p.batch * p.m_tiles * p.n_tiles;
   if (total == 0 || (VARM != 2 && p.k_blocks == 0)) return cudaSuccess;
-  if (PAIR) {
-    const int clusters = total < max_clusters ? total : max_clusters;
-    cfg.gridDim = dim3(2 * clusters);
-    return cudaLaunchKernelEx(&cfg, kern, a0, a1, b0, b1, o0, o1, o2, p);
-  }
-  const int grid = total < sm_count() ? total : sm_count();
-  kern<<<grid, threads, smem, st>>>(a0, a1, b0, b1, o0, o1, o2, p);
-  return cudaGetLastError();
+  const int walkers = PAIR ? max_clusters : sm_count();
+  const int grid = (PAIR ? 2 : 1) * (total < walkers ? total : walkers);
+  return launch_kernel(kern, grid, threads, smem, st, PAIR ? 2 : 1, a0, a1, b0, b1, o0, o1, o2, p);
 }
 
 Args base_args(int batch, int M, int N, int K, int BN_tile, int* status) {
@@ -1419,6 +1411,7 @@ Args base_args(int batch, int M, int N, int K, int BN_tile, int* status) {
 
 __global__ void pad_router_weights(const bf16* __restrict__ Wr, bf16* __restrict__ Wp, int d,
                                    int E, int Ep) {
+  pdl_begin(Wr);
   const int64_t n = (int64_t)d * Ep;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -1452,15 +1445,14 @@ bool router_needs_pad(int E) { return E % 64 != 0; }
 
 cudaError_t tc_router_softmax(const void* X, const void* Wr, void* Wr_pad, const float* br,
                               float* S, float* ST, int* slot_init, int N, int d, int E,
-                              int* status, cudaStream_t st) {
+                              int* status, LaunchStream st) {
   if (N == 0) return cudaSuccess;
   const int Ep = (E + 63) / 64 * 64;
   // Wr [d][E] already has the padded layout when E is a multiple of 64
   const void* Wb = Wr;
   if (router_needs_pad(E)) {
-    pad_router_weights<<<256, 256, 0, st>>>(static_cast<const bf16*>(Wr),
-                                            static_cast<bf16*>(Wr_pad), d, E, Ep);
-    TC_TRY(cudaGetLastError());
+    TC_TRY(launch_kernel(pad_router_weights, 256, 256, 0, st, 1, static_cast<const bf16*>(Wr),
+                         static_cast<bf16*>(Wr_pad), d, E, Ep));
     Wb = Wr_pad;
   }
   CUtensorMap ma, mb;
@@ -1542,7 +1534,7 @@ template <int BN, bool A_MN, bool B_MN, bool B_SPLIT, bool K_SPLIT, int EPI>
 static cudaError_t launch_rows(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0,
                                const CUtensorMap& b1, const CUtensorMap& o0, const CUtensorMap& o1,
                                const CUtensorMap& o2, const Args& p, const VarRows* vr,
-                               cudaStream_t st) {
+                               LaunchStream st) {
   // the dU GEMM's epilogue reads A and B through L1: a 5-deep ring leaves it 32 KB more;
   // wide tiles take 48 KB per k-slice
   constexpr int ST = BN == 512 ? kWideStages : EPI == EPI_SWIGLU_BWD ? kDuStages : 6;
@@ -1554,7 +1546,7 @@ static cudaError_t launch_rows(const CUtensorMap& a0, const CUtensorMap& a1, con
 }
 
 cudaError_t tc_expert_up(const void* H, const void* Wg, const void* Wu, void* A, void* B, void* U,
-                         int E, int M, int d, int F, int* status, cudaStream_t st,
+                         int E, int M, int d, int F, int* status, LaunchStream st,
                          const VarRows* vr, const float* gate, int tiles) {
   CUtensorMap ma, mg, mu, oa, ob, ou;
   TC_TRY(act_map(&ma, H, d, E, M, vr, BM));
@@ -1579,7 +1571,7 @@ cudaError_t tc_expert_up(const void* H, const void* Wg, const void* Wu, void* A,
 }
 
 cudaError_t tc_expert_down(const void* U, const void* Wd, void* O, int E, int M, int d, int F,
-                           int* status, cudaStream_t st, const VarRows* vr, int tiles) {
+                           int* status, LaunchStream st, const VarRows* vr, int tiles) {
   CUtensorMap ma, mb, mo;
   TC_TRY(act_map(&ma, U, F, E, M, vr, BM));
   TC_TRY(make_map(&mb, Wd, d, F, E, 64));
@@ -1598,7 +1590,7 @@ cudaError_t tc_expert_down(const void* U, const void* Wd, void* O, int E, int M,
 
 cudaError_t tc_expert_dgrad_up(const void* dO, const void* Wd, const void* A, const void* B,
                                void* dA, void* dB, int E, int M, int d, int F, int* status,
-                               cudaStream_t st, const VarRows* vr, const float* gate,
+                               LaunchStream st, const VarRows* vr, const float* gate,
                                float* dgate_part, int64_t dgate_stride, int tiles) {
   CUtensorMap ma, mb, oa, ob;
   TC_TRY(act_map(&ma, dO, d, E, M, vr, BM));
@@ -1629,7 +1621,7 @@ cudaError_t tc_expert_dgrad_up(const void* dO, const void* Wd, const void* A, co
 }
 
 cudaError_t tc_expert_dgrad_h(const void* dA, const void* dB, const void* Wg, const void* Wu,
-                              void* dH, int E, int M, int d, int F, int* status, cudaStream_t st,
+                              void* dH, int E, int M, int d, int F, int* status, LaunchStream st,
                               const VarRows* vr, int tiles) {
   CUtensorMap ma0, ma1, mb0, mb1;
   TC_TRY(act_map(&ma0, dA, F, E, M, vr, BM));
@@ -1653,7 +1645,7 @@ cudaError_t tc_expert_dgrad_h(const void* dA, const void* dB, const void* Wg, co
 
 cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const void* dA,
                             const void* dB, float* dWg, float* dWu, float* dWd, int E, int M,
-                            int d, int F, int* status, cudaStream_t st, const VarRows* vr,
+                            int d, int F, int* status, LaunchStream st, const VarRows* vr,
                             int tiles) {
   // Variable rows: the K loop of expert e runs over its own padded region (count rows,
   // rounded up to the 64-row k-step, the rest of which is zero in both operands).
@@ -1725,7 +1717,7 @@ cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const 
 }
 
 cudaError_t tc_router_dgrad(const void* dZb, const void* Wr_pad, void* dXr, int N, int d, int Ep,
-                            int* status, cudaStream_t st) {
+                            int* status, LaunchStream st) {
   if (N == 0) return cudaSuccess;
   // dXr [N][d] = (dZ_hi + dZ_lo) [N][Ep] . Wr^T as one K loop over both planes;
   // B[n=i][k=e] = Wr_pad[i][e] is K-major
@@ -1746,7 +1738,7 @@ cudaError_t tc_router_dgrad(const void* dZb, const void* Wr_pad, void* dXr, int 
 }
 
 cudaError_t tc_router_wgrad(const void* X, const void* dZb, float* part, int N, int d, int Ep,
-                            int splits, int* status, cudaStream_t st) {
+                            int splits, int* status, LaunchStream st) {
   if (N == 0) return cudaSuccess;
   // part[h][s] [d][Ep] = X_s^T . dZ_h,s over the s-th block of N/splits tokens (split K as the
   // batch), h = hi / lo plane of dZ (the two column halves of each tile)
@@ -1772,7 +1764,7 @@ cudaError_t tc_router_wgrad(const void* X, const void* dZb, float* part, int N, 
                                                                       p, st);
 }
 
-cudaError_t tc_wait_probe(int* status, unsigned long long limit_ns, cudaStream_t st) {
+cudaError_t tc_wait_probe(int* status, unsigned long long limit_ns, LaunchStream st) {
   wait_probe_kernel<<<1, 32, 0, st>>>(status, limit_ns);
   return cudaGetLastError();
 }

@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "launch.h"
+
 namespace ecmoe {
 
 // Variable rows per expert (token-choice routing): expert e owns the padded rows
@@ -35,18 +37,18 @@ struct VarRows {
 bool router_needs_pad(int E);
 cudaError_t tc_router_softmax(const void* X, const void* Wr, void* Wr_pad, const float* br,
                               float* S, float* ST, int* slot_init, int N, int d, int E,
-                              int* status, cudaStream_t st);
+                              int* status, LaunchStream st);
 
 // [A | B] = H.[Wg | Wu] per expert; U = g * silu(A) * B with g the row's gate (gate [E*M]
 // or, with vr, [P]; NULL: g = 1). H [E][M][d]; Wg, Wu [E][d][F]; A, B, U [E][M][F] bf16.
 cudaError_t tc_expert_up(const void* H, const void* Wg, const void* Wu, void* A, void* B, void* U,
-                         int E, int M, int d, int F, int* status, cudaStream_t st,
+                         int E, int M, int d, int F, int* status, LaunchStream st,
                          const VarRows* vr = nullptr, const float* gate = nullptr,
                          int tiles = 0);
 
 // O = U.Wd per expert. U [E][M][F]; Wd [E][F][d]; O [E][M][d] bf16.
 cudaError_t tc_expert_down(const void* U, const void* Wd, void* O, int E, int M, int d, int F,
-                           int* status, cudaStream_t st, const VarRows* vr = nullptr,
+                           int* status, LaunchStream st, const VarRows* vr = nullptr,
                            int tiles = 0);
 
 // dU' = dO.Wd^T per expert, dU = g dU' (g the row's gate as in tc_expert_up, NULL: 1), then
@@ -55,13 +57,13 @@ cudaError_t tc_expert_down(const void* U, const void* Wd, void* O, int E, int M,
 // [256 j, 256 j + 256)), partial j of row r at dgate_part[j * dgate_stride + r].
 cudaError_t tc_expert_dgrad_up(const void* dO, const void* Wd, const void* A, const void* B,
                                void* dA, void* dB, int E, int M, int d, int F, int* status,
-                               cudaStream_t st, const VarRows* vr = nullptr,
+                               LaunchStream st, const VarRows* vr = nullptr,
                                const float* gate = nullptr, float* dgate_part = nullptr,
                                int64_t dgate_stride = 0, int tiles = 0);
 
 // dH = dA.Wg^T + dB.Wu^T per expert (one K loop over both halves). dH [E][M][d] bf16.
 cudaError_t tc_expert_dgrad_h(const void* dA, const void* dB, const void* Wg, const void* Wu,
-                              void* dH, int E, int M, int d, int F, int* status, cudaStream_t st,
+                              void* dH, int E, int M, int d, int F, int* status, LaunchStream st,
                               const VarRows* vr = nullptr, int tiles = 0);
 
 // Weight gradients per expert, fp32: dWd = U^T.dO, dWg = H^T.dA, dWu = H^T.dB (dWd NULL:
@@ -69,21 +71,21 @@ cudaError_t tc_expert_dgrad_h(const void* dA, const void* dB, const void* Wg, co
 // expert with none gets zeros).
 cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const void* dA,
                             const void* dB, float* dWg, float* dWu, float* dWd, int E, int M,
-                            int d, int F, int* status, cudaStream_t st,
+                            int d, int F, int* status, LaunchStream st,
                             const VarRows* vr = nullptr, int tiles = 0);
 
 // Router backward on the tensor cores. dZb [2][N][Ep] bf16: hi and lo planes of the
 // zero-padded softmax gradient (dZ ~ hi + lo); Wr_pad [d][Ep] bf16 (the padded router
 // weights of the forward pass). dXr [N][d] bf16 = dZ . Wr^T (summed in fp32, rounded once).
 cudaError_t tc_router_dgrad(const void* dZb, const void* Wr_pad, void* dXr, int N, int d, int Ep,
-                            int* status, cudaStream_t st);
+                            int* status, LaunchStream st);
 // part [2][splits][d][Ep] fp32: X^T . dZ_plane over `splits` equal blocks of tokens
 // (N % splits == 0); dWr is the sum of all 2*splits partials.
 cudaError_t tc_router_wgrad(const void* X, const void* dZb, float* part, int N, int d, int Ep,
-                            int splits, int* status, cudaStream_t st);
+                            int splits, int* status, LaunchStream st);
 
 // Launch a kernel that waits, with the given limit, on an mbarrier nothing completes, so
 // the bounded-wait path (status word, early return) can be exercised without a hang.
-cudaError_t tc_wait_probe(int* status, unsigned long long limit_ns, cudaStream_t st);
+cudaError_t tc_wait_probe(int* status, unsigned long long limit_ns, LaunchStream st);
 
 }  // namespace ecmoe

@@ -4,6 +4,8 @@
 #include <stdint.h>
 #include <cuda_bf16.h>
 
+#include "launch.h"
+
 namespace ecmoe {
 
 // ---------------------------------------------------------------- router + selection
@@ -11,7 +13,7 @@ namespace ecmoe {
 // written) and S^T [E][N]; sets the slot map slot [N][E] (if given) to -1, the state launch_topk
 // expects. X [N][d], Wr [d][E].
 cudaError_t launch_router_f32(const float* X, const float* Wr, const float* br, float* S,
-                              float* ST, int* slot, int N, int d, int E, cudaStream_t st);
+                              float* ST, int* slot, int N, int d, int E, LaunchStream st);
 // Expert-choice top-k per (expert, group) over the scores ST [E][N]: idx/gate [E][M], and where
 // given a second copy of both (idx2, gate2), a copy of the scores (S_copy [E][N]) and, for the
 // selected pairs only, the token->slot map slot [N][E] (= m), whose other entries must already
@@ -25,13 +27,13 @@ struct TopkArgs {
   float *gate = nullptr, *gate2 = nullptr, *S_copy = nullptr;
   int* slot = nullptr;
 };
-cudaError_t launch_topk(const TopkArgs& p, int G, int max_group, bool aligned, cudaStream_t st);
+cudaError_t launch_topk(const TopkArgs& p, int G, int max_group, bool aligned, LaunchStream st);
 
 // Capacity update from device memory (one CTA): if 0 <= k_new[g] <= L_g for every group and
 // sum k_new == M, writes k_g [G] and its prefix sums k_off [G+1]; otherwise leaves both and
 // records DEV_BAD_CAPACITY in the status word.
 cudaError_t launch_set_capacity(const int* k_new, const int* group_off, int G, int M, int* k_g,
-                                int* k_off, int* status, cudaStream_t st);
+                                int* k_off, int* status, LaunchStream st);
 
 // ---------------------------------------------------------------- token-choice routing
 // Row top-k of S [N][E] (k <= 32, E <= 512), per-expert counts capped at cap (cap < 0:
@@ -46,41 +48,41 @@ cudaError_t launch_set_capacity(const int* k_new, const int* group_off, int G, i
 cudaError_t launch_tc_route(const float* S, int N, int E, int k, int cap, int* choice,
                             float* tgate, float* Z, int* count, int* tiles, int* row_token,
                             float* row_gate, int* slot, int* kept, int* scratch,
-                            cudaStream_t st);
+                            LaunchStream st);
 int64_t tc_route_scratch_ints(int N, int E);
 // Router gradient of token choice: dZ [N][E] (and optionally the bf16 hi/lo planes
 // dZb [2][N][Ep]) from the per-row gate gradients row_dgate [P].
 cudaError_t launch_tc_softmax_bwd(const float* S, const int* choice, const float* tgate,
                                   const float* Z, const int* slot, const float* row_dgate,
                                   float* dZ, __nv_bfloat16* dZb, int N, int E, int Ep, int k,
-                                  cudaStream_t st);
+                                  LaunchStream st);
 
 // ---------------------------------------------------------------- data movement
 // Token-major form of the gather: for each token t, X row t is copied to row e*M + slot[t][e]
 // of H for every expert e with slot[t][e] >= 0 (M = 0: slot holds absolute rows).
 template <typename T>
 cudaError_t launch_scatter_rows(const T* X, const int* slot, T* H, int N, int E, int M, int d,
-                                cudaStream_t st);
+                                LaunchStream st);
 // Zeros the unused (padding) rows of variable-row expert regions (count [E], tiles [E+1] in
 // 256-row blocks, device arrays).
 template <typename T>
 cudaError_t launch_zero_pad_rows(const int* count, const int* tiles, T* H, int E, int d,
-                                 cudaStream_t st);
+                                 LaunchStream st);
 // Y_t = R_t + R2_t (each if given) + sum over the experts that chose t of gate * O row
 // (gate NULL: 1, for O rows already scaled by their gates).
 template <typename T>
 cudaError_t launch_combine(const T* O, const float* gate, const int* slot, const T* R, const T* R2,
-                           T* Y, int N, int E, int M, int d, cudaStream_t st);
+                           T* Y, int N, int E, int M, int d, LaunchStream st);
 // dO row r = gate[r] dY row idx[r], dgate[r] = <dY row idx[r], O row r> (zero rows where
 // idx[r] < 0), for the P rows (fp32 path).
 template <typename T>
 cudaError_t launch_bwd_gather_scale(const T* dY, const T* O, const int* idx, const float* gate,
-                                    T* dO, float* dgate, int64_t P, int d, cudaStream_t st);
+                                    T* dO, float* dgate, int64_t P, int d, LaunchStream st);
 // Router softmax Jacobian: dS[t][e] = dgate of the pair (t chosen by e) else 0,
 // dZ = S (dS - <dS, S>_row). dgate [E*M] summed beforehand; writes dZ [N][E] and, with dZb,
 // the bf16 hi/lo planes [2][N][Ep] (any E <= 512).
 cudaError_t launch_softmax_bwd(const float* S, const int* slot, const float* dgate, float* dZ,
-                               __nv_bfloat16* dZb, int N, int E, int Ep, int M, cudaStream_t st);
+                               __nv_bfloat16* dZb, int N, int E, int Ep, int M, LaunchStream st);
 // The same, fused with the sum of the gate-gradient partials dg_part [parts][E*M] (in part
 // order) and, with dbr, with the router bias gradient dbr[e] = sum_t dZ[t][e] (per-CTA
 // column sums in scratch, then summed in a fixed order: deterministic). dZ and dZb are each
@@ -91,21 +93,21 @@ int64_t router_bwd_scratch_floats(int N, int E);
 cudaError_t launch_router_softmax_bwd(const float* S, const int* slot, const float* dg_part,
                                       int parts, float* dZ, __nv_bfloat16* dZb, float* dbr,
                                       float* scratch, int N, int E, int Ep, int M,
-                                      cudaStream_t st);
+                                      LaunchStream st);
 cudaError_t launch_reduce_partials(const float* part, float* out, int rows, int cols, int ld,
-                                   int splits, cudaStream_t st);
+                                   int splits, LaunchStream st);
 // dX_t = dXr_t + R_t + R2_t (each if given) + sum of the token's dH rows, summed in fp32;
 // dXr (the router's part of the input gradient) is in the layer's dtype.
 template <typename T>
 cudaError_t launch_dx_combine(const T* dH, const int* slot, const T* dXr, const T* R,
-                              const T* R2, T* dX, int N, int E, int M, int d, cudaStream_t st);
+                              const T* R2, T* dX, int N, int E, int M, int d, LaunchStream st);
 // out[e] = sum over the N rows of Z [N][E]; scratch: colsum_scratch_floats(N, E) floats.
 // Two kernels.
 cudaError_t launch_colsum(const float* Z, float* out, int N, int E, float* scratch,
-                          cudaStream_t st);
+                          LaunchStream st);
 int64_t colsum_scratch_floats(int N, int E);
 cudaError_t launch_reduce_splits(const float* part, float* out, int64_t n, int splits,
-                                 cudaStream_t st);
+                                 LaunchStream st);
 
 // ---------------------------------------------------------------- fp32 SIMT GEMM
 // C[b] = A[b].B[b], A logical [M][K], B logical [K][N], C [M][N] (row stride c_ld). Each operand
@@ -133,6 +135,6 @@ struct SimtGemmArgs {
   int kchunk = 0;
   bool vec_a = false, vec_b = false, vec_c = false;
 };
-cudaError_t launch_simt_gemm(SimtGemmArgs a, cudaStream_t st);
+cudaError_t launch_simt_gemm(SimtGemmArgs a, LaunchStream st);
 
 }  // namespace ecmoe

@@ -51,6 +51,7 @@ __global__ void combine_kernel(const T* __restrict__ O, const float* __restrict_
                                const int* __restrict__ slot, const T* __restrict__ R,
                                const T* __restrict__ R2, T* __restrict__ Y, int N, int E, int M,
                                int d) {
+  pdl_begin(O, gate, slot, R, R2);
   extern __shared__ int sh[];
   int* s_e = sh;
   int* s_m = sh + E;
@@ -119,14 +120,14 @@ __global__ void combine_kernel(const T* __restrict__ O, const float* __restrict_
 
 template <typename T>
 cudaError_t launch_combine(const T* O, const float* gate, const int* slot, const T* R, const T* R2,
-                           T* Y, int N, int E, int M, int d, cudaStream_t st) {
+                           T* Y, int N, int E, int M, int d, LaunchStream st) {
   if (N == 0) return cudaSuccess;
   const size_t smem = (size_t)3 * E * sizeof(int);
   // two 16-byte column groups per thread: half a row's groups per CTA, 32 to 128 threads
   const int nv = d * (int)sizeof(T) / 16;
   const int threads = std::min(128, std::max(32, (nv / 2 + 31) / 32 * 32));
-  combine_kernel<T><<<N, threads, smem, st>>>(O, gate, slot, R, R2, Y, N, E, M, d);
-  return cudaGetLastError();
+  return launch_kernel(combine_kernel<T>, N, threads, smem, st, 1, O, gate, slot, R, R2, Y, N, E, M,
+                       d);
 }
 
 // ------------------------------------------------------------------ token-major scatter
@@ -136,6 +137,7 @@ cudaError_t launch_combine(const T* O, const float* gate, const int* slot, const
 template <typename T>
 __global__ void scatter_rows_kernel(const T* __restrict__ X, const int* __restrict__ slot,
                                     T* __restrict__ H, int N, int E, int M, int d) {
+  pdl_begin(X, slot);
   extern __shared__ int sh[];
   int* s_e = sh;
   int* s_m = sh + E;
@@ -154,11 +156,10 @@ __global__ void scatter_rows_kernel(const T* __restrict__ X, const int* __restri
 
 template <typename T>
 cudaError_t launch_scatter_rows(const T* X, const int* slot, T* H, int N, int E, int M, int d,
-                                cudaStream_t st) {
+                                LaunchStream st) {
   if (N == 0) return cudaSuccess;
   const size_t smem = (size_t)2 * E * sizeof(int);
-  scatter_rows_kernel<T><<<N, 128, smem, st>>>(X, slot, H, N, E, M, d);
-  return cudaGetLastError();
+  return launch_kernel(scatter_rows_kernel<T>, N, 128, smem, st, 1, X, slot, H, N, E, M, d);
 }
 
 // Zero the padding rows of variable-row expert regions: rows count[e] .. 256*(tiles[e+1] -
@@ -166,6 +167,7 @@ cudaError_t launch_scatter_rows(const T* X, const int* slot, T* H, int N, int E,
 template <typename T>
 __global__ void zero_pad_rows_kernel(const int* __restrict__ count, const int* __restrict__ tiles,
                                      T* __restrict__ H, int E, int d) {
+  pdl_begin(count, tiles);
   const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   const int e = (int)(w / 256);
@@ -179,10 +181,10 @@ __global__ void zero_pad_rows_kernel(const int* __restrict__ count, const int* _
 
 template <typename T>
 cudaError_t launch_zero_pad_rows(const int* count, const int* tiles, T* H, int E, int d,
-                                 cudaStream_t st) {
+                                 LaunchStream st) {
   const int64_t warps = (int64_t)E * 256;
-  zero_pad_rows_kernel<T><<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(count, tiles, H, E, d);
-  return cudaGetLastError();
+  return launch_kernel(zero_pad_rows_kernel<T>, (unsigned)((warps + 7) / 8), 256, 0, st, 1, count,
+                       tiles, H, E, d);
 }
 
 // ------------------------------------------------------------------ backward: dO = g dY_t, dgate = <dY_t, O>
@@ -191,6 +193,7 @@ __global__ void bwd_gather_scale_kernel(const T* __restrict__ dY, const T* __res
                                         const int* __restrict__ idx, const float* __restrict__ gate,
                                         T* __restrict__ dO, float* __restrict__ dgate, int64_t P,
                                         int d) {
+  pdl_begin(dY, O, idx, gate);
   const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= P) return;
@@ -225,12 +228,11 @@ __global__ void bwd_gather_scale_kernel(const T* __restrict__ dY, const T* __res
 
 template <typename T>
 cudaError_t launch_bwd_gather_scale(const T* dY, const T* O, const int* idx, const float* gate,
-                                    T* dO, float* dgate, int64_t P, int d, cudaStream_t st) {
+                                    T* dO, float* dgate, int64_t P, int d, LaunchStream st) {
   if (P == 0) return cudaSuccess;
   const int warps = 8;
-  bwd_gather_scale_kernel<T><<<(unsigned)((P + warps - 1) / warps), warps * 32, 0, st>>>(
-      dY, O, idx, gate, dO, dgate, P, d);
-  return cudaGetLastError();
+  return launch_kernel(bwd_gather_scale_kernel<T>, (unsigned)((P + warps - 1) / warps), warps * 32, 0,
+                       st, 1, dY, O, idx, gate, dO, dgate, P, d);
 }
 
 // ------------------------------------------------------------------ softmax Jacobian
@@ -243,6 +245,7 @@ cudaError_t launch_bwd_gather_scale(const T* dY, const T* O, const int* idx, con
 __global__ void softmax_bwd_kernel(const float* __restrict__ S, const int* __restrict__ slot,
                                    const float* __restrict__ dgate, float* __restrict__ dZ,
                                    bf16* __restrict__ dZb, int N, int E, int Ep, int M) {
+  pdl_begin(S, slot, dgate);
   constexpr int MAXC = 16;
   const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -283,11 +286,11 @@ __global__ void softmax_bwd_kernel(const float* __restrict__ S, const int* __res
 }
 
 cudaError_t launch_softmax_bwd(const float* S, const int* slot, const float* dgate, float* dZ,
-                               bf16* dZb, int N, int E, int Ep, int M, cudaStream_t st) {
+                               bf16* dZb, int N, int E, int Ep, int M, LaunchStream st) {
   if (N == 0) return cudaSuccess;
   if (E > 512) return cudaErrorInvalidValue;
-  softmax_bwd_kernel<<<(N + 7) / 8, 256, 0, st>>>(S, slot, dgate, dZ, dZb, N, E, Ep, M);
-  return cudaGetLastError();
+  return launch_kernel(softmax_bwd_kernel, (N + 7) / 8, 256, 0, st, 1, S, slot, dgate, dZ, dZb, N, E,
+                       Ep, M);
 }
 
 // Fused form. A group of LPT lanes owns a token (LPT = 16 up to 64 experts, 32 up to 128),
@@ -305,6 +308,7 @@ router_softmax_bwd_kernel(const float* __restrict__ S, const int* __restrict__ s
                           const float* __restrict__ dg_part, int parts, int64_t P,
                           float* __restrict__ dZ, bf16* __restrict__ dZb,
                           float* __restrict__ bpart, int N, int E, int Ep, int M) {
+  pdl_begin(S, slot, dg_part);
   constexpr int TPW = 32 / LPT;                   // tokens per warp per step
   constexpr int TPB = kRbWarps * TPW * kRbIter;   // tokens per CTA
   constexpr int NC = kRbIter * 4;                 // (token, expert) candidates per lane
@@ -431,6 +435,7 @@ router_softmax_bwd_kernel(const float* __restrict__ S, const int* __restrict__ s
 // over strided partials, then a fixed butterfly.
 __global__ void colsum_rows_kernel(const float* __restrict__ part, int nblk, int E,
                                    float* __restrict__ out) {
+  pdl_begin(part);
   const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (c >= E) return;
   float s = 0.f;
@@ -450,40 +455,42 @@ int64_t router_bwd_scratch_floats(int N, int E) {
 }
 
 template <int LPT, bool WDZ, bool BIAS>
-static void router_bwd_go(int nblk, const float* S, const int* slot, const float* dg_part,
+static cudaError_t router_bwd_go(int nblk, const float* S, const int* slot, const float* dg_part,
                           int parts, int64_t P, float* dZ, bf16* dZb, float* bpart, int N, int E,
-                          int Ep, int M, cudaStream_t st) {
-  router_softmax_bwd_kernel<LPT, WDZ, BIAS><<<nblk, kRbWarps * 32, 0, st>>>(
-      S, slot, dg_part, parts, P, dZ, dZb, bpart, N, E, Ep, M);
+                          int Ep, int M, LaunchStream st) {
+  return launch_kernel(router_softmax_bwd_kernel<LPT, WDZ, BIAS>, nblk, kRbWarps * 32, 0, st, 1, S,
+                       slot, dg_part, parts, P, dZ, dZb, bpart, N, E, Ep, M);
 }
 
 template <int LPT>
-static void router_bwd_pick(int nblk, const float* S, const int* slot, const float* dg_part,
+static cudaError_t router_bwd_pick(int nblk, const float* S, const int* slot, const float* dg_part,
                             int parts, int64_t P, float* dZ, bf16* dZb, float* bpart, int N,
-                            int E, int Ep, int M, cudaStream_t st) {
+                            int E, int Ep, int M, LaunchStream st) {
   if (dZ) {
-    if (bpart) router_bwd_go<LPT, true, true>(nblk, S, slot, dg_part, parts, P, dZ, dZb, bpart, N, E, Ep, M, st);
-    else router_bwd_go<LPT, true, false>(nblk, S, slot, dg_part, parts, P, dZ, dZb, bpart, N, E, Ep, M, st);
-  } else {
-    if (bpart) router_bwd_go<LPT, false, true>(nblk, S, slot, dg_part, parts, P, dZ, dZb, bpart, N, E, Ep, M, st);
-    else router_bwd_go<LPT, false, false>(nblk, S, slot, dg_part, parts, P, dZ, dZb, bpart, N, E, Ep, M, st);
+    if (bpart)
+      return router_bwd_go<LPT, true, true>(nblk, S, slot, dg_part, parts, P, dZ, dZb, bpart, N, E, Ep, M, st);
+    return router_bwd_go<LPT, true, false>(nblk, S, slot, dg_part, parts, P, dZ, dZb, bpart, N, E, Ep, M, st);
   }
+    if (bpart)
+      return router_bwd_go<LPT, false, true>(nblk, S, slot, dg_part, parts, P, dZ, dZb, bpart, N, E, Ep, M, st);
+    return router_bwd_go<LPT, false, false>(nblk, S, slot, dg_part, parts, P, dZ, dZb, bpart, N, E, Ep, M, st);
 }
 
 cudaError_t launch_router_softmax_bwd(const float* S, const int* slot, const float* dg_part,
                                       int parts, float* dZ, bf16* dZb, float* dbr,
                                       float* scratch, int N, int E, int Ep, int M,
-                                      cudaStream_t st) {
+                                      LaunchStream st) {
   const int64_t P = (int64_t)E * M;
   if (!router_bwd_fused(E, P) || parts < 1 || (dZb && (Ep < E || Ep % 4)))
     return cudaErrorInvalidValue;
   if (N == 0) return dbr ? cudaMemsetAsync(dbr, 0, (size_t)E * sizeof(float), st) : cudaSuccess;
   const int nblk = (N + router_bwd_tpb(E) - 1) / router_bwd_tpb(E);
   float* bpart = dbr ? scratch : nullptr;
-  if (E <= 64) router_bwd_pick<16>(nblk, S, slot, dg_part, parts, P, dZ, dZb, bpart, N, E, Ep, M, st);
-  else router_bwd_pick<32>(nblk, S, slot, dg_part, parts, P, dZ, dZb, bpart, N, E, Ep, M, st);
-  if (dbr) colsum_rows_kernel<<<(E + 7) / 8, 256, 0, st>>>(bpart, nblk, E, dbr);
-  return cudaGetLastError();
+  const cudaError_t e =
+      E <= 64 ? router_bwd_pick<16>(nblk, S, slot, dg_part, parts, P, dZ, dZb, bpart, N, E, Ep, M, st)
+              : router_bwd_pick<32>(nblk, S, slot, dg_part, parts, P, dZ, dZb, bpart, N, E, Ep, M, st);
+  if (e != cudaSuccess || !dbr) return e;
+  return launch_kernel(colsum_rows_kernel, (E + 7) / 8, 256, 0, st, 1, bpart, nblk, E, dbr);
 }
 
 // out[i][e] = sum_s part[s][i][e] for the first `cols` of `ld` columns.
@@ -494,6 +501,7 @@ cudaError_t launch_router_softmax_bwd(const float* S, const int* slot, const flo
 template <int V>
 __global__ void reduce_partials_kernel(const float* __restrict__ part, float* __restrict__ out,
                                        int rows, int cols, int ld, int splits) {
+  pdl_begin(part);
   typedef typename std::conditional<V == 4, float4, float>::type vec;
   const int cv = cols / V;
   const int64_t n = (int64_t)rows * cv;
@@ -530,19 +538,14 @@ __global__ void reduce_partials_kernel(const float* __restrict__ part, float* __
 }
 
 cudaError_t launch_reduce_partials(const float* part, float* out, int rows, int cols, int ld,
-                                   int splits, cudaStream_t st) {
+                                   int splits, LaunchStream st) {
   if (rows == 0 || cols == 0) return cudaSuccess;
   const bool v4 = cols % 4 == 0 && ld % 4 == 0 &&
                   (reinterpret_cast<uintptr_t>(part) & 15u) == 0 &&
                   (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
   const int64_t n = (int64_t)rows * cols / (v4 ? 4 : 1);
-  if (v4)
-    reduce_partials_kernel<4><<<grid_for(n, 152 * 16), 256, 0, st>>>(part, out, rows, cols, ld,
-                                                                       splits);
-  else
-    reduce_partials_kernel<1><<<grid_for(n, 152 * 16), 256, 0, st>>>(part, out, rows, cols, ld,
-                                                                       splits);
-  return cudaGetLastError();
+  return launch_kernel(v4 ? reduce_partials_kernel<4> : reduce_partials_kernel<1>,
+                       grid_for(n, 152 * 16), 256, 0, st, 1, part, out, rows, cols, ld, splits);
 }
 
 // ------------------------------------------------------------------ dX_t = dXr_t + sum dH rows
@@ -551,6 +554,7 @@ __global__ void dx_combine_kernel(const T* __restrict__ dH, const int* __restric
                                   const T* __restrict__ dXr, const T* __restrict__ R,
                                   const T* __restrict__ R2, T* __restrict__ dX, int N, int E,
                                   int M, int d) {
+  pdl_begin(dH, slot, dXr, R, R2);
   extern __shared__ int sh[];
   int* s_e = sh;
   int* s_m = sh + E;
@@ -620,13 +624,13 @@ __global__ void dx_combine_kernel(const T* __restrict__ dH, const int* __restric
 
 template <typename T>
 cudaError_t launch_dx_combine(const T* dH, const int* slot, const T* dXr, const T* R,
-                              const T* R2, T* dX, int N, int E, int M, int d, cudaStream_t st) {
+                              const T* R2, T* dX, int N, int E, int M, int d, LaunchStream st) {
   if (N == 0) return cudaSuccess;
   const size_t smem = (size_t)2 * E * sizeof(int);
   const int nv = d * (int)sizeof(T) / 16;
   const int threads = std::min(128, std::max(32, (nv / 2 + 31) / 32 * 32));
-  dx_combine_kernel<T><<<N, threads, smem, st>>>(dH, slot, dXr, R, R2, dX, N, E, M, d);
-  return cudaGetLastError();
+  return launch_kernel(dx_combine_kernel<T>, N, threads, smem, st, 1, dH, slot, dXr, R, R2, dX, N, E,
+                       M, d);
 }
 
 // ------------------------------------------------------------------ column sums of Z [N][E]
@@ -636,6 +640,7 @@ constexpr int kColRows = 512;
 
 __global__ void colsum_part_kernel(const float* __restrict__ Z, float* __restrict__ part, int N,
                                    int E) {
+  pdl_begin(Z);
   __shared__ float sh[8][33];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int e = blockIdx.x * 32 + lane;
@@ -657,6 +662,7 @@ __global__ void colsum_part_kernel(const float* __restrict__ Z, float* __restric
 
 __global__ void colsum_final_kernel(const float* __restrict__ part, int nrb, int E,
                                     float* __restrict__ out) {
+  pdl_begin(part);
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= E) return;
   float s = 0.f;
@@ -669,16 +675,18 @@ int64_t colsum_scratch_floats(int N, int E) {
 }
 
 cudaError_t launch_colsum(const float* Z, float* out, int N, int E, float* scratch,
-                          cudaStream_t st) {
+                          LaunchStream st) {
   const int nrb = (N + kColRows - 1) / kColRows;
   if (nrb == 0) return cudaMemsetAsync(out, 0, (size_t)E * sizeof(float), st);
-  colsum_part_kernel<<<dim3((E + 31) / 32, nrb), 256, 0, st>>>(Z, scratch, N, E);
-  colsum_final_kernel<<<(E + 127) / 128, 128, 0, st>>>(scratch, nrb, E, out);
-  return cudaGetLastError();
+  const cudaError_t e = launch_kernel(colsum_part_kernel, dim3((E + 31) / 32, nrb), 256, 0, st, 1, Z,
+                                      scratch, N, E);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(colsum_final_kernel, (E + 127) / 128, 128, 0, st, 1, scratch, nrb, E, out);
 }
 
 __global__ void reduce_splits_kernel(const float* __restrict__ part, float* __restrict__ out,
                                      int64_t n, int splits) {
+  pdl_begin(part);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     // split order, eight loads in flight before they are added
@@ -697,28 +705,27 @@ __global__ void reduce_splits_kernel(const float* __restrict__ part, float* __re
 }
 
 cudaError_t launch_reduce_splits(const float* part, float* out, int64_t n, int splits,
-                                 cudaStream_t st) {
+                                 LaunchStream st) {
   if (n == 0) return cudaSuccess;
   const unsigned blocks = grid_for(n, 152 * 16);
-  reduce_splits_kernel<<<blocks, 256, 0, st>>>(part, out, n, splits);
-  return cudaGetLastError();
+  return launch_kernel(reduce_splits_kernel, blocks, 256, 0, st, 1, part, out, n, splits);
 }
 
 #define ECMOE_INST(T)                                                                            \
   template cudaError_t launch_combine<T>(const T*, const float*, const int*, const T*, const T*,  \
-                                         T*, int, int, int, int, cudaStream_t);                   \
+                                         T*, int, int, int, int, LaunchStream);                   \
   template cudaError_t launch_dx_combine<T>(const T*, const int*, const T*, const T*,             \
-                                            const T*, T*, int, int, int, int, cudaStream_t);
+                                            const T*, T*, int, int, int, int, LaunchStream);
 ECMOE_INST(float)
 ECMOE_INST(bf16)
 // the fp32 path gathers rows inside its GEMMs; the bf16 path takes the gate and its gradient
 // into the expert GEMMs' epilogues
 template cudaError_t launch_scatter_rows<bf16>(const bf16*, const int*, bf16*, int, int, int, int,
-                                               cudaStream_t);
+                                               LaunchStream);
 template cudaError_t launch_zero_pad_rows<bf16>(const int*, const int*, bf16*, int, int,
-                                                cudaStream_t);
+                                                LaunchStream);
 template cudaError_t launch_bwd_gather_scale<float>(const float*, const float*, const int*,
                                                     const float*, float*, float*, int64_t, int,
-                                                    cudaStream_t);
+                                                    LaunchStream);
 
 }  // namespace ecmoe

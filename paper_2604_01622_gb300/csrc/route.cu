@@ -99,7 +99,7 @@ __device__ __forceinline__ void rank_candidates(const uint32_t* cand, int n, int
 constexpr uint32_t kNoKey = 0xFFFFFFFFu;   // offset of a register that holds no score
 
 template <int KPT, int NT, int MINB>
-__global__ void __launch_bounds__(NT, MINB) topk_reg_kernel(const TopkArgs p) {
+__global__ void __launch_bounds__(NT, MINB) topk_reg_kernel(TopkArgs p) {
   constexpr int nw = NT / 32;
   __shared__ __align__(16) int hist[2][256];
   __shared__ uint32_t s_mn[nw], s_mx[nw], s_cnt[nw], s_cand[kCand];
@@ -108,6 +108,7 @@ __global__ void __launch_bounds__(NT, MINB) topk_reg_kernel(const TopkArgs p) {
   __shared__ uint32_t s_T;
   const int e = blockIdx.x, g = blockIdx.y;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_begin(p.ST, p.group_off, p.k_g, p.k_off);
   const int lo = p.group_off[g];
   const int L = p.group_off[g + 1] - lo;
   const int k = p.k_g[g];
@@ -313,7 +314,7 @@ constexpr int kStep = 512;   // keys a warp handles at a time
 constexpr int kList = 512;
 
 template <int CL>
-__global__ void __launch_bounds__(256, 4) topk_cluster_kernel(const TopkArgs p, int chunk) {
+__global__ void __launch_bounds__(256, 4) topk_cluster_kernel(TopkArgs p, int chunk) {
   constexpr int nw = 8, TW = nw * CL;
   extern __shared__ uint4 skeys4[];
   uint32_t* skeys = reinterpret_cast<uint32_t*>(skeys4);
@@ -323,6 +324,7 @@ __global__ void __launch_bounds__(256, 4) topk_cluster_kernel(const TopkArgs p, 
   const int rank = (int)cluster_rank();
   const int e = blockIdx.x / CL, g = blockIdx.y;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_begin(p.ST, p.group_off, p.k_g, p.k_off);
   const int lo = p.group_off[g];
   const int L = p.group_off[g + 1] - lo;
   const int k = p.k_g[g];
@@ -587,13 +589,14 @@ __device__ __forceinline__ unsigned long long block_excl_scan2(unsigned long lon
 
 // Columns too long for a cluster's shared memory (above 393216 scores): one CTA per column,
 // every pass reads the scores again.
-__global__ void __launch_bounds__(512) topk_long_kernel(const TopkArgs p) {
+__global__ void __launch_bounds__(512) topk_long_kernel(TopkArgs p) {
   __shared__ __align__(16) int hist[256];
   __shared__ unsigned long long s_scan[32];
   __shared__ uint32_t s_mn[32], s_mx[32];
   const int e = blockIdx.x, g = blockIdx.y;
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const int nw = nthr >> 5;
+  pdl_begin(p.ST, p.group_off, p.k_g, p.k_off);
   const int lo = p.group_off[g];
   const int L = p.group_off[g + 1] - lo;
   const int k = p.k_g[g];
@@ -678,32 +681,21 @@ __global__ void __launch_bounds__(512) topk_long_kernel(const TopkArgs p) {
 }
 
 template <int CL>
-static cudaError_t topk_cluster(const TopkArgs& p, int G, int span, cudaStream_t st) {
+static cudaError_t topk_cluster(const TopkArgs& p, int G, int span, LaunchStream st) {
   auto kern = topk_cluster_kernel<CL>;
   const int chunk = ((span + CL - 1) / CL + 8 * kStep - 1) / (8 * kStep) * (8 * kStep);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(p.E * CL), (unsigned)G);
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = (size_t)chunk * 4;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = CL;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  if (cfg.dynamicSmemBytes > 40 * 1024) {   // with the static part above the 48 KB default
+  const size_t smem = (size_t)chunk * 4;
+  if (smem > 40 * 1024) {   // with the static part above the 48 KB default
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)cfg.dynamicSmemBytes);
+                                               (int)smem);
     if (e != cudaSuccess) return e;
   }
-  return cudaLaunchKernelEx(&cfg, kern, p, chunk);
+  return launch_kernel(kern, dim3((unsigned)(p.E * CL), (unsigned)G), 256, smem, st, CL, p, chunk);
 }
 
 constexpr int kClusterKeys = 49152;   // 192 KB of keys per CTA
 
-cudaError_t launch_topk(const TopkArgs& p, int G, int max_group, bool aligned, cudaStream_t st) {
+cudaError_t launch_topk(const TopkArgs& p, int G, int max_group, bool aligned, LaunchStream st) {
   if (G == 0 || p.E == 0) return cudaSuccess;
   // The registers that hold the longest column: 4 scores per thread for short ones (a 256-token
   // column then uses 64 threads, not 16), else 16; 128 threads up to 2048, so that every
@@ -712,15 +704,14 @@ cudaError_t launch_topk(const TopkArgs& p, int G, int max_group, bool aligned, c
   // take up to 3 places more.
   const int span = max_group + (aligned ? 0 : 3);
   const dim3 grid(p.E, G);
-  if (span <= 512) topk_reg_kernel<4, 128, 8><<<grid, 128, 0, st>>>(p);
-  else if (span <= 2048) topk_reg_kernel<16, 128, 8><<<grid, 128, 0, st>>>(p);
-  else if (span <= 4096) topk_reg_kernel<16, 256, 4><<<grid, 256, 0, st>>>(p);
-  else if (span <= 8192) topk_reg_kernel<16, 512, 2><<<grid, 512, 0, st>>>(p);
-  else if (span <= 16384) return topk_cluster<2>(p, G, span, st);
-  else if (span <= 32768) return topk_cluster<4>(p, G, span, st);
-  else if (span <= 8 * kClusterKeys) return topk_cluster<8>(p, G, span, st);
-  else topk_long_kernel<<<grid, 512, 0, st>>>(p);
-  return cudaGetLastError();
+  if (span <= 512) return launch_kernel(topk_reg_kernel<4, 128, 8>, grid, 128, 0, st, 1, p);
+  if (span <= 2048) return launch_kernel(topk_reg_kernel<16, 128, 8>, grid, 128, 0, st, 1, p);
+  if (span <= 4096) return launch_kernel(topk_reg_kernel<16, 256, 4>, grid, 256, 0, st, 1, p);
+  if (span <= 8192) return launch_kernel(topk_reg_kernel<16, 512, 2>, grid, 512, 0, st, 1, p);
+  if (span <= 16384) return topk_cluster<2>(p, G, span, st);
+  if (span <= 32768) return topk_cluster<4>(p, G, span, st);
+  if (span <= 8 * kClusterKeys) return topk_cluster<8>(p, G, span, st);
+  return launch_kernel(topk_long_kernel, grid, 512, 0, st, 1, p);
 }
 
 // ------------------------------------------------------------------ capacity update
@@ -734,6 +725,7 @@ __global__ void __launch_bounds__(1024) set_capacity_kernel(const int* __restric
                                                             int* __restrict__ status) {
   __shared__ long long s_part[1024];
   __shared__ int s_bad;
+  pdl_begin(k_new, group_off);
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int chunk = (G + nthr - 1) / nthr;
   const int g0 = min(G, tid * chunk), g1 = min(G, g0 + chunk);
@@ -771,10 +763,10 @@ __global__ void __launch_bounds__(1024) set_capacity_kernel(const int* __restric
 }
 
 cudaError_t launch_set_capacity(const int* k_new, const int* group_off, int G, int M, int* k_g,
-                                int* k_off, int* status, cudaStream_t st) {
+                                int* k_off, int* status, LaunchStream st) {
   if (G <= 0) return cudaSuccess;
-  set_capacity_kernel<<<1, 1024, 0, st>>>(k_new, group_off, G, M, k_g, k_off, status);
-  return cudaGetLastError();
+  return launch_kernel(set_capacity_kernel, 1, 1024, 0, st, 1, k_new, group_off, G, M, k_g, k_off,
+                       status);
 }
 
 }  // namespace ecmoe

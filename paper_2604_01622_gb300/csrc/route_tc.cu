@@ -58,6 +58,7 @@ __device__ __forceinline__ uint32_t score_key(float v) {
 __global__ void tc_topk_rows_kernel(const float* __restrict__ S, int N, int E, int k,
                                     int* __restrict__ choice, float* __restrict__ tgate,
                                     float* __restrict__ Z) {
+  pdl_begin(S);
   constexpr int MAXC = 8;
   const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -107,6 +108,7 @@ constexpr int kTopkFastE = 64, kTopkFastK = 8;
 __global__ void __launch_bounds__(256)
 tc_topk_rows4_kernel(const float* __restrict__ S, int N, int E, int k, int* __restrict__ choice,
                      float* __restrict__ tgate, float* __restrict__ Z, int* __restrict__ slot) {
+  pdl_begin(S);
   const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int t = (int)(gt >> 2), j = threadIdx.x & 3;
   const bool ok = t < N;                  // the token's four threads agree
@@ -193,6 +195,7 @@ constexpr int kMaxE = 256;        // experts the ranking handles (8 mask words)
 __global__ void __launch_bounds__(kRankBlock)
 tc_rank_kernel(const int* __restrict__ choice, int N, int E, int k, int* __restrict__ slot,
                int* __restrict__ hist) {
+  pdl_begin(choice);
   __shared__ int s_cnt[kRankBlock / 32][kMaxE];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x * kRankBlock + threadIdx.x;
@@ -247,6 +250,7 @@ tc_rank_kernel(const int* __restrict__ choice, int N, int E, int k, int* __restr
 // over the blocks), total[e] = all tokens that chose e.
 __global__ void tc_block_scan_kernel(const int* __restrict__ hist, int nblk, int E,
                                      int* __restrict__ boff, int* __restrict__ total) {
+  pdl_begin(hist);
   __shared__ int s_warp[33];
   const int e = blockIdx.x;
   int carry = 0;
@@ -266,6 +270,7 @@ __global__ void tc_block_scan_kernel(const int* __restrict__ hist, int nblk, int
 // the padded rows in use.
 __global__ void tc_offsets_kernel(int E, int cap, const int* __restrict__ total,
                                   int* __restrict__ count, int* __restrict__ tiles) {
+  pdl_begin(total);
   __shared__ int s_warp[33];
   const int e = threadIdx.x;
   int c = e < E ? total[e] : 0;
@@ -290,6 +295,7 @@ __global__ void tc_fill_kernel(const int* __restrict__ choice, const float* __re
                                const int* __restrict__ count, const int* __restrict__ tiles,
                                int* __restrict__ row_token, float* __restrict__ row_gate,
                                int* __restrict__ slot, int* __restrict__ kept) {
+  pdl_begin(choice, tgate, boff, count, tiles);
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t NK = (int64_t)N * k;
   if (j < NK) {
@@ -322,29 +328,33 @@ __global__ void tc_fill_kernel(const int* __restrict__ choice, const float* __re
 cudaError_t launch_tc_route(const float* S, int N, int E, int k, int cap, int* choice,
                             float* tgate, float* Z, int* count, int* tiles, int* row_token,
                             float* row_gate, int* slot, int* kept, int* scratch,
-                            cudaStream_t st) {
+                            LaunchStream st) {
   if (N == 0) return cudaSuccess;
   if (E > kMaxE || k > 32 || k > E) return cudaErrorInvalidValue;
   const int nblk = (N + kRankBlock - 1) / kRankBlock;
   int* hist = scratch;                          // [nblk][E]
   int* boff = scratch + (size_t)nblk * E;       // [nblk][E]
   int* total = boff + (size_t)nblk * E;         // [E]
+  cudaError_t err;
   if (E % 4 == 0 && E <= kTopkFastE && k <= kTopkFastK) {
     // four threads per token; the slot map's -1 rows are written there too
-    tc_topk_rows4_kernel<<<(unsigned)(((int64_t)N * 4 + 255) / 256), 256, 0, st>>>(
-        S, N, E, k, choice, tgate, Z, slot);
+    err = launch_kernel(tc_topk_rows4_kernel, (unsigned)(((int64_t)N * 4 + 255) / 256), 256, 0, st, 1,
+                        S, N, E, k, choice, tgate, Z, slot);
   } else {
-    cudaError_t err = cudaMemsetAsync(slot, 0xFF, (size_t)N * E * sizeof(int), st);   // -1
+    err = cudaMemsetAsync(slot, 0xFF, (size_t)N * E * sizeof(int), st);   // -1
     if (err != cudaSuccess) return err;
-    tc_topk_rows_kernel<<<(N + 7) / 8, 256, 0, st>>>(S, N, E, k, choice, tgate, Z);
+    err = launch_kernel(tc_topk_rows_kernel, (N + 7) / 8, 256, 0, st, 1, S, N, E, k, choice, tgate, Z);
   }
-  tc_rank_kernel<<<nblk, kRankBlock, 0, st>>>(choice, N, E, k, slot, hist);
-  tc_block_scan_kernel<<<E, 256, 0, st>>>(hist, nblk, E, boff, total);
-  tc_offsets_kernel<<<1, kMaxE, 0, st>>>(E, cap, total, count, tiles);
+  if (err != cudaSuccess) return err;
+  err = launch_kernel(tc_rank_kernel, nblk, kRankBlock, 0, st, 1, choice, N, E, k, slot, hist);
+  if (err != cudaSuccess) return err;
+  err = launch_kernel(tc_block_scan_kernel, E, 256, 0, st, 1, hist, nblk, E, boff, total);
+  if (err != cudaSuccess) return err;
+  err = launch_kernel(tc_offsets_kernel, 1, kMaxE, 0, st, 1, E, cap, total, count, tiles);
+  if (err != cudaSuccess) return err;
   const int64_t threads = (int64_t)N * k + (int64_t)E * kPadRows;
-  tc_fill_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(
-      choice, tgate, N, E, k, boff, count, tiles, row_token, row_gate, slot, kept);
-  return cudaGetLastError();
+  return launch_kernel(tc_fill_kernel, (unsigned)((threads + 255) / 256), 256, 0, st, 1, choice, tgate,
+                       N, E, k, boff, count, tiles, row_token, row_gate, slot, kept);
 }
 
 // Scratch ints launch_tc_route needs for N tokens and E experts.
@@ -362,6 +372,7 @@ __global__ void tc_softmax_bwd_kernel(const float* __restrict__ S, const int* __
                                       const int* __restrict__ slot,
                                       const float* __restrict__ row_dgate, float* __restrict__ dZ,
                                       bf16* __restrict__ dZb, int N, int E, int Ep, int k) {
+  pdl_begin(S, choice, tgate, Z, slot, row_dgate);
   const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (t >= N) return;
@@ -400,12 +411,11 @@ __global__ void tc_softmax_bwd_kernel(const float* __restrict__ S, const int* __
 cudaError_t launch_tc_softmax_bwd(const float* S, const int* choice, const float* tgate,
                                   const float* Z, const int* slot, const float* row_dgate,
                                   float* dZ, bf16* dZb, int N, int E, int Ep, int k,
-                                  cudaStream_t st) {
+                                  LaunchStream st) {
   if (N == 0) return cudaSuccess;
   if (k > 32 || Ep % 32) return cudaErrorInvalidValue;
-  tc_softmax_bwd_kernel<<<(N + 7) / 8, 256, 0, st>>>(S, choice, tgate, Z, slot, row_dgate, dZ, dZb,
-                                                     N, E, Ep, k);
-  return cudaGetLastError();
+  return launch_kernel(tc_softmax_bwd_kernel, (N + 7) / 8, 256, 0, st, 1, S, choice, tgate, Z, slot,
+                       row_dgate, dZ, dZb, N, E, Ep, k);
 }
 
 }  // namespace ecmoe
