@@ -7,23 +7,20 @@ from __future__ import annotations
 
 import torch
 
-from . import (EC_BF16, EC_F32, ec_check_device, ec_ctx_create, ec_ctx_destroy,
+from . import (EC_BF16, EC_F32, _check, ec_check_device, ec_ctx_create, ec_ctx_destroy,
                ec_ctx_profile, ec_ctx_set_capacity, ec_ctx_set_profiling, ec_ctx_set_residual,
-               ec_ctx_set_tiles,
-               ec_ctx_set_shared, ec_ctx_set_workspace, ec_kernel_launches,
-               ec_moe_backward, ec_moe_backward_shared, ec_moe_forward, ec_moe_forward_shared,
-               ec_ctx_set_capacity_async, ec_route, ec_rows_per_expert, ec_tc_backward,
-               ec_tc_capacity, ec_tc_ctx_create, ec_tc_forward, ec_workspace_bytes)
+               ec_ctx_set_shared, ec_ctx_set_tiles, ec_ctx_set_workspace, ec_kernel_launches,
+               ec_rows_per_expert, ec_tc_capacity, ec_tc_ctx_create, ec_workspace_bytes, load)
 
 _DT = {"f32": (EC_F32, torch.float32), "bf16": (EC_BF16, torch.bfloat16)}
 
 
-def _p(t):
-    return None if t is None else t.data_ptr()
-
-
 def _stream(stream):
-    return (stream or torch.cuda.current_stream()).cuda_stream
+    """Handle of `stream`, or of the current device's current stream (asked for without making
+    a Stream object: 2.8 us of a call's host time)."""
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 class ECMoELayer:
@@ -53,7 +50,7 @@ class ECMoELayer:
 
     def set_capacity_async(self, k_g_dev, stream=None):
         """k_g from an int32 device tensor [G] in stream order (sum must keep M)."""
-        ec_ctx_set_capacity_async(self.ctx, k_g_dev.data_ptr(), _stream(stream))
+        self._call(load().ec_ctx_set_capacity_async, (k_g_dev,), stream)
 
     def set_residual(self, on: bool):
         """Y = X + EC(X) and dX = dY + EC input gradient (stacked layers)."""
@@ -63,61 +60,71 @@ class ECMoELayer:
         """Expert-GEMM tile policy: EC_TILES_AUTO, EC_TILES_256 or EC_TILES_512."""
         ec_ctx_set_tiles(self.ctx, policy)
 
+    def _call(self, fn, tensors, stream):
+        """One C call: context, the tensors' addresses (None: NULL), the stream."""
+        status = fn(self.ctx, *[None if t is None else t.data_ptr() for t in tensors],
+                    _stream(stream))
+        if status:
+            _check(self.ctx, status)
+
     def _empty(self, *shape, dtype=None):
-        return torch.empty(*shape, dtype=dtype or self.tdtype, device=self.device)
+        return torch.empty(shape, dtype=dtype or self.tdtype, device=self.device)
+
+    def _selection(self):
+        """Empty idx [E][M], gate [E][M] and S [E][N]."""
+        E, M, dev, f32 = self.E, self.M, self.device, torch.float32
+        return (torch.empty((E, M), dtype=torch.int32, device=dev),
+                torch.empty((E, M), dtype=f32, device=dev),
+                torch.empty((E, self.N), dtype=f32, device=dev))
+
+    def _grads(self, with_bias):
+        d, E, F, dev, f32 = self.d, self.E, self.d_ff, self.device, torch.float32
+        empty = torch.empty
+        return {
+            "dX": empty((self.N, d), dtype=self.tdtype, device=dev),
+            "dWr": empty((d, E), dtype=f32, device=dev),
+            "dbr": empty((E,), dtype=f32, device=dev) if with_bias else None,
+            "dWg": empty((E, d, F), dtype=f32, device=dev),
+            "dWu": empty((E, d, F), dtype=f32, device=dev),
+            "dWd": empty((E, F, d), dtype=f32, device=dev),
+        }
 
     def route(self, X=None, Wr=None, br=None, S_in=None, stream=None):
         """Selection only. Returns (idx [E][M] int32, gate [E][M] f32, S [E][N] f32)."""
-        idx = self._empty(self.E, self.M, dtype=torch.int32)
-        gate = self._empty(self.E, self.M, dtype=torch.float32)
-        S = self._empty(self.E, self.N, dtype=torch.float32)
-        ec_route(self.ctx, _p(X), _p(Wr), _p(br), _p(S_in), _p(S), _p(idx), _p(gate),
-                 _stream(stream))
+        idx, gate, S = self._selection()
+        self._call(load().ec_route, (X, Wr, br, S_in, S, idx, gate), stream)
         return idx, gate, S
 
     def forward(self, X, Wr, br, Wg, Wu, Wd, Y=None, stream=None, outputs=True, shared=None):
         """Y = EC-MoE(X) (+ shared experts). Returns (Y, idx, gate, S); idx/gate/S are None if
         outputs=False. shared = (Wg_s, Wu_s, Wd_s) in concatenated form when configured."""
         Y = self._empty(self.N, self.d) if Y is None else Y
-        idx = gate = S = None
-        if outputs:
-            idx = self._empty(self.E, self.M, dtype=torch.int32)
-            gate = self._empty(self.E, self.M, dtype=torch.float32)
-            S = self._empty(self.E, self.N, dtype=torch.float32)
+        idx, gate, S = self._selection() if outputs else (None, None, None)
+        lib = load()
         if self.d_ff_shared:
             Wgs, Wus, Wds = shared
-            ec_moe_forward_shared(self.ctx, _p(X), _p(Wr), _p(br), _p(Wg), _p(Wu), _p(Wd),
-                                  _p(Wgs), _p(Wus), _p(Wds), _p(Y), _p(idx), _p(gate), _p(S),
-                                  _stream(stream))
+            self._call(lib.ec_moe_forward_shared,
+                       (X, Wr, br, Wg, Wu, Wd, Wgs, Wus, Wds, Y, idx, gate, S), stream)
         else:
-            ec_moe_forward(self.ctx, _p(X), _p(Wr), _p(br), _p(Wg), _p(Wu), _p(Wd), _p(Y),
-                           _p(idx), _p(gate), _p(S), _stream(stream))
+            self._call(lib.ec_moe_forward, (X, Wr, br, Wg, Wu, Wd, Y, idx, gate, S), stream)
         # the backward pass reads these through the pointers the context remembered
         self._keep = (X, Wr, br, Wg, Wu, Wd, shared)
         return Y, idx, gate, S
 
     def backward(self, dY, grads=None, stream=None, with_bias=False):
         """Gradients of <dY, Y> for the last forward. Returns a dict of tensors."""
-        g = grads or {
-            "dX": self._empty(self.N, self.d),
-            "dWr": self._empty(self.d, self.E, dtype=torch.float32),
-            "dbr": self._empty(self.E, dtype=torch.float32) if with_bias else None,
-            "dWg": self._empty(self.E, self.d, self.d_ff, dtype=torch.float32),
-            "dWu": self._empty(self.E, self.d, self.d_ff, dtype=torch.float32),
-            "dWd": self._empty(self.E, self.d_ff, self.d, dtype=torch.float32),
-        }
+        g = grads or self._grads(with_bias)
+        main = (dY, g["dX"], g["dWr"], g.get("dbr"), g["dWg"], g["dWu"], g["dWd"])
         if self.d_ff_shared:
             for k, shape in (("dWg_s", (self.d, self.d_ff_shared)),
                              ("dWu_s", (self.d, self.d_ff_shared)),
                              ("dWd_s", (self.d_ff_shared, self.d))):
                 if g.get(k) is None:
                     g[k] = self._empty(*shape, dtype=torch.float32)
-            ec_moe_backward_shared(self.ctx, _p(dY), _p(g["dX"]), _p(g["dWr"]), _p(g.get("dbr")),
-                                   _p(g["dWg"]), _p(g["dWu"]), _p(g["dWd"]), _p(g["dWg_s"]),
-                                   _p(g["dWu_s"]), _p(g["dWd_s"]), _stream(stream))
+            self._call(load().ec_moe_backward_shared,
+                       main + (g["dWg_s"], g["dWu_s"], g["dWd_s"]), stream)
         else:
-            ec_moe_backward(self.ctx, _p(dY), _p(g["dX"]), _p(g["dWr"]), _p(g.get("dbr")),
-                            _p(g["dWg"]), _p(g["dWu"]), _p(g["dWd"]), _stream(stream))
+            self._call(load().ec_moe_backward, main, stream)
         return g
 
     def set_profiling(self, on: bool):
@@ -187,20 +194,12 @@ class TCMoELayer(ECMoELayer):
                     self._empty(self.N, self.k, dtype=torch.int32),
                     self._empty(self.E, dtype=torch.int32),
                     self._empty(self.N, self.E, dtype=torch.float32)]
-        ec_tc_forward(self.ctx, _p(X), _p(Wr), _p(br), _p(Wg), _p(Wu), _p(Wd), _p(Y),
-                      *[_p(t) for t in outs], _stream(stream))
+        self._call(load().ec_tc_forward, (X, Wr, br, Wg, Wu, Wd, Y, *outs), stream)
         self._keep = (X, Wr, br, Wg, Wu, Wd)
         return (Y, *outs)
 
     def backward(self, dY, grads=None, stream=None, with_bias=False):
-        g = grads or {
-            "dX": self._empty(self.N, self.d),
-            "dWr": self._empty(self.d, self.E, dtype=torch.float32),
-            "dbr": self._empty(self.E, dtype=torch.float32) if with_bias else None,
-            "dWg": self._empty(self.E, self.d, self.d_ff, dtype=torch.float32),
-            "dWu": self._empty(self.E, self.d, self.d_ff, dtype=torch.float32),
-            "dWd": self._empty(self.E, self.d_ff, self.d, dtype=torch.float32),
-        }
-        ec_tc_backward(self.ctx, _p(dY), _p(g["dX"]), _p(g["dWr"]), _p(g.get("dbr")),
-                       _p(g["dWg"]), _p(g["dWu"]), _p(g["dWd"]), _stream(stream))
+        g = grads or self._grads(with_bias)
+        self._call(load().ec_tc_backward,
+                   (dY, g["dX"], g["dWr"], g.get("dbr"), g["dWg"], g["dWu"], g["dWd"]), stream)
         return g
