@@ -24,7 +24,8 @@ struct VarRows {
 // Tile shapes of the expert GEMMs (the `tiles` argument below): 0 chooses per GEMM (256 x 512
 // pair tiles where the output columns fill them and the K loop is long enough to hide the
 // hand-over of their two accumulator halves, else 256 x 256), 1 always 256 x 256, 2 wide
-// tiles wherever the columns fill them. The dU GEMM takes 256 x 512 tiles only under
+// tiles wherever the columns fill them. With at most 128 rows per expert 0 takes one-CTA tiles of
+// 128 rows. The dU GEMM takes 256 x 512 tiles only under
 // policy 2 (and never with variable rows): its epilogue reads A and B per row and cannot
 // drain an accumulator half within the MMAs that cover it.
 
