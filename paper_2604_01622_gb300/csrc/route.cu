@@ -61,7 +61,7 @@ __device__ __forceinline__ int find_bin(const int (&c)[8], int remaining, int& a
 // largest leaves itself and the number of its equals that are taken.
 constexpr int kCand = 64;
 __device__ __forceinline__ void rank_candidates(const uint32_t* cand, int n, int remaining,
-                                                uint32_t* T, int* need) {
+                                                uint32_t* T, int* need, int* all = nullptr) {
   if ((int)threadIdx.x >= n) return;
   const uint32_t mine = cand[threadIdx.x];
   int gt = 0, eq = 0;
@@ -74,6 +74,7 @@ __device__ __forceinline__ void rank_candidates(const uint32_t* cand, int n, int
   if (gt < remaining && remaining <= gt + eq) {   // the same for equal keys
     *T = mine;
     *need = remaining - gt;
+    if (all) *all = remaining - gt == eq;   // whether that is all of them
   }
 }
 
@@ -296,10 +297,320 @@ __device__ __forceinline__ int4 ld_peer4(uint32_t addr) {
   return v;
 }
 
-// Columns above 8192 scores: one per cluster of CL CTAs of 256 threads, each with `chunk` keys
+// Columns of 8193 to 49152 scores: one CTA of NT threads with the column's keys in shared memory
+// (`chunk` of them, a multiple of kStep NT / 32). Warp w owns the keys [w wlen, (w+1) wlen), each
+// lane 16 consecutive ones of every kStep (16-byte units swizzled so that these reads and the
+// coalesced fills are free of bank conflicts).
+//
+// The k-th key is bracketed first: one key in 16 goes into a histogram, the sample's rank of the
+// k-th key plus and minus four standard deviations gives two bins, and only the keys between
+// them (6-10%) are listed, those above being counted by comparison; the radix passes then read
+// the list. If the k-th key is outside, or the list overflows (many equal scores), the passes
+// read all keys. Selected keys are found once, as a bit mask per lane, and compacted in order in
+// place: the list of a warp's selected keys is never longer than the keys it has read.
+//
+// What bounds it: instructions of the block-wide steps (listing the bracket 6 k of a column's 25 k
+// cycles, the selection masks 3 k, the load 4-7 k). The shared atomics of a full pass cost about
+// 21 cycles a warp, a third of the time before the bracket, and a cluster of four CTAs per
+// column paid 2.7 k cycles of barrier and search per pass: 256 columns of 32768 scores, 37 -> 29
+// us (with the slot map instead of the copy of the scores 39 -> 33); 128 of 16384, 16.5 -> 12.4.
+constexpr int kStep = 512;    // keys a warp handles at a time
+constexpr int kList = 4096;   // keys of the bracket
+
+template <int NT>
+__global__ void __launch_bounds__(NT, NT <= 512 ? 2 : 1) topk_block_kernel(TopkArgs p, int chunk) {
+  constexpr int nw = NT / 32, MAXS = 3;   // steps per warp: chunk <= MAXS kStep nw
+  extern __shared__ uint4 skeys4[];
+  uint32_t* skeys = reinterpret_cast<uint32_t*>(skeys4);
+  uint32_t* s_list = skeys + chunk;
+  __shared__ __align__(16) int hist[2][256];
+  __shared__ uint32_t s_mn[nw], s_mx[nw], s_cand[kCand], s_T;
+  __shared__ int s_gt[nw], s_eq[nw], s_bin[4], s_n, s_above, s_ncand, s_need, s_whole;
+  const int e = blockIdx.x, g = blockIdx.y;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_begin(p.ST, p.group_off, p.k_g, p.k_off);
+  const int lo = p.group_off[g];
+  const int L = p.group_off[g + 1] - lo;
+  const int k = p.k_g[g];
+  const int base = p.k_off[g];
+  const float* col = p.ST + (size_t)e * p.N + lo;
+  // place i is score c0 + i of the column, for i in [v0, v1)
+  const int v0 = (int)((reinterpret_cast<uintptr_t>(col) >> 2) & 3u), c0 = -v0, v1 = v0 + L;
+  const int wlen = chunk / nw, w0 = warp * wlen;
+  float* copy = p.S_copy ? p.S_copy + (size_t)e * p.N + lo + c0 : nullptr;
+  const bool cvec = (reinterpret_cast<uintptr_t>(copy) & 15u) == 0;
+  auto unit = [](int v) { return v ^ ((v >> 3) & 3); };   // where 16-byte unit v is kept
+  uint32_t mn = 0xFFFFFFFFu, mx = 0u;
+  for (int i0 = w0; i0 < w0 + wlen; i0 += kStep) {
+    const int i = i0 + lane * 4;
+    if (i0 >= v0 && i0 + kStep <= v1) {
+      float4 x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        x[u] = __ldg(reinterpret_cast<const float4*>(col + c0 + i + u * 128));
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (copy) {
+          float* dst = copy + i + u * 128;
+          if (cvec) {
+            *reinterpret_cast<float4*>(dst) = x[u];
+          } else {
+            dst[0] = x[u].x; dst[1] = x[u].y; dst[2] = x[u].z; dst[3] = x[u].w;
+          }
+        }
+        const uint4 q = make_uint4(score_key(x[u].x), score_key(x[u].y), score_key(x[u].z),
+                                   score_key(x[u].w));
+        mn = min(min(min(mn, q.x), min(q.y, q.z)), q.w);
+        mx = max(max(max(mx, q.x), max(q.y, q.z)), q.w);
+        skeys4[unit((i + u * 128) >> 2)] = q;
+      }
+    } else {
+      for (int u = 0; u < 4; ++u)
+        for (int j = i + u * 128; j < i + u * 128 + 4; ++j) {
+          uint32_t q = 0u;
+          if (j >= v0 && j < v1) {
+            const float v = __ldg(col + c0 + j);
+            if (copy) copy[j] = v;
+            q = score_key(v);
+            mn = min(mn, q);
+            mx = max(mx, q);
+          }
+          skeys[unit(j >> 2) * 4 + (j & 3)] = q;
+        }
+    }
+  }
+  if (k == 0) return;
+  mn = __reduce_min_sync(0xffffffffu, mn);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 0) { s_mn[warp] = mn; s_mx[warp] = mx; }
+  for (int i = tid; i < 512; i += NT) (&hist[0][0])[i] = 0;
+  if (tid == 0) s_n = s_above = s_ncand = 0;
+  __syncthreads();
+  mn = __reduce_min_sync(0xffffffffu, lane < nw ? s_mn[lane] : 0xFFFFFFFFu);
+  mx = __reduce_max_sync(0xffffffffu, lane < nw ? s_mx[lane] : 0u);
+
+  // the 16 keys of this lane from place i0 + 16 lane on, and which of them exist
+  auto load16 = [&](int i0, uint32_t (&q)[16]) -> uint32_t {
+    const int i = i0 + lane * 16;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint4 x = skeys4[unit((i >> 2) + u)];
+      q[4 * u] = x.x; q[4 * u + 1] = x.y; q[4 * u + 2] = x.z; q[4 * u + 3] = x.w;
+    }
+    if (i0 >= v0 && i0 + kStep <= v1) return 0xFFFFu;
+    const int a = min(max(v0 - i, 0), 16), z = min(max(v1 - i, 0), 16);
+    return a < z ? ((1u << z) - 1u) & ~((1u << a) - 1u) : 0u;
+  };
+  auto each = [&](auto f) {
+    for (int i0 = w0; i0 < w0 + wlen; i0 += kStep) {
+      uint32_t q[16];
+      const uint32_t ok = load16(i0, q);
+      if (ok == 0xFFFFu) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) f(q[j]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          if (ok >> j & 1u) f(q[j]);
+      }
+    }
+  };
+  auto excl = [&](int v, int& total) {   // exclusive scan over the warp
+    int incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    total = __shfl_sync(0xffffffffu, incl, 31);
+    return incl - v;
+  };
+  // bin of the rem-th largest key in histogram h, by one warp: out[0..2] = bin, keys above, in it
+  auto search = [&](const int* h, int rem, int* out, int n_out) {
+    const int4 x = *reinterpret_cast<const int4*>(h + lane * 8);
+    const int4 y = *reinterpret_cast<const int4*>(h + lane * 8 + 4);
+    const int c[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+    int above = 0, in = 0;
+    const int bin = find_bin(c, rem, above, in);
+    if (lane == 0) {
+      out[0] = bin;
+      if (n_out > 1) { out[1] = above; out[2] = in; }
+    }
+  };
+
+  int hi = mx == mn ? 0 : 32 - __clz(mx - mn);   // every offset key - org lies in [0, 2^hi)
+  uint32_t org = mn;
+  int remaining = k, b = 0, inside = L;
+  int listed = -1;                               // keys in the list, once they are bracketed
+  const int n_s = (v1 + 15) / 16 - (v0 + 15) / 16;
+  if (hi > 0 && n_s >= 64) {
+    const int shift = max(hi - 8, 0);
+    const uint32_t dmask = (1u << (hi - shift)) - 1u;
+    for (int i0 = w0; i0 < w0 + wlen; i0 += kStep) {
+      const int i = i0 + lane * 16;
+      if (i >= v0 && i < v1) atomicAdd(&hist[0][(skeys[unit(i >> 2) * 4] - mn) >> shift], 1);
+    }
+    __syncthreads();
+    const float c = (float)k * n_s / L, m = 4.0f * sqrtf(c * (n_s - c) / n_s) + 2.0f;
+    if (warp == 0 && c - m >= 1.0f) search(hist[0], (int)(c - m), s_bin, 1);
+    if (warp == 1 && c + m < n_s) search(hist[0], (int)ceilf(c + m), s_bin + 3, 1);
+    __syncthreads();
+    const uint32_t bhi = c - m >= 1.0f ? (uint32_t)s_bin[0] : dmask;
+    const uint32_t blo = c + m < n_s ? (uint32_t)s_bin[3] : 0u;
+    const uint32_t khi = (bhi << shift) + ((1u << shift) - 1u), klo = blo << shift;
+    int above = 0;
+    for (int i0 = w0; i0 < w0 + wlen; i0 += kStep) {
+      uint32_t q[16], in = 0u;
+      const uint32_t ok = load16(i0, q);
+      const uint32_t lowest = mn + klo, width = khi - klo, highest = mn + khi;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        above += q[j] > highest;   // (a place without a score holds key 0)
+        if (q[j] - lowest <= width) in |= 1u << j;
+      }
+      in &= ok;
+      int total;
+      int at = excl(__popc(in), total);
+      int first = 0;
+      if (lane == 0 && total) first = atomicAdd(&s_n, total);
+      at += __shfl_sync(0xffffffffu, first, 0);
+      // dynamic indexing would put q into local memory: the keys are read again
+      while (in) {
+        const int j = __ffs(in) - 1;
+        in &= in - 1u;
+        const int i = i0 + lane * 16 + j;
+        if (at < kList) s_list[at] = skeys[unit(i >> 2) * 4 + (i & 3)];
+        ++at;
+      }
+    }
+    above = __reduce_add_sync(0xffffffffu, above);
+    if (lane == 0) atomicAdd(&s_above, above);
+    if (tid < 256) hist[0][tid] = 0;
+    __syncthreads();
+    const int n = s_n, rem = k - s_above;
+    if (n <= kList && rem >= 1 && rem <= n) {
+      listed = inside = n;
+      remaining = rem;
+      org = mn + klo;
+      hi = khi == klo ? 0 : 32 - __clz(khi - klo);
+    }
+  }
+  uint32_t prefix = 0u, mask = hi == 32 ? 0u : ~((1u << hi) - 1u);
+  bool whole = false;   // every key that shares the prefix is selected
+  while (!whole && hi > 0) {
+    auto keys = [&](auto f) {
+      if (listed >= 0)
+        for (int i = tid; i < listed; i += NT) f(s_list[i]);
+      else
+        each(f);
+    };
+    if (inside <= kCand) {
+      keys([&](uint32_t key) {
+        const uint32_t u = key - org;
+        if (((u ^ prefix) & mask) == 0u) s_cand[atomicAdd(&s_ncand, 1)] = u;
+      });
+      __syncthreads();
+      rank_candidates(s_cand, inside, remaining, &s_T, &s_need, &s_whole);
+      __syncthreads();
+      prefix = s_T;
+      remaining = s_need;
+      whole = s_whole;
+      break;
+    }
+    const int shift = max(hi - 8, 0);
+    const uint32_t dmask = (1u << (hi - shift)) - 1u;
+    // the other buffer was last read before the previous pass's second barrier
+    if (tid < 256) hist[b ^ 1][tid] = 0;
+    int* h = hist[b];
+    keys([&](uint32_t key) {
+      const uint32_t u = key - org;
+      if (((u ^ prefix) & mask) == 0u) atomicAdd(&h[(u >> shift) & dmask], 1);
+    });
+    __syncthreads();
+    if (warp == 0) search(h, remaining, s_bin, 3);
+    __syncthreads();
+    prefix |= (uint32_t)s_bin[0] << shift;
+    remaining -= s_bin[1];
+    inside = s_bin[2];
+    whole = inside == remaining;
+    mask |= dmask << shift;
+    hi = shift;
+    b ^= 1;
+  }
+  // every key >= T is selected if all that share the prefix are, else those above T and the first
+  // `remaining` equal to it
+  const uint32_t T = prefix + org;
+  const int need_eq = remaining;
+  uint32_t sel[MAXS];   // per step: keys above T in the low half, equal to T in the high half
+  int gt = 0, eq = 0;
+#pragma unroll
+  for (int t = 0; t < MAXS; ++t) {
+    sel[t] = 0u;
+    if (t * kStep < wlen) {
+      uint32_t q[16];
+      const uint32_t ok = load16(w0 + t * kStep, q);
+      if (whole) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          if (q[j] >= T) sel[t] |= 1u << j;
+      } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          if (q[j] > T) sel[t] |= 1u << j;
+          if (q[j] == T) sel[t] |= 0x10000u << j;
+        }
+      }
+      sel[t] &= ok | ok << 16;
+      gt += __popc(sel[t] & 0xFFFFu);
+      eq += __popc(sel[t] >> 16);
+    }
+  }
+  gt = __reduce_add_sync(0xffffffffu, gt);
+  eq = __reduce_add_sync(0xffffffffu, eq);
+  if (lane == 0) { s_gt[warp] = gt; s_eq[warp] = eq; }
+  __syncthreads();
+  const int gt0 = __reduce_add_sync(0xffffffffu, lane < warp ? s_gt[lane] : 0);   // lower warps'
+  int eq0 = __reduce_add_sync(0xffffffffu, lane < warp ? s_eq[lane] : 0);
+  const int first = gt0 + min(eq0, need_eq);   // selected keys before this warp's
+  int n = 0;                                   // selected keys of this warp so far
+#pragma unroll
+  for (int t = 0; t < MAXS; ++t) {
+    if (t * kStep >= wlen) break;
+    uint32_t seq = sel[t] >> 16;
+    if (__any_sync(0xffffffffu, seq)) {
+      int all;
+      const int before = eq0 + excl(__popc(seq), all);
+      eq0 += all;
+      while (__popc(seq) > max(need_eq - before, 0)) seq &= ~(0x80000000u >> __clz(seq));
+    }
+    uint32_t m = (sel[t] & 0xFFFFu) | seq;
+    int all;
+    int at = w0 + n + excl(__popc(m), all);
+    n += all;
+    while (m) {   // the masks hold all that is still needed of the keys
+      const int j = __ffs(m) - 1;
+      m &= m - 1u;
+      skeys[at++] = (uint32_t)(w0 + t * kStep + lane * 16 + j);
+    }
+  }
+  __syncwarp();
+  const size_t row = (size_t)e * p.M + base + first;
+#pragma unroll 4
+  for (int i = lane; i < n; i += 32) {
+    const int c = c0 + (int)skeys[w0 + i], t = lo + c;
+    const float sv = __ldg(col + c);
+    p.idx[row + i] = t;
+    p.gate[row + i] = sv;
+    if (p.idx2) p.idx2[row + i] = t;
+    if (p.gate2) p.gate2[row + i] = sv;
+    if (p.slot) p.slot[(size_t)t * p.E + e] = base + first + i;
+  }
+}
+
+// Columns above 49152 scores: one per cluster of CL CTAs of 256 threads, each with `chunk` keys
 // (a multiple of 8 kStep) in its shared memory, so that several CTAs per SM cover one another's
 // loads and barriers. The CTAs add up their histograms through distributed shared memory, one
-// cluster barrier per pass; once at most kList keys share the k-th key's prefix, each CTA lists
+// cluster barrier per pass; once at most kTail keys share the k-th key's prefix, each CTA lists
 // its own of them and the later passes read the lists. Warp w owns the keys
 // [w chunk/8, (w+1) chunk/8), each lane 16 consecutive ones of every kStep (16-byte units
 // swizzled so that these reads and the coalesced fills are free of bank conflicts), and compacts
@@ -307,11 +618,9 @@ __device__ __forceinline__ int4 ld_peer4(uint32_t addr) {
 // read.
 //
 // What bounds it: the first pass's shared atomics (about 21 cycles a warp) and the cluster
-// barriers (1-1.4 k cycles each with the search behind them); 256 columns of 32768 scores take
-// 37 us, or 39 with the slot map instead of the copy of the scores (one CTA of 131 KB of keys
-// per column took 74 us; keys in registers, 2 CTAs per SM, 55 us; 4 to 6 CTAs per SM the same).
-constexpr int kStep = 512;   // keys a warp handles at a time
-constexpr int kList = 512;
+// barriers (1-1.4 k cycles each with the search behind them); 64 columns of 131072 scores take
+// 52 us.
+constexpr int kTail = 512;
 
 template <int CL>
 __global__ void __launch_bounds__(256, 4) topk_cluster_kernel(TopkArgs p, int chunk) {
@@ -319,7 +628,7 @@ __global__ void __launch_bounds__(256, 4) topk_cluster_kernel(TopkArgs p, int ch
   extern __shared__ uint4 skeys4[];
   uint32_t* skeys = reinterpret_cast<uint32_t*>(skeys4);
   __shared__ __align__(16) int hist[3][256];
-  __shared__ uint32_t s_mn[TW], s_mx[TW], s_keys[kList];
+  __shared__ uint32_t s_mn[TW], s_mx[TW], s_keys[kTail];
   __shared__ int s_gt[TW], s_eq[TW], s_bin[3], s_n;
   const int rank = (int)cluster_rank();
   const int e = blockIdx.x / CL, g = blockIdx.y;
@@ -420,7 +729,7 @@ __global__ void __launch_bounds__(256, 4) topk_cluster_kernel(TopkArgs p, int ch
     const int bn = b == 2 ? 0 : b + 1;
     hist[bn][tid] = 0;
     int* h = hist[b];
-    if (listed < 0 && inside <= kList) {
+    if (listed < 0 && inside <= kTail) {
       each([&](uint32_t key) {
         if ((((key - mn) ^ prefix) & mask) == 0u) s_keys[atomicAdd(&s_n, 1)] = key;
       });
@@ -693,23 +1002,35 @@ static cudaError_t topk_cluster(const TopkArgs& p, int G, int span, LaunchStream
   return launch_kernel(kern, dim3((unsigned)(p.E * CL), (unsigned)G), 256, smem, st, CL, p, chunk);
 }
 
+template <int NT>
+static cudaError_t topk_block(const TopkArgs& p, int G, int span, LaunchStream st) {
+  auto kern = topk_block_kernel<NT>;
+  constexpr int unit = kStep * NT / 32;
+  const int chunk = (span + unit - 1) / unit * unit;
+  const size_t smem = ((size_t)chunk + kList) * 4;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(kern, dim3(p.E, G), NT, smem, st, 1, p, chunk);
+}
+
 constexpr int kClusterKeys = 49152;   // 192 KB of keys per CTA
 
 cudaError_t launch_topk(const TopkArgs& p, int G, int max_group, bool aligned, LaunchStream st) {
   if (G == 0 || p.E == 0) return cudaSuccess;
   // The registers that hold the longest column: 4 scores per thread for short ones (a 256-token
   // column then uses 64 threads, not 16), else 16; 128 threads up to 2048, so that every
-  // column of a 16-sequence batch is resident at once. Beyond 8192 scores a column is spread
-  // over a cluster, 8192 scores per CTA up to 8 CTAs. Columns that start off the 16-byte grid
-  // take up to 3 places more.
+  // column of a 16-sequence batch is resident at once. Above 8192 scores the keys go to shared
+  // memory, of one CTA up to 49152, else of a cluster of eight. Columns that start off the
+  // 16-byte grid take up to 3 places more.
   const int span = max_group + (aligned ? 0 : 3);
   const dim3 grid(p.E, G);
   if (span <= 512) return launch_kernel(topk_reg_kernel<4, 128, 8>, grid, 128, 0, st, 1, p);
   if (span <= 2048) return launch_kernel(topk_reg_kernel<16, 128, 8>, grid, 128, 0, st, 1, p);
   if (span <= 4096) return launch_kernel(topk_reg_kernel<16, 256, 4>, grid, 256, 0, st, 1, p);
   if (span <= 8192) return launch_kernel(topk_reg_kernel<16, 512, 2>, grid, 512, 0, st, 1, p);
-  if (span <= 16384) return topk_cluster<2>(p, G, span, st);
-  if (span <= 32768) return topk_cluster<4>(p, G, span, st);
+  if (span <= 16384) return topk_block<512>(p, G, span, st);
+  if (span <= 49152) return topk_block<1024>(p, G, span, st);
   if (span <= 8 * kClusterKeys) return topk_cluster<8>(p, G, span, st);
   return launch_kernel(topk_long_kernel, grid, 512, 0, st, 1, p);
 }
