@@ -199,12 +199,10 @@ void layout(ec_ctx* c) {
   c->o_dXr = take(N * d * es);   // the router's part of dX, in the layer dtype
   c->o_colsum = take((size_t)std::max(colsum_scratch_floats((int)N, (int)E),
                                        router_bwd_scratch_floats((int)N, (int)E)) * 4);
-  // split-K partials of dWr = X^T dZ (tensor cores: equal token blocks, so N % splits == 0)
+  // split-K partials of dWr = X^T dZ
   if (use_tc(c)) {
-    c->wr_splits = 1;
-    for (int s = 16; s > 1; s >>= 1)
-      if (N % s == 0 && N / s >= 256) { c->wr_splits = s; break; }
-    c->o_part = take((size_t)2 * c->wr_splits * d * c->Ep * 4);
+    c->wr_splits = router_wgrad_splits((int)N, (int)d, c->Ep);
+    c->o_part = take((size_t)c->wr_splits * d * c->Ep * 4);
   } else {
     // one split per 64 tokens (at most 64): X^T dZ has only d*E outputs for the whole GPU
     c->wr_splits = (int)std::max<size_t>(1, std::min<size_t>(64, N / 64));
@@ -286,8 +284,8 @@ SimtGemmArgs sg(const float* A, int64_t a_bs, int64_t a_ld, bool a_kfast, const 
 
 const float* f32p(const void* p) { return static_cast<const float*>(p); }
 
-// The router weights as the tensor cores read them, [d][Ep] bf16: Wr itself when E is a
-// multiple of 64, else the zero-padded copy the forward pass made.
+// The router weights as the tensor cores read them: Wr itself when E is a multiple of 8, else the
+// zero-padded copy [d][Ep] the forward pass made.
 const void* router_b(ec_ctx* c) {
   return router_needs_pad(c->E) ? at<void>(c, c->o_wrpad) : c->Wr;
 }
@@ -547,6 +545,27 @@ ec_status run_forward(ec_ctx* c, const void* X, const void* Wg, const void* Wu, 
 }
 
 // ---------------------------------------------------------------- backward
+// dWr = X^T dZ on the tensor cores: straight into dWr for a single block of tokens (rows of E
+// floats need 16-byte multiples), else partial sums and their sum in order.
+ec_status router_wgrad(ec_ctx* c, const bf16* dZb, float* dWr, LaunchStream st) {
+  const int N = c->N, d = c->d, E = c->E, Ep = c->Ep;
+  int* status = at<int>(c, c->o_status);
+  if (N == 0) {
+    EC_CUDA(cudaMemsetAsync(dWr, 0, (size_t)d * E * 4, st), "zero dWr");
+    return EC_OK;
+  }
+  if (c->wr_splits == 1 && E % 4 == 0) {
+    EC_KERNEL("router_wgrad_gemm", 1, tc_router_wgrad(c->X, dZb, dWr, E, N, d, Ep, 1, status, st));
+    return EC_OK;
+  }
+  float* part = at<float>(c, c->o_part);
+  EC_KERNEL("router_wgrad_gemm", 1,
+            tc_router_wgrad(c->X, dZb, part, Ep, N, d, Ep, c->wr_splits, status, st));
+  EC_KERNEL("router_wgrad_reduce", 1,
+            launch_reduce_partials(part, dWr, d, E, Ep, c->wr_splits, st));
+  return EC_OK;
+}
+
 template <typename T>
 ec_status run_backward(ec_ctx* c, const void* dY, void* dX, float* dWr, float* dbr, float* dWg,
                        float* dWu, float* dWd, float* dWgs, float* dWus, float* dWds,
@@ -592,7 +611,6 @@ ec_status run_backward(ec_ctx* c, const void* dY, void* dX, float* dWr, float* d
   }
   // router: dZ = S (dS - <dS,S>), dX = dZ Wr^T + sum dH, dWr = X^T dZ, dbr = sum dZ
   T* dXr = at<T>(c, c->o_dXr);
-  float* part = at<float>(c, c->o_part);
   const T* res = c->residual ? dYt : nullptr;
   // Up to 128 experts one kernel sums the gate-gradient partials, applies the softmax
   // Jacobian and takes the bias gradient's column sums (plus one kernel that adds those up).
@@ -613,13 +631,10 @@ ec_status run_backward(ec_ctx* c, const void* dY, void* dX, float* dWr, float* d
                 launch_softmax_bwd(S, slot, dgsum, dZ, dZb, N, E, c->Ep, M, st));
     }
     EC_KERNEL("router_dgrad_gemm", nz,
-              tc_router_dgrad(dZb, router_b(c), dXr, N, d, c->Ep, status, st));
+              tc_router_dgrad(dZb, router_b(c), dXr, N, d, E, status, st));
     EC_KERNEL("dx_combine", nz,
               launch_dx_combine<T>(dH, slot, dXr, res, dHsh, static_cast<T*>(dX), N, E, M, d, st));
-    EC_KERNEL("router_wgrad_gemm", nz,
-              tc_router_wgrad(c->X, dZb, part, N, d, c->Ep, c->wr_splits, status, st));
-    EC_KERNEL("router_wgrad_reduce", 1,
-              launch_reduce_partials(part, dWr, d, E, c->Ep, 2 * c->wr_splits, st));
+    EC_TRY(router_wgrad(c, dZb, dWr, st));
   } else {
     if (fused)
       EC_KERNEL("softmax_bwd", rb_launches,
@@ -633,6 +648,7 @@ ec_status run_backward(ec_ctx* c, const void* dY, void* dX, float* dWr, float* d
                                st));
     EC_KERNEL("dx_combine", nz,
               launch_dx_combine<T>(dH, slot, dXr, res, dHsh, static_cast<T*>(dX), N, E, M, d, st));
+    float* part = at<float>(c, c->o_part);
     SimtGemmArgs a = sg(f32p(c->X), 0, d, false, dZ, 0, E, false, part, 0, E, d, E, N, 1);
     a.splits = c->wr_splits;
     a.c_split = (int64_t)d * E;
@@ -729,22 +745,17 @@ ec_status run_tc_backward(ec_ctx* c, const void* dY, void* dX, float* dWr, float
   float* dZ = at<float>(c, c->o_dZ);
   bf16* dZb = at<bf16>(c, c->o_dZb);
   bf16* dXr = at<bf16>(c, c->o_dXr);
-  float* part = at<float>(c, c->o_part);
   float* dgsum = at<float>(c, c->o_dgsum);
   EC_KERNEL("dgate_reduce", 1, launch_reduce_splits(row_dgate, dgsum, c->P_tc, c->dg_parts, st));
   EC_KERNEL("softmax_bwd", 1,
             launch_tc_softmax_bwd(at<float>(c, c->o_S), at<int>(c, c->o_choice),
                                   at<float>(c, c->o_tgate), at<float>(c, c->o_Zs), slot, dgsum, dZ,
                                   dZb, N, E, c->Ep, k, st));
-  EC_KERNEL("router_dgrad_gemm", 1,
-            tc_router_dgrad(dZb, router_b(c), dXr, N, d, c->Ep, status, st));
+  EC_KERNEL("router_dgrad_gemm", 1, tc_router_dgrad(dZb, router_b(c), dXr, N, d, E, status, st));
   EC_KERNEL("dx_combine", 1,
             launch_dx_combine<bf16>(dH, slot, dXr, c->residual ? dYt : nullptr, nullptr,
                                     static_cast<bf16*>(dX), N, E, 0, d, st));
-  EC_KERNEL("router_wgrad_gemm", 1,
-            tc_router_wgrad(c->X, dZb, part, N, d, c->Ep, c->wr_splits, status, st));
-  EC_KERNEL("router_wgrad_reduce", 1,
-            launch_reduce_partials(part, dWr, d, E, c->Ep, 2 * c->wr_splits, st));
+  EC_TRY(router_wgrad(c, dZb, dWr, st));
   if (dbr)
     EC_KERNEL("router_dbias", 2, launch_colsum(dZ, dbr, N, E, at<float>(c, c->o_colsum), st));
   return EC_OK;

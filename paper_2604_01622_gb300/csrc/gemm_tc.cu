@@ -37,6 +37,7 @@ enum Epi : int {
   EPI_SWIGLU_BWD = 3,    // acc = dU; reads A, B; writes dA, dB bf16
   EPI_STORE_F32 = 4,     // plain fp32 store
   EPI_STORE_F32_SPLIT = 5, // cols [0,BN/2) -> out0, [BN/2,BN) -> out1, fp32
+  EPI_STORE_F32_SUM = 7, // cols [0,BN/2) + [BN/2,BN) -> out0, fp32
   EPI_ROUTER_ST = 6      // the router softmax with S and S^T leaving by TMA stores (BN <= 128)
 };
 
@@ -387,7 +388,8 @@ __device__ __forceinline__ void bulk_wait_all() {
 // gradients: K runs over the expert's padded rows); 3 one problem whose rows are split
 // evenly over the CTAs in 32-row units (the router: every CTA streams its own contiguous
 // block of tokens, in tiles of up to 128 rows, so no SM is left with a second wave of whole
-// tiles while others idle).
+// tiles while others idle); 4 one problem whose K rows are split into blocks of k_blocks
+// k-slices, the last one shorter, as the output's batch (the router's weight gradient).
 struct Tile {
   int b, mt, nt;
   int row0;      // first row of this CTA in the A / output row space
@@ -441,6 +443,9 @@ __device__ __forceinline__ Tile tile_at(const Args& p, int tile, int tiles_per_b
     if constexpr (VARM == 2) {
       t.kbl = (__ldg(p.vm_count + t.b) + BK - 1) / BK;
       t.krow0 = __ldg(p.vm_tiles + t.b) * PADR;
+    } else if constexpr (VARM == 4) {
+      t.kbl = min(p.k_blocks, (p.K + BK - 1) / BK - t.b * p.k_blocks);
+      t.krow0 = t.b * p.k_blocks * BK;
     } else {
       t.kbl = p.k_blocks;
       t.krow0 = 0;
@@ -561,7 +566,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
         const int nt = T.nt;
         const int m0 = T.row0;
         const int ab = VARM ? 0 : T.b;          // batch coordinate of A
-        const int bb = VARM == 2 ? 0 : T.b;     // batch coordinate of B
+        const int bb = VARM == 2 || VARM == 4 ? 0 : T.b;     // batch coordinate of B
         for (int kb = 0; kb < T.kbl; ++kb) {
           if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag, p.status)) { ok = false; break; }
           if (!PAIR || leader) mbar_arrive_expect_tx(&full[s], (A_BYTES + B_BYTES) * (PAIR ? 2 : 1));
@@ -1054,6 +1059,21 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
               else put_f32(&mO0, n, f);
             }
           }
+        } else if constexpr (EPI == EPI_STORE_F32_SUM) {
+          uint32_t w[32];
+          constexpr int NC64 = SEGW / 64 / NPART;
+#pragma unroll 1
+          for (int c = part * NC64; c < (part + 1) * NC64; ++c) {
+            tmem_ld32(tacc + c * 32, v);
+            tmem_ld32(tacc + SEGW / 2 + c * 32, w);
+            tmem_wait_ld();
+            const int n = nt * (BN / 2) + c * 32;
+            if (st_any && n < p.N) {
+#pragma unroll
+              for (int i = 0; i < 32; ++i) f[i] = f32(v[i]) + f32(w[i]);
+              put_f32(&mO0, n, f);
+            }
+          }
         } else if constexpr (EPI == EPI_STORE_F32_SPLIT) {
 #pragma unroll 1
           for (int c = c32; c < c32 + NC32; ++c) {
@@ -1441,14 +1461,15 @@ __global__ void wait_probe_kernel(int* status, unsigned long long limit) {
     if (_e != cudaSuccess) return _e;    \
   } while (0)
 
-bool router_needs_pad(int E) { return E % 64 != 0; }
+// Rows of Wr [d][E] must be a multiple of 16 bytes for the tensor map; the columns up to the next
+// multiple of 64 are then filled with zeros by the loads.
+bool router_needs_pad(int E) { return E % 8 != 0; }
 
 cudaError_t tc_router_softmax(const void* X, const void* Wr, void* Wr_pad, const float* br,
                               float* S, float* ST, int* slot_init, int N, int d, int E,
                               int* status, LaunchStream st) {
   if (N == 0) return cudaSuccess;
   const int Ep = (E + 63) / 64 * 64;
-  // Wr [d][E] already has the padded layout when E is a multiple of 64
   const void* Wb = Wr;
   if (router_needs_pad(E)) {
     TC_TRY(launch_kernel(pad_router_weights, 256, 256, 0, st, 1, static_cast<const bf16*>(Wr),
@@ -1457,7 +1478,7 @@ cudaError_t tc_router_softmax(const void* X, const void* Wr, void* Wr_pad, const
   }
   CUtensorMap ma, mb;
   TC_TRY(make_map(&ma, X, d, N, 1, BM));
-  TC_TRY(make_map(&mb, Wb, Ep, d, 1, 64));
+  TC_TRY(make_map(&mb, Wb, router_needs_pad(E) ? Ep : E, d, 1, 64));
   Args p = base_args(1, N, Ep, d, Ep, status);
   p.out0 = S;
   p.out1 = ST;
@@ -1744,16 +1765,17 @@ cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const 
   return cudaSuccess;
 }
 
-cudaError_t tc_router_dgrad(const void* dZb, const void* Wr_pad, void* dXr, int N, int d, int Ep,
+cudaError_t tc_router_dgrad(const void* dZb, const void* Wr, void* dXr, int N, int d, int E,
                             int* status, LaunchStream st) {
+  const int Ep = (E + 63) / 64 * 64;
   if (N == 0) return cudaSuccess;
   // dXr [N][d] = (dZ_hi + dZ_lo) [N][Ep] . Wr^T as one K loop over both planes;
-  // B[n=i][k=e] = Wr_pad[i][e] is K-major
+  // B[n=i][k=e] = Wr[i][e] is K-major
   const bf16* hi = static_cast<const bf16*>(dZb);
   CUtensorMap ma0, ma1, mb;
   TC_TRY(make_map(&ma0, hi, Ep, N, 1, BM));
   TC_TRY(make_map(&ma1, hi + (size_t)N * Ep, Ep, N, 1, BM));
-  TC_TRY(make_map(&mb, Wr_pad, Ep, d, 1, 256));
+  TC_TRY(make_map(&mb, Wr, router_needs_pad(E) ? Ep : E, d, 1, 256));
   CUtensorMap mo;
   TC_TRY(make_out_map(&mo, dXr, false, d, N, 1));
   Args p = base_args(1, N, d, 2 * Ep, 256, status);
@@ -1765,31 +1787,40 @@ cudaError_t tc_router_dgrad(const void* dZb, const void* Wr_pad, void* dXr, int 
                                                                    st);
 }
 
-cudaError_t tc_router_wgrad(const void* X, const void* dZb, float* part, int N, int d, int Ep,
+// Splits of X^T.dZ over the tokens: as many as make one wave of output tiles (128 rows of d x up
+// to 128 experts), each of at least two k-slices. More tiles than SMs cost a second wave for
+// nothing (16 splits at d 2048 were 1.7 waves), and each split is a partial sum to write and read
+// back.
+int router_wgrad_splits(int N, int d, int Ep) {
+  const int tiles = ((d + BM - 1) / BM) * ((Ep + 127) / 128), blocks = (N + BK - 1) / BK;
+  const int want = tiles < 152 ? 152 / tiles : 1;
+  const int most = blocks / 2 > 0 ? blocks / 2 : 1;
+  const int s = want < most ? want : most;
+  const int per = (blocks + s - 1) / s;
+  return per > 0 ? (blocks + per - 1) / per : 1;
+}
+
+cudaError_t tc_router_wgrad(const void* X, const void* dZb, float* out, int ld, int N, int d, int Ep,
                             int splits, int* status, LaunchStream st) {
   if (N == 0) return cudaSuccess;
-  // part[h][s] [d][Ep] = X_s^T . dZ_h,s over the s-th block of N/splits tokens (split K as the
-  // batch), h = hi / lo plane of dZ (the two column halves of each tile)
-  const int rows = N / splits;
+  // out[s] [d][ld] = X_s^T . dZ_s over the s-th block of tokens; the two column halves of a tile
+  // are the hi and lo planes of dZ, added in the epilogue
   const bf16* hi = static_cast<const bf16*>(dZb);
-  CUtensorMap ma, mb0, mb1;
-  TC_TRY(make_map(&ma, X, d, rows, splits, 64));
-  TC_TRY(make_map(&mb0, hi, Ep, rows, splits, 64));
-  TC_TRY(make_map(&mb1, hi + (size_t)N * Ep, Ep, rows, splits, 64));
-  CUtensorMap mo0, mo1;
-  TC_TRY(make_out_map(&mo0, part, true, Ep, d, splits));
-  TC_TRY(make_out_map(&mo1, part + (size_t)splits * d * Ep, true, Ep, d, splits));
+  CUtensorMap ma, mb0, mb1, mo;
+  TC_TRY(make_map(&ma, X, d, N, 1, 64));
+  TC_TRY(make_map(&mb0, hi, Ep, N, 1, 64));
+  TC_TRY(make_map(&mb1, hi + (size_t)N * Ep, Ep, N, 1, 64));
+  TC_TRY(make_out_map(&mo, out, true, ld, d, splits));
   const int BNt = Ep > 64 ? 256 : 128;
-  Args p = base_args(splits, d, Ep, rows, BNt / 2, status);
-  p.out0 = part;
-  p.out1 = part + (size_t)splits * d * Ep;
-  p.ld = Ep;
-  p.bstride = (int64_t)d * Ep;
+  Args p = base_args(splits, d, Ep, N, BNt / 2, status);
+  p.k_blocks = (p.k_blocks + splits - 1) / splits;
+  p.N = ld < Ep ? ld : Ep;   // columns past the output's are not stored
+  p.out0 = out;
   if (BNt == 128)
-    return launch<128, true, true, true, false, EPI_STORE_F32_SPLIT, 6>(ma, ma, mb0, mb1, mo0, mo1, mo1,
-                                                                        p, st);
-  return launch<256, true, true, true, false, EPI_STORE_F32_SPLIT, 4>(ma, ma, mb0, mb1, mo0, mo1, mo1,
-                                                                      p, st);
+    return launch<128, true, true, true, false, EPI_STORE_F32_SUM, 6, 8, false, 4>(
+        ma, ma, mb0, mb1, mo, mo, mo, p, st);
+  return launch<256, true, true, true, false, EPI_STORE_F32_SUM, 4, 8, false, 4>(
+      ma, ma, mb0, mb1, mo, mo, mo, p, st);
 }
 
 cudaError_t tc_wait_probe(int* status, unsigned long long limit_ns, LaunchStream st) {

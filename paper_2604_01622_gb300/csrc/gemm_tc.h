@@ -31,7 +31,7 @@ struct VarRows {
 
 // Router: Z = X.Wr (+br), S = row softmax over the E experts, written as S [N][E] (NULL: not
 // written) and S^T [E][N]. X [N][d] bf16, Wr [d][E] bf16. Wr_pad: device scratch of d*round_up(E,64)
-// bf16 (zero-padded copy of Wr made on the stream when E is not a multiple of 64,
+// bf16 (zero-padded copy of Wr made on the stream when E is not a multiple of 8,
 // router_needs_pad; otherwise Wr itself is read and Wr_pad is untouched). slot_init
 // (nullable): an int [N][E] map set to -1 beside S (the expert-choice slot map before
 // selection).
@@ -76,13 +76,15 @@ cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const 
                             const VarRows* vr = nullptr, int tiles = 0);
 
 // Router backward on the tensor cores. dZb [2][N][Ep] bf16: hi and lo planes of the
-// zero-padded softmax gradient (dZ ~ hi + lo); Wr_pad [d][Ep] bf16 (the padded router
-// weights of the forward pass). dXr [N][d] bf16 = dZ . Wr^T (summed in fp32, rounded once).
-cudaError_t tc_router_dgrad(const void* dZb, const void* Wr_pad, void* dXr, int N, int d, int Ep,
+// zero-padded softmax gradient (dZ ~ hi + lo); Wr: the router weights as the forward pass read
+// them (padded copy or in place). dXr [N][d] bf16 = dZ . Wr^T (summed in fp32, rounded once).
+cudaError_t tc_router_dgrad(const void* dZb, const void* Wr, void* dXr, int N, int d, int E,
                             int* status, LaunchStream st);
-// part [2][splits][d][Ep] fp32: X^T . dZ_plane over `splits` equal blocks of tokens
-// (N % splits == 0); dWr is the sum of all 2*splits partials.
-cudaError_t tc_router_wgrad(const void* X, const void* dZb, float* part, int N, int d, int Ep,
+// out [splits][d][ld] fp32 (ld >= E, a multiple of 4; columns from ld on are not written):
+// X^T . dZ over `splits` blocks of tokens (router_wgrad_splits, blocks of whole 64-token
+// k-slices); dWr is the sum of all partials.
+int router_wgrad_splits(int N, int d, int Ep);
+cudaError_t tc_router_wgrad(const void* X, const void* dZb, float* out, int ld, int N, int d, int Ep,
                             int splits, int* status, LaunchStream st);
 
 // Launch a kernel that waits, with the given limit, on an mbarrier nothing completes, so

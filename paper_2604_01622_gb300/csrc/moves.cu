@@ -544,8 +544,12 @@ cudaError_t launch_reduce_partials(const float* part, float* out, int rows, int 
                   (reinterpret_cast<uintptr_t>(part) & 15u) == 0 &&
                   (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
   const int64_t n = (int64_t)rows * cols / (v4 ? 4 : 1);
+  // few outputs: 64-thread CTAs spread them over more SMs
+  const int nt = n < 152 * 256 ? 64 : 256;
+  const int64_t blocks = (n + nt - 1) / nt;
   return launch_kernel(v4 ? reduce_partials_kernel<4> : reduce_partials_kernel<1>,
-                       grid_for(n, 152 * 16), 256, 0, st, 1, part, out, rows, cols, ld, splits);
+                       (unsigned)(blocks < 152 * 16 ? blocks : 152 * 16), nt, 0, st, 1, part, out,
+                       rows, cols, ld, splits);
 }
 
 // ------------------------------------------------------------------ dX_t = dXr_t + sum dH rows
