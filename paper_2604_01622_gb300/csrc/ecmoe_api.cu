@@ -45,7 +45,7 @@ struct ec_ctx {
   // state saved by the forward pass
   bool residual = false;   // Y = X + EC(X), dX = dY + EC input gradient
   int Fs = 0;              // shared experts: total hidden width (0 = none)
-  size_t o_Ash = 0, o_Bsh = 0, o_Ush = 0, o_Osh = 0, o_dAsh = 0, o_dBsh = 0, o_shpart = 0;
+  size_t o_Ash = 0, o_Bsh = 0, o_Ush = 0, o_Osh = 0, o_dAsh = 0, o_dBsh = 0;
   const void *Wgs = nullptr, *Wus = nullptr, *Wds = nullptr;
   float *dWgs = nullptr, *dWus = nullptr, *dWds = nullptr;
   bool have_fwd = false;
@@ -134,18 +134,6 @@ size_t esize(const ec_ctx* c) { return c->dtype == EC_BF16 ? 2 : 4; }
 
 bool use_tc(const ec_ctx* c) { return c->dtype == EC_BF16; }
 
-// SM pairs of the current device (the tensor-core GEMMs run one 2-CTA cluster per pair)
-int sm_pairs(const ec_ctx*) {
-  static int pairs = 0;
-  if (!pairs) {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    pairs = n > 1 ? n / 2 : 1;
-  }
-  return pairs;
-}
-
 void layout(ec_ctx* c) {
   const size_t N = c->N, d = c->d, E = c->E, F = c->F, M = c->M_cap, G = c->G, es = esize(c);
   // expert rows: E x M for expert choice; token choice keeps each expert's rows in a region
@@ -194,8 +182,6 @@ void layout(ec_ctx* c) {
   c->o_Osh = take(Fs ? N * d * es : 0);
   c->o_dAsh = take(N * Fs * es);
   c->o_dBsh = take(N * Fs * es);
-  // the shared FFN's dWd as two split-K halves (tensor cores; see ffn_backward)
-  c->o_shpart = take(use_tc(c) && Fs ? 2 * Fs * d * 4 : 0);
   c->o_dXr = take(N * d * es);   // the router's part of dX, in the layer dtype
   c->o_colsum = take((size_t)std::max(colsum_scratch_floats((int)N, (int)E),
                                        router_bwd_scratch_floats((int)N, (int)E)) * 4);
@@ -434,17 +420,12 @@ ec_status ffn_forward(ec_ctx* c, const FfnNames& nm, const T* H, const int* idx,
 // ones (as ffn_forward wrote them): dU = gate * dO.Wd^T, dWd = U^T.dO, and the gate
 // gradients <dO.Wd^T, silu(A) B> land in dgate_part (c->dg_parts partials, stride E*M).
 // fp32: H is gathered through idx as in ffn_forward.
-// dwd_split: optional scratch of 2*F*d floats for the single-FFN case (E = 1, the shared
-// experts), whose dWd = U^T.dO has few output tiles for the whole GPU and a K loop over all
-// M rows: the rows are split into two halves computed as two batch entries at once and
-// summed in order afterwards.
 template <typename T>
 ec_status ffn_backward(ec_ctx* c, const FfnNames& nm, const T* dO, const T* H, const int* idx,
                        const T* A, const T* B, const T* U, const void* Wg, const void* Wu,
                        const void* Wd,
                        T* dA, T* dB, T* dH, float* dWg, float* dWu, float* dWd, int E, int M, int F,
-                       LaunchStream st, const float* gate = nullptr, float* dgate_part = nullptr,
-                       float* dwd_split = nullptr) {
+                       LaunchStream st, const float* gate = nullptr, float* dgate_part = nullptr) {
   const int d = c->d;
   const int64_t P = (int64_t)E * M;
   if (P == 0) {
@@ -460,21 +441,11 @@ ec_status ffn_backward(ec_ctx* c, const FfnNames& nm, const T* dO, const T* H, c
                                  dgate_part, P, c->tiles));
     EC_KERNEL(nm.dgrad_h, 1,
               tc_expert_dgrad_h(dA, dB, Wg, Wu, dH, E, M, d, F, status, st, nullptr, c->tiles));
-    if (dwd_split && E == 1 && M % 2 == 0 && M >= 2048 &&
-        2 * ((F + 255) / 256) * ((d + 511) / 512) <= sm_pairs(c)) {
-      EC_KERNEL(nm.wgrad, 1,
-                tc_expert_wgrad(H, U, dO, dA, dB, dWg, dWu, nullptr, 1, M, d, F, status, st,
-                                nullptr, c->tiles));
-      EC_KERNEL(nm.wgrad, 1,
-                tc_expert_wgrad(H, U, dO, nullptr, nullptr, nullptr, nullptr, dwd_split, 2, M / 2,
-                                d, F, status, st, nullptr, c->tiles));
-      EC_KERNEL(nm.wgrad, 1,
-                launch_reduce_splits(dwd_split, dWd, (int64_t)F * d, 2, st));
-    } else {
-      EC_KERNEL(nm.wgrad, 2,
-                tc_expert_wgrad(H, U, dO, dA, dB, dWg, dWu, dWd, E, M, d, F, status, st, nullptr,
-                                c->tiles));
-    }
+    int launched = 0;
+    EC_KERNEL(nm.wgrad, 0,
+              tc_expert_wgrad(H, U, dO, dA, dB, dWg, dWu, dWd, E, M, d, F, status, st, &launched,
+                              nullptr, c->tiles));
+    c->launches += launched;
   } else {
     const int64_t hs = (int64_t)M * d, fs = (int64_t)M * F, wgs = (int64_t)d * F;
     // dU = dO . Wd^T (B[k=i][n=j] = Wd[j][i]), its SwiGLU backward in the epilogue
@@ -605,8 +576,7 @@ ec_status run_backward(ec_ctx* c, const void* dY, void* dX, float* dWr, float* d
     EC_TRY(ffn_backward<T>(c, kShared, dYt, static_cast<const T*>(c->X), nullptr, at<T>(c, c->o_Ash),
                            at<T>(c, c->o_Bsh), at<T>(c, c->o_Ush), c->Wgs, c->Wus, c->Wds,
                            at<T>(c, c->o_dAsh), at<T>(c, c->o_dBsh), dh, dWgs, dWus, dWds, 1, N,
-                           Fs, st, nullptr, nullptr,
-                           use_tc(c) ? at<float>(c, c->o_shpart) : nullptr));
+                           Fs, st));
     dHsh = dh;
   }
   // router: dZ = S (dS - <dS,S>), dX = dZ Wr^T + sum dH, dWr = X^T dZ, dbr = sum dZ
@@ -739,9 +709,11 @@ ec_status run_tc_backward(ec_ctx* c, const void* dY, void* dX, float* dWr, float
                                c->P_tc));
   EC_KERNEL("gemm_dgrad_h", 1,
             tc_expert_dgrad_h(dA, dB, c->Wg, c->Wu, dH, E, 0, d, F, status, st, &vr, c->tiles));
-  EC_KERNEL("gemm_wgrad", 2,
+  int launched = 0;
+  EC_KERNEL("gemm_wgrad", 0,
             tc_expert_wgrad(at<bf16>(c, c->o_H), at<bf16>(c, c->o_U), dO, dA, dB, dWg, dWu, dWd, E,
-                            0, d, F, status, st, &vr, c->tiles));
+                            0, d, F, status, st, &launched, &vr, c->tiles));
+  c->launches += launched;
   float* dZ = at<float>(c, c->o_dZ);
   bf16* dZb = at<bf16>(c, c->o_dZb);
   bf16* dXr = at<bf16>(c, c->o_dXr);

@@ -35,8 +35,9 @@ enum Epi : int {
   EPI_SWIGLU_FWD = 1,    // cols [0,BN/2) gate, [BN/2,BN) up -> A, B, U bf16
   EPI_STORE_BF16 = 2,    // plain bf16 store
   EPI_SWIGLU_BWD = 3,    // acc = dU; reads A, B; writes dA, dB bf16
-  EPI_STORE_F32 = 4,     // plain fp32 store
-  EPI_STORE_F32_SPLIT = 5, // cols [0,BN/2) -> out0, [BN/2,BN) -> out1, fp32
+  // The weight gradients, two problems in one tile list (fp32 stores): first C0 = A0.[B0|B1], cols
+  // [0,BN/2) -> out0, [BN/2,BN) -> out1; then C1 = A1.B2 -> out2.
+  EPI_WGRAD = 4,
   EPI_STORE_F32_SUM = 7, // cols [0,BN/2) + [BN/2,BN) -> out0, fp32
   EPI_ROUTER_ST = 6      // the router softmax with S and S^T leaving by TMA stores (BN <= 128)
 };
@@ -44,6 +45,7 @@ enum Epi : int {
 struct Args {
   int batch, M, N, K;           // C[b] is M x N (N per half for split-column epilogues)
   int m_tiles, n_tiles, k_blocks, k_blocks0;
+  int M2, N2, m_tiles2, n_tiles2;   // EPI_WGRAD: the second problem, C1[b] is M2 x N2
   void* out0;
   void* out1;
   void* out2;
@@ -392,17 +394,20 @@ __device__ __forceinline__ void bulk_wait_all() {
 // k-slices, the last one shorter, as the output's batch (the router's weight gradient).
 struct Tile {
   int b, mt, nt;
+  int prob;      // EPI_WGRAD: which problem
   int row0;      // first row of this CTA in the A / output row space
   int valid;     // rows from row0 that are real (the rest are masked)
   int kbl;       // k-blocks of this tile
   int krow0;     // first K row (variable K)
 };
 
-template <int VARM, int TM>
+template <int VARM, int TM, bool TWO>
 __device__ __forceinline__ Tile tile_at(const Args& p, int tile, int tiles_per_b, uint32_t rank) {
+  static_assert(!TWO || VARM == 0 || VARM == 2, "two problems: batches over the experts");
   static_assert(VARM != 1 || TM == PADR, "variable-row tiles are one padding unit high");
   static_assert(VARM != 3 || TM == BM, "row-split tiles are one CTA high");
   Tile t;
+  t.prob = 0;
   if constexpr (VARM == 3) {
     // CTA c owns the 32-row units [c U / G, (c+1) U / G) of the U = ceil(M / 32) units; its
     // j-th tile (tile = c + j G) starts 128 j rows into that block. valid <= 0: the CTA has
@@ -434,12 +439,22 @@ __device__ __forceinline__ Tile tile_at(const Args& p, int tile, int tiles_per_b
     t.kbl = p.k_blocks;
     t.krow0 = 0;
   } else {
-    t.b = tile / tiles_per_b;
-    const int rem = tile - t.b * tiles_per_b;
-    t.mt = rem / p.n_tiles;
-    t.nt = rem - t.mt * p.n_tiles;
+    int per_b = tiles_per_b, n_tiles = p.n_tiles, M = p.M;
+    if constexpr (TWO) {
+      if (tile >= p.batch * per_b) {
+        tile -= p.batch * per_b;
+        t.prob = 1;
+        n_tiles = p.n_tiles2;
+        per_b = p.m_tiles2 * n_tiles;
+        M = p.M2;
+      }
+    }
+    t.b = tile / per_b;
+    const int rem = tile - t.b * per_b;
+    t.mt = rem / n_tiles;
+    t.nt = rem - t.mt * n_tiles;
     t.row0 = t.mt * TM + (int)rank * BM;
-    t.valid = p.M - t.row0;
+    t.valid = M - t.row0;
     if constexpr (VARM == 2) {
       t.kbl = (__ldg(p.vm_count + t.b) + BK - 1) / BK;
       t.krow0 = __ldg(p.vm_tiles + t.b) * PADR;
@@ -472,6 +487,7 @@ template <int BN, bool A_MN, bool B_MN, bool B_SPLIT, bool K_SPLIT, int EPI, int
 __global__ void __launch_bounds__(64 + 32 * EPW, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
                const __grid_constant__ CUtensorMap mB0, const __grid_constant__ CUtensorMap mB1,
+               const __grid_constant__ CUtensorMap mB2,
                const __grid_constant__ CUtensorMap mO0, const __grid_constant__ CUtensorMap mO1,
                const __grid_constant__ CUtensorMap mO2, Args p) {
   constexpr bool WIDE = BN == 512;            // single accumulator handed over in two halves
@@ -493,6 +509,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
   static_assert(EPI != EPI_ROUTER_ST || (BN <= 128 && !PAIR), "staged router: up to 128 experts");
   // every epilogue except the plain router's writes through shared memory and TMA stores
   constexpr bool STAGED = EPI != EPI_ROUTER;
+  constexpr bool TWO = EPI == EPI_WGRAD;
+  static_assert(!TWO || (PAIR && B_SPLIT && !K_SPLIT), "weight gradients: pair tiles");
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -530,15 +548,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
   if (warp == 0 && lane == 0) {
     prefetch_map(&mA0);
     prefetch_map(&mB0);
-    if (K_SPLIT) prefetch_map(&mA1);
+    if (K_SPLIT || TWO) prefetch_map(&mA1);
     if (K_SPLIT || B_SPLIT) prefetch_map(&mB1);
+    if (TWO) prefetch_map(&mB2);
   }
   if (STAGED && warp >= 2 && lane == 0) {
     prefetch_map(&mO0);
-    if (EPI == EPI_SWIGLU_FWD || EPI == EPI_SWIGLU_BWD || EPI == EPI_STORE_F32_SPLIT ||
-        EPI == EPI_ROUTER_ST)
+    if (EPI == EPI_SWIGLU_FWD || EPI == EPI_SWIGLU_BWD || TWO || EPI == EPI_ROUTER_ST)
       prefetch_map(&mO1);
-    if (EPI == EPI_SWIGLU_FWD) prefetch_map(&mO2);
+    if (EPI == EPI_SWIGLU_FWD || TWO) prefetch_map(&mO2);
   }
   if (warp == 1) {
     if constexpr (PAIR) tmem_alloc_pair(tmem_holder, TCOLS);
@@ -552,7 +570,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
   pdl_begin(p.in0, p.in1, p.bias, p.vm_tiles, p.vm_count, p.gate);
 
   const int tiles_per_b = p.m_tiles * p.n_tiles;
-  const int total = VARM == 1 ? __ldg(p.vm_tiles + p.vm_E) * p.n_tiles : p.batch * tiles_per_b;
+  const int total = VARM == 1 ? __ldg(p.vm_tiles + p.vm_E) * p.n_tiles
+                              : p.batch * (tiles_per_b + (TWO ? p.m_tiles2 * p.n_tiles2 : 0));
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -561,7 +580,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
       uint32_t ph = 0;
       bool ok = true;
       for (int tile = cid; tile < total && ok; tile += nwalk) {
-        const Tile T = tile_at<VARM, TM>(p, tile, tiles_per_b, rank);
+        const Tile T = tile_at<VARM, TM, TWO>(p, tile, tiles_per_b, rank);
         if (VARM == 3 && T.valid <= 0) continue;
         const int nt = T.nt;
         const int m0 = T.row0;
@@ -580,7 +599,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
             load_b(dst, m, c0, c1, bb);
           };
           const bool second = K_SPLIT && kb >= p.k_blocks0;
-          const CUtensorMap* mA = second ? &mA1 : &mA0;
+          const bool p1 = TWO && T.prob;           // the second problem: A1 and B2, not split
+          const CUtensorMap* mA = second || p1 ? &mA1 : &mA0;
           const CUtensorMap* mB = second ? &mB1 : &mB0;
           const int k0 = (second ? kb - p.k_blocks0 : kb) * BK + T.krow0;
           uint8_t* a_dst = sA + s * A_BYTES;
@@ -594,12 +614,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
           if constexpr (PAIR) {
             // this CTA's half of each segment's B columns: for split tiles the gate (rank 0)
             // or up half
-            const CUtensorMap* mb = B_SPLIT ? (rank ? &mB1 : &mB0) : mB;
+            const CUtensorMap* mb = p1 ? &mB2 : B_SPLIT ? (rank ? &mB1 : &mB0) : mB;
 #pragma unroll
             for (int h = 0; h < NH; ++h) {
               uint8_t* bh = b_dst + h * (B_BYTES / NH);
-              const int n0 = B_SPLIT ? nt * (BN / 2) + h * (SEGW / 2)
-                                     : nt * BN + h * SEGW + (int)rank * (BNL / NH);
+              const int n0 = B_SPLIT && !p1 ? nt * (BN / 2) + h * (SEGW / 2)
+                                            : nt * BN + h * SEGW + (int)rank * (BNL / NH);
               if (!B_MN) {
                 load(bh, mb, k0, n0);
               } else {
@@ -667,7 +687,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
         else mma_commit(bar);
       };
       for (int tile = cid; tile < total && ok; tile += nwalk, ++it) {
-        const Tile T0 = tile_at<VARM, TM>(p, tile, tiles_per_b, 0);
+        const Tile T0 = tile_at<VARM, TM, TWO>(p, tile, tiles_per_b, 0);
         if (VARM == 3 && T0.valid <= 0) { --it; continue; }
         const int kbl = T0.kbl;
         if constexpr (!WIDE) {
@@ -766,7 +786,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
       asm volatile("bar.sync 1, %0;" ::"n"(32 * EPW) : "memory");
     }
     for (int tile = cid; tile < total && !stop; tile += nwalk, ++it) {
-      const Tile T = tile_at<VARM, TM>(p, tile, tiles_per_b, rank);
+      const Tile T = tile_at<VARM, TM, TWO>(p, tile, tiles_per_b, rank);
       if (VARM == 3 && T.valid <= 0) { --it; continue; }
       const int nt = T.nt;
       const int gm = T.row0 + r;
@@ -881,6 +901,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
         const int cb = h * SEGW;                   // first tile column of the segment
         constexpr int NC32 = SEGW / 32 / NPART;    // 32-column chunks per warp
         const int c32 = part * NC32;
+        // weight gradients: a warp's chunks are one half of the segment's columns, which all go to
+        // one output from column wn on
+        static_assert(!TWO || NPART == 2, "one column half per warp of a lane quarter");
+        const CUtensorMap* wm = TWO && T.prob ? &mO2 : part ? &mO1 : &mO0;
+        const int wn = TWO && T.prob ? nt * BN + cb + part * (SEGW / 2) : nt * (BN / 2) + cb / 2;
+        const int wend = !st_any ? 0 : TWO && T.prob ? p.N2 : p.N;
         if constexpr (EPI == EPI_SWIGLU_BWD) {
           // Both tile forms, segment by segment (columns cb.. of the tile). A and B of the next
           // chunk are requested before the current one is computed (not with variable rows,
@@ -985,7 +1011,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
               const int n = nt * BN + cb + (c32 + i) * 32;
               if (st_any && n < p.N) put_bf16w(&mO0, n, pk[i]);
             }
-          } else if constexpr (EPI == EPI_STORE_F32 || EPI == EPI_STORE_F32_SPLIT) {
+          } else if constexpr (EPI == EPI_WGRAD) {
             uint32_t raw[NC32][32];
 #pragma unroll
             for (int i = 0; i < NC32; ++i) tmem_ld32(tacc + (c32 + i) * 32, raw[i]);
@@ -993,19 +1019,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
             release(a);
 #pragma unroll
             for (int i = 0; i < NC32; ++i) {
-              const int c = c32 + i;
               if (no_k) {
 #pragma unroll
                 for (int j = 0; j < 32; ++j) raw[i][j] = 0u;
               }
-              if constexpr (EPI == EPI_STORE_F32) {
-                const int n = nt * BN + cb + c * 32;
-                if (st_any && n < p.N) put_f32w(&mO0, n, raw[i]);
-              } else {
-                const int half = c >= SEGW / 64;
-                const int n = nt * (BN / 2) + cb / 2 + (c % (SEGW / 64)) * 32;
-                if (st_any && n < p.N) put_f32w(half ? &mO1 : &mO0, n, raw[i]);
-              }
+              if (wn + i * 32 < wend) put_f32w(wm, wn + i * 32, raw[i]);
             }
           } else if constexpr (EPI == EPI_SWIGLU_FWD) {
             // column pairs (gate chunk, up chunk): a pair's A, B, U are packed while the next
@@ -1046,7 +1064,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
             }
             store_pair(part * NC64 + NC64 - 1);
           }
-        } else if constexpr (EPI == EPI_STORE_BF16 || EPI == EPI_STORE_F32) {
+        } else if constexpr (EPI == EPI_STORE_BF16) {
 #pragma unroll 1
           for (int c = c32; c < c32 + NC32; ++c) {
             tmem_ld32(tacc + c * 32, v);
@@ -1055,8 +1073,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
             if (st_any && n < p.N) {
 #pragma unroll
               for (int i = 0; i < 32; ++i) f[i] = no_k ? 0.f : f32(v[i]);
-              if constexpr (EPI == EPI_STORE_BF16) put_bf16(&mO0, n, f);
-              else put_f32(&mO0, n, f);
+              put_bf16(&mO0, n, f);
             }
           }
         } else if constexpr (EPI == EPI_STORE_F32_SUM) {
@@ -1074,17 +1091,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
               put_f32(&mO0, n, f);
             }
           }
-        } else if constexpr (EPI == EPI_STORE_F32_SPLIT) {
+        } else if constexpr (EPI == EPI_WGRAD) {
 #pragma unroll 1
-          for (int c = c32; c < c32 + NC32; ++c) {
-            tmem_ld32(tacc + c * 32, v);
+          for (int i = 0; i < NC32; ++i) {
+            tmem_ld32(tacc + (c32 + i) * 32, v);
             tmem_wait_ld();
-            const int half = c >= SEGW / 64;
-            const int n = nt * (BN / 2) + cb / 2 + (c % (SEGW / 64)) * 32;
-            if (st_any && n < p.N) {
+            if (wn + i * 32 < wend) {
 #pragma unroll
-              for (int i = 0; i < 32; ++i) f[i] = no_k ? 0.f : f32(v[i]);
-              put_f32(half ? &mO1 : &mO0, n, f);
+              for (int j = 0; j < 32; ++j) f[j] = no_k ? 0.f : f32(v[j]);
+              put_f32(wm, wn + i * 32, f);
             }
           }
         } else if constexpr (EPI == EPI_SWIGLU_FWD) {
@@ -1366,7 +1381,7 @@ template <int BN, bool A_MN, bool B_MN, bool B_SPLIT, bool K_SPLIT, int EPI, int
           int EPW = 8, bool PAIR = false, int VARM = 0>
 cudaError_t launch(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b0,
                    const CUtensorMap& b1, const CUtensorMap& o0, const CUtensorMap& o1,
-                   const CUtensorMap& o2, Args p, LaunchStream st) {
+                   const CUtensorMap& o2, Args p, LaunchStream st, const CUtensorMap* b2 = nullptr) {
   auto kern = tc_gemm_kernel<BN, A_MN, B_MN, B_SPLIT, K_SPLIT, EPI, STAGES, EPW, PAIR, VARM>;
   constexpr uint32_t smem = smem_bytes<BN, STAGES, PAIR, EPW, EPI>();
   static_assert(smem <= 232448, "dynamic shared memory above the 227 KB per-block limit");
@@ -1395,7 +1410,10 @@ cudaError_t launch(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorM
     attr = true;
   }
   // variable rows: p.M carries an upper bound of the padded rows, so `total` bounds the tiles
-  if (PAIR) p.m_tiles = (p.M + 2 * BM - 1) / (2 * BM);
+  if (PAIR) {
+    p.m_tiles = (p.M + 2 * BM - 1) / (2 * BM);
+    p.m_tiles2 = (p.M2 + 2 * BM - 1) / (2 * BM);
+  }
   if constexpr (VARM == 3) {
     // one CTA per SM (at most one per 32-row unit), each with the tiles of its row block
     static_assert(!PAIR, "row split: single-CTA tiles");
@@ -1406,13 +1424,14 @@ cudaError_t launch(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorM
     p.batch = 1;
     p.n_tiles = 1;
     p.m_tiles = g * (int)((max_rows + BM - 1) / BM);
-    return launch_kernel(kern, g, threads, smem, st, 1, a0, a1, b0, b1, o0, o1, o2, p);
+    return launch_kernel(kern, g, threads, smem, st, 1, a0, a1, b0, b1, b1, o0, o1, o2, p);
   }
-  const int total = p.batch * p.m_tiles * p.n_tiles;
+  const int total = p.batch * (p.m_tiles * p.n_tiles + p.m_tiles2 * p.n_tiles2);
   if (total == 0 || (VARM != 2 && p.k_blocks == 0)) return cudaSuccess;
   const int walkers = PAIR ? max_clusters : sm_count();
   const int grid = (PAIR ? 2 : 1) * (total < walkers ? total : walkers);
-  return launch_kernel(kern, grid, threads, smem, st, PAIR ? 2 : 1, a0, a1, b0, b1, o0, o1, o2, p);
+  return launch_kernel(kern, grid, threads, smem, st, PAIR ? 2 : 1, a0, a1, b0, b1, b2 ? *b2 : b1, o0,
+                       o1, o2, p);
 }
 
 Args base_args(int batch, int M, int N, int K, int BN_tile, int* status) {
@@ -1692,77 +1711,70 @@ cudaError_t tc_expert_dgrad_h(const void* dA, const void* dB, const void* Wg, co
                                                                      p, vr, st);
 }
 
+// [dWg | dWu][e] [d][F] = H[e]^T . [dA | dB][e] and dWd[e] [F][d] = U[e]^T . dO[e] (A[m][k=t] = H[t][m]
+// and U[t][m], MN-major). Up to 16 waves of tiles they are one tile list, so a launch, its ramp
+// and a partly empty last wave fall away: small ragged step 83 -> 76 us, 4096 tokens with 32
+// experts of d_ff 512 252 -> 246 us, and the shared experts' d_ff x d gradient needs no split over
+// K and no sum of its halves.
 cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const void* dA,
                             const void* dB, float* dWg, float* dWu, float* dWd, int E, int M,
-                            int d, int F, int* status, LaunchStream st, const VarRows* vr,
-                            int tiles) {
+                            int d, int F, int* status, LaunchStream st, int* launches,
+                            const VarRows* vr, int tiles) {
   // Variable rows: the K loop of expert e runs over its own padded region (count rows,
   // rounded up to the 64-row k-step, the rest of which is zero in both operands).
-  // K rows per expert (variable rows: on average)
-  const int rows = vr ? vr->P / (E > 0 ? E : 1) : M;
-  auto wg_args = [&](int Mo, int No, int BNt) {
-    Args p = base_args(E, Mo, No, vr ? vr->P : M, BNt, status);
+  CUtensorMap ma0, ma1, mb0, mb1, mb2, mo0, mo1, mo2;
+  TC_TRY(act_map(&ma0, H, d, E, M, vr, 64));
+  TC_TRY(act_map(&ma1, U, F, E, M, vr, 64));
+  TC_TRY(act_map(&mb0, dA, F, E, M, vr, 64));
+  TC_TRY(act_map(&mb1, dB, F, E, M, vr, 64));
+  TC_TRY(act_map(&mb2, dO, d, E, M, vr, 64));
+  TC_TRY(make_out_map(&mo0, dWg, true, F, d, E));
+  TC_TRY(make_out_map(&mo1, dWu, true, F, d, E));
+  TC_TRY(make_out_map(&mo2, dWd, true, d, F, E));
+  // which: bit 0 the gate/up gradients, bit 1 the down gradient
+  auto go = [&](int which, bool wide) -> cudaError_t {
+    Args p = base_args(E, which & 1 ? d : 0, F, vr ? vr->P : M, wide ? 256 : 128, status);
     if (vr) {
       p.vm_tiles = vr->tiles;
       p.vm_count = vr->count;
       p.vm_E = E;
     }
-    return p;
+    p.M2 = which & 2 ? F : 0;
+    p.N2 = d;
+    p.n_tiles2 = (d + (wide ? 511 : 255)) / (wide ? 512 : 256);
+    ++*launches;
+    if (wide && vr)
+      return launch<512, true, true, true, false, EPI_WGRAD, kWideStages, 8, true, 2>(
+          ma0, ma1, mb0, mb1, mo0, mo1, mo2, p, st, &mb2);
+    if (wide)
+      return launch<512, true, true, true, false, EPI_WGRAD, kWideStages, 8, true>(
+          ma0, ma1, mb0, mb1, mo0, mo1, mo2, p, st, &mb2);
+    if (vr)
+      return launch<256, true, true, true, false, EPI_WGRAD, 6, 8, true, 2>(
+          ma0, ma1, mb0, mb1, mo0, mo1, mo2, p, st, &mb2);
+    return launch<256, true, true, true, false, EPI_WGRAD, 6, 8, true>(ma0, ma1, mb0, mb1, mo0, mo1,
+                                                                       mo2, p, st, &mb2);
   };
-  if (dWd) {
-    // dWd[e] [F][d] = U[e]^T . dO[e]: A[m=f][k=t] = U[t][f] (MN-major), B[k=t][n=i] = dO[t][i]
-    CUtensorMap ma, mb, mo;
-    TC_TRY(act_map(&ma, U, F, E, M, vr, 64));
-    TC_TRY(act_map(&mb, dO, d, E, M, vr, 64));
-    TC_TRY(make_out_map(&mo, dWd, true, d, F, E));
-    const bool wide = wide_cols(tiles, d, rows);
-    Args p = wg_args(F, d, wide ? 512 : 256);
-    p.out0 = dWd;
-    p.ld = d;
-    p.bstride = (int64_t)F * d;
-    constexpr int EP = EPI_STORE_F32, WS = kWideStages;
-    if (wide && vr)
-      TC_TRY((launch<512, true, true, false, false, EP, WS, 8, true, 2>(ma, ma, mb, mb, mo, mo, mo, p,
-                                                                      st)));
-    else if (wide)
-      TC_TRY((launch<512, true, true, false, false, EP, WS, 8, true>(ma, ma, mb, mb, mo, mo, mo, p,
-                                                                   st)));
-    else if (vr)
-      TC_TRY((launch<256, true, true, false, false, EP, 6, 8, true, 2>(ma, ma, mb, mb, mo, mo, mo, p,
-                                                                     st)));
-    else
-      TC_TRY((launch<256, true, true, false, false, EP, 6, 8, true>(ma, ma, mb, mb, mo, mo, mo, p,
-                                                                  st)));
+  // K rows per expert (variable rows: on average)
+  const int rows = vr ? vr->P / (E > 0 ? E : 1) : M;
+  const bool w0 = wide_cols(tiles, 2 * F, rows), w1 = wide_cols(tiles, d, rows);
+  const int pairs = sm_count() / 2 > 0 ? sm_count() / 2 : 1;
+  const int64_t mt = (d + 255) / 256, mt2 = (F + 255) / 256;   // row tiles of the two problems
+  const int64_t narrow = E * (mt * ((F + 127) / 128) + mt2 * ((d + 255) / 256));
+  // Many tiles: two launches, down first (one list of both cost the 32768-token step of d 2048
+  // 1.6%, 7340 -> 7460 us). Two as well where only one problem has columns for wide tiles.
+  if (narrow > 16 * (int64_t)pairs || w0 != w1) {
+    TC_TRY(go(2, w1));
+    return go(1, w0);
   }
-  if (dWg) {
-    // [dWg | dWu][e] [d][F] = H[e]^T . [dA | dB][e]
-    CUtensorMap ma, mb0, mb1, mo0, mo1;
-    TC_TRY(act_map(&ma, H, d, E, M, vr, 64));
-    TC_TRY(act_map(&mb0, dA, F, E, M, vr, 64));
-    TC_TRY(act_map(&mb1, dB, F, E, M, vr, 64));
-    TC_TRY(make_out_map(&mo0, dWg, true, F, d, E));
-    TC_TRY(make_out_map(&mo1, dWu, true, F, d, E));
-    const bool wide = wide_cols(tiles, 2 * F, rows);
-    Args p = wg_args(d, F, wide ? 256 : 128);
-    p.out0 = dWg;
-    p.out1 = dWu;
-    p.ld = F;
-    p.bstride = (int64_t)d * F;
-    constexpr int EP = EPI_STORE_F32_SPLIT, WS = kWideStages;
-    if (wide && vr)
-      TC_TRY((launch<512, true, true, true, false, EP, WS, 8, true, 2>(ma, ma, mb0, mb1, mo0, mo1, mo1,
-                                                                     p, st)));
-    else if (wide)
-      TC_TRY((launch<512, true, true, true, false, EP, WS, 8, true>(ma, ma, mb0, mb1, mo0, mo1, mo1, p,
-                                                                  st)));
-    else if (vr)
-      TC_TRY((launch<256, true, true, true, false, EP, 6, 8, true, 2>(ma, ma, mb0, mb1, mo0, mo1, mo1,
-                                                                    p, st)));
-    else
-      TC_TRY((launch<256, true, true, true, false, EP, 6, 8, true>(ma, ma, mb0, mb1, mo0, mo1, mo1, p,
-                                                                 st)));
+  bool wide = w0;
+  if (wide && tiles == 0) {
+    // half as wide tiles where their last wave leaves less idle; one takes more than half of a
+    // wide one's time (its MMAs wait longer for operands: 7% on the large shapes)
+    const int64_t nw = E * (mt * (F / 256) + mt2 * (d / 512));
+    wide = 2.0 * ((nw + pairs - 1) / pairs) <= 1.07 * ((narrow + pairs - 1) / pairs);
   }
-  return cudaSuccess;
+  return go(3, wide);
 }
 
 cudaError_t tc_router_dgrad(const void* dZb, const void* Wr, void* dXr, int N, int d, int E,
