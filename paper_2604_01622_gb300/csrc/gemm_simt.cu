@@ -8,13 +8,13 @@
 // a bit of the result.
 //
 // What bounds it: the FMA pipes. With 8 x 8 outputs per thread they are busy 69% of an SM's
-// active cycles (ncu; the most frequent stall is the pipe itself), and 40-46 TFLOP/s come out of
+// active cycles (ncu; the most frequent stall is the pipe itself), and 35-47 TFLOP/s come out of
 // the 75 that the pipes allow, the rest lost to the last wave and the edge tiles. The scalar
 // 4 x 4 kernel with 4-byte loads before it ran 22 TFLOP/s on the same shapes (16 experts of 1000
 // rows, d 500, d_ff 364). The row gather of H = X[idx], the SwiGLU and its derivative, and the
 // second product of dH are part of the same launches, so no intermediate is written that a
-// later kernel only reads back: that layer's step 2820 -> 1424 us, a 256-token layer's (24
-// kernels, now 15) 195 -> 89-96 us.
+// later kernel only reads back: that layer's step 2820 -> 1387 us, a 256-token layer's (24
+// kernels, now 15) 195 -> 64-69 us, most of it host time by now.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -335,27 +335,34 @@ cudaError_t go(const SimtGemmArgs& a, LaunchStream st) {
 
 // Tile shape: the one whose busiest SM has the least work, tiles per SM (rounded up) times the
 // tile's outputs times its measured cost per output against 128 x 128 (the shapes below, on
-// 16 problems of M 1000 and M 96, N 364 and 500, K 364 to 1000: 64 x 128 1.02-1.12, 64 x 64
-// 1.14, 32 x 32 2.1-2.4; 16 x 8 outputs per thread were slower in every shape). It takes 64 x 128
-// where 128 x 128 leaves a nearly empty last wave (1000 x 500 x 364: 129 against 141 us) and
-// the small tiles for a few rows per expert (96 x 500 x 364: 27 against 43 us).
+// 16 problems of M 1000 and M 96, N 364 and 500, K 364 to 1000: half tiles 1.0-1.12, 64 x 64
+// 1.14, 32 x 32 2.1-2.4; 16 x 8 outputs per thread were slower in every shape, and so were A
+// pairs kept in shared memory and fragments loaded a step ahead). Half tiles where 128 x 128
+// leaves a nearly empty last wave, tall ones where A's rows are contiguous (gate/up 260 against
+// 279 us, down 123 against 140, dH 254 against 281), wide ones for the weight gradients (dWd 160
+// against 193) and dU; the small tiles for a few rows per expert (96 x 500 x 364: 27 against 43).
 template <bool A_K, bool B_K, int EPI>
 cudaError_t pick(const SimtGemmArgs& a, LaunchStream st) {
   constexpr int half = (EPI == SIMT_DUAL || EPI == SIMT_SWIGLU_FWD) ? 2 : 1;
+  constexpr bool TALL = A_K && EPI != SIMT_SWIGLU_BWD;
   const int64_t sms = simt_sms();
   auto cost = [&](int bm, int bn, double per_output) {
     const int64_t tiles = (int64_t)((a.M + bm - 1) / bm) * (((int64_t)a.N * half + bn - 1) / bn) *
                           a.batch * a.splits;
     return (double)((tiles + sms - 1) / sms) * bm * bn * per_output;
   };
-  const double c[4] = {cost(128, 128, 1.0), cost(64, 128, 1.06), cost(64, 64, 1.14),
-                       cost(32, 32, 2.2)};
+  const double c[4] = {cost(128, 128, 1.0), TALL ? cost(128, 64, 1.02) : cost(64, 128, 1.06),
+                       cost(64, 64, 1.14), cost(32, 32, 2.2)};
   int best = 0;
   for (int i = 1; i < 4; ++i)
     if (c[i] < c[best]) best = i;
   switch (best) {
     case 0: return go<128, 128, 16, 8, 8, 2, A_K, B_K, EPI>(a, st);
-    case 1: return go<64, 128, 16, 8, 8, 4, A_K, B_K, EPI>(a, st);
+    case 1:
+      if constexpr (TALL)
+        return go<128, 64, 16, 8, 8, EPI == SIMT_SWIGLU_FWD ? 3 : 4, A_K, B_K, EPI>(a, st);
+      else
+        return go<64, 128, 16, 8, 8, 4, A_K, B_K, EPI>(a, st);
     case 2: return go<64, 64, 16, 8, 4, 4, A_K, B_K, EPI>(a, st);
   }
   return go<32, 32, 32, 2, 4, 4, A_K, B_K, EPI>(a, st);

@@ -1,6 +1,6 @@
 """The fp32 path's GEMMs at the sizes where a tile shape or a load form changes, against the
 oracle (relative max-norm 1e-4, the fp32 parity bound of the other tests): one shape per tile
-(128 x 128, 64 x 128, 64 x 64, 32 x 32), each with ragged row, column and k edges, an expert
+(128 x 128, 128 x 64 and 64 x 128, 64 x 64, 32 x 32), each with ragged row, column and k edges, an expert
 count that is not a multiple of 4 (scalar loads and stores in the router products), more than 64
 experts (several column tiles of the router kernel) and fewer than 64 tokens (one split of
 X^T dZ)."""
@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("L,d,E,d_ff,k", [
     (3000, 260, 24, 132, 700),    # 128 x 128: a 60-row tail, 4 columns past a tile
-    (2000, 260, 16, 132, 260),    # 64 x 128
+    (2000, 260, 16, 132, 260),    # half tiles
     (900, 132, 14, 132, 130),     # 64 x 64, 14 experts
     (130, 68, 6, 36, 33),         # 32 x 32: one row past a tile
     (1000, 36, 70, 20, 40),       # 70 experts: two column tiles of the router
