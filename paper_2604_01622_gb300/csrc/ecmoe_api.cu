@@ -155,7 +155,7 @@ void layout(ec_ctx* c) {
   c->o_koff = take((G + 1) * 4);
   c->o_ST = take(E * N * 4);
   c->o_S = take(N * E * 4);
-  c->o_idx = take(P * 4);
+  c->o_idx = take(c->tc_k ? 0 : P * 4);
   c->o_gate = take(P * 4);
   c->o_slot = take(N * E * 4);
   c->o_H = take(use_tc(c) ? P * d * es : 0);   // fp32: rows are gathered from X by the GEMMs
@@ -631,14 +631,6 @@ ec_status run_backward(ec_ctx* c, const void* dY, void* dX, float* dWr, float* d
 }
 
 // ---------------------------------------------------------------- token choice (bf16)
-// Token-major copy of X (or dY) rows into the padded expert regions, padding rows zeroed.
-cudaError_t tc_scatter(const bf16* X, const int* slot, const int* count, const int* tiles, bf16* H,
-                       int N, int E, int d, LaunchStream st) {
-  cudaError_t e = launch_scatter_rows<bf16>(X, slot, H, N, E, 0, d, st);
-  if (e != cudaSuccess) return e;
-  return launch_zero_pad_rows<bf16>(count, tiles, H, E, d, st);
-}
-
 // Sec. 2.2 "Token-choice": router -> per-token top-k with renormalised gates and the
 // per-expert cap -> gather into padded expert regions -> variable-row expert GEMMs ->
 // gated combine through the token->row map.
@@ -650,7 +642,6 @@ ec_status run_tc_forward(ec_ctx* c, const void* X, const void* Wr, const float* 
   float* S = at<float>(c, c->o_S);
   int* count = at<int>(c, c->o_count);
   int* tiles = at<int>(c, c->o_tiles);
-  int* row_token = at<int>(c, c->o_idx);
   float* row_gate = at<float>(c, c->o_gate);
   int* slot = at<int>(c, c->o_slot);
   const bf16* Xt = static_cast<const bf16*>(X);
@@ -661,13 +652,12 @@ ec_status run_tc_forward(ec_ctx* c, const void* X, const void* Wr, const float* 
   EC_KERNEL("router_gemm_softmax", router_needs_pad(E) ? 2 : 1,
             tc_router_softmax(X, Wr, at<void>(c, c->o_wrpad), br, S, at<float>(c, c->o_ST),
                               nullptr, N, d, E, status, st));
-  EC_KERNEL("tc_route", 5,
+  EC_KERNEL("tc_route", 4,
             launch_tc_route(S, N, E, k, c->tc_cap, at<int>(c, c->o_choice),
-                            at<float>(c, c->o_tgate), at<float>(c, c->o_Zs), count, tiles,
-                            row_token, row_gate, slot, at<int>(c, c->o_kept),
-                            at<int>(c, c->o_tcscr), st));
+                            at<float>(c, c->o_tgate), at<float>(c, c->o_Zs), count, tiles, row_gate,
+                            slot, at<int>(c, c->o_kept), at<int>(c, c->o_tcscr), st));
   const VarRows vr{tiles, count, (int)c->P_tc};
-  EC_KERNEL("gather", 2, tc_scatter(Xt, slot, count, tiles, H, N, E, d, st));
+  EC_KERNEL("gather", 1, launch_scatter_rows<bf16>(Xt, slot, H, N, E, 0, d, st, count, tiles));
   EC_KERNEL("gemm_gate_up_swiglu", 1,
             tc_expert_up(H, Wg, Wu, at<bf16>(c, c->o_A), at<bf16>(c, c->o_B), U, E, 0, d, F,
                          status, st, &vr, row_gate, c->tiles));
@@ -702,7 +692,8 @@ ec_status run_tc_backward(ec_ctx* c, const void* dY, void* dX, float* dWr, float
   float* row_dgate = at<float>(c, c->o_dgate);
   const int* slot = at<int>(c, c->o_slot);
   // dO = dY rows ungated; the dU epilogue applies the row gates and forms their gradients
-  EC_KERNEL("gather_dy", 2, tc_scatter(dYt, slot, count, vr.tiles, dO, N, E, d, st));
+  EC_KERNEL("gather_dy", 1,
+            launch_scatter_rows<bf16>(dYt, slot, dO, N, E, 0, d, st, count, vr.tiles));
   EC_KERNEL("gemm_dgrad_up_swiglu", 1,
             tc_expert_dgrad_up(dO, c->Wd, at<bf16>(c, c->o_A), at<bf16>(c, c->o_B), dA, dB, E, 0,
                                d, F, status, st, &vr, at<float>(c, c->o_gate), row_dgate,
@@ -717,12 +708,10 @@ ec_status run_tc_backward(ec_ctx* c, const void* dY, void* dX, float* dWr, float
   float* dZ = at<float>(c, c->o_dZ);
   bf16* dZb = at<bf16>(c, c->o_dZb);
   bf16* dXr = at<bf16>(c, c->o_dXr);
-  float* dgsum = at<float>(c, c->o_dgsum);
-  EC_KERNEL("dgate_reduce", 1, launch_reduce_splits(row_dgate, dgsum, c->P_tc, c->dg_parts, st));
   EC_KERNEL("softmax_bwd", 1,
             launch_tc_softmax_bwd(at<float>(c, c->o_S), at<int>(c, c->o_choice),
-                                  at<float>(c, c->o_tgate), at<float>(c, c->o_Zs), slot, dgsum, dZ,
-                                  dZb, N, E, c->Ep, k, st));
+                                  at<float>(c, c->o_tgate), at<float>(c, c->o_Zs), slot, row_dgate,
+                                  c->dg_parts, c->P_tc, dZ, dZb, N, E, c->Ep, k, st));
   EC_KERNEL("router_dgrad_gemm", 1, tc_router_dgrad(dZb, router_b(c), dXr, N, d, E, status, st));
   EC_KERNEL("dx_combine", 1,
             launch_dx_combine<bf16>(dH, slot, dXr, c->residual ? dYt : nullptr, nullptr,

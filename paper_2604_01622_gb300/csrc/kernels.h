@@ -36,38 +36,32 @@ cudaError_t launch_set_capacity(const int* k_new, const int* group_off, int G, i
                                 int* k_off, int* status, LaunchStream st);
 
 // ---------------------------------------------------------------- token-choice routing
-// Row top-k of S [N][E] (k <= 32, E <= 512), per-expert counts capped at cap (cap < 0:
-// dropless), padded expert regions (tiles[e] in 256-row blocks), row->token map (-1 in
-// padding), row gates, slot map [N][E] (absolute row or -1) and kept flags [N][k].
 // Token-choice routing of the scores S [N][E] (k <= 32, E <= 256; cap < 0: no cap):
 // choice/tgate/kept [N][k] (experts best first, normalised gates, kept flags), Z [N] (sum of
 // the k chosen scores), count [E+1] (kept rows per expert; count[E] = padded rows in use),
-// tiles [E+1] (cumulative 256-row blocks), row_token/row_gate [P] per padded row (-1 / 0 in
-// padding), slot [N][E] absolute padded row of each kept pair, else -1.
-// scratch: tc_route_scratch_ints(N, E) ints. Five kernels (and a memset of slot).
+// tiles [E+1] (cumulative 256-row blocks), row_gate [P] of each kept pair's row (padding rows
+// untouched), slot [N][E] absolute padded row of each kept pair, else -1.
+// scratch: tc_route_scratch_ints(N, E) ints. Four kernels.
 cudaError_t launch_tc_route(const float* S, int N, int E, int k, int cap, int* choice,
-                            float* tgate, float* Z, int* count, int* tiles, int* row_token,
-                            float* row_gate, int* slot, int* kept, int* scratch,
-                            LaunchStream st);
+                            float* tgate, float* Z, int* count, int* tiles, float* row_gate,
+                            int* slot, int* kept, int* scratch, LaunchStream st);
 int64_t tc_route_scratch_ints(int N, int E);
 // Router gradient of token choice: dZ [N][E] (and optionally the bf16 hi/lo planes
-// dZb [2][N][Ep]) from the per-row gate gradients row_dgate [P].
+// dZb [2][N][Ep]) from the per-row gate-gradient partials row_dgate [parts][P].
 cudaError_t launch_tc_softmax_bwd(const float* S, const int* choice, const float* tgate,
-                                  const float* Z, const int* slot, const float* row_dgate,
-                                  float* dZ, __nv_bfloat16* dZb, int N, int E, int Ep, int k,
-                                  LaunchStream st);
+                                  const float* Z, const int* slot, const float* row_dgate, int parts,
+                                  int64_t P, float* dZ, __nv_bfloat16* dZb, int N, int E, int Ep,
+                                  int k, LaunchStream st);
 
 // ---------------------------------------------------------------- data movement
 // Token-major form of the gather: for each token t, X row t is copied to row e*M + slot[t][e]
-// of H for every expert e with slot[t][e] >= 0 (M = 0: slot holds absolute rows).
+// of H for every expert e with slot[t][e] >= 0 (M = 0: slot holds absolute rows). With count [E]
+// and tiles [E+1] (in 256-row blocks, device arrays) the unused rows of the variable-row expert
+// regions are zeroed as well.
 template <typename T>
 cudaError_t launch_scatter_rows(const T* X, const int* slot, T* H, int N, int E, int M, int d,
-                                LaunchStream st);
-// Zeros the unused (padding) rows of variable-row expert regions (count [E], tiles [E+1] in
-// 256-row blocks, device arrays).
-template <typename T>
-cudaError_t launch_zero_pad_rows(const int* count, const int* tiles, T* H, int E, int d,
-                                 LaunchStream st);
+                                LaunchStream st, const int* count = nullptr,
+                                const int* tiles = nullptr);
 // Y_t = R_t + R2_t (each if given) + sum over the experts that chose t of gate * O row
 // (gate NULL: 1, for O rows already scaled by their gates).
 template <typename T>

@@ -134,10 +134,29 @@ cudaError_t launch_combine(const T* O, const float* gate, const int* slot, const
 // H[row] = X[t] for every (expert, row) that selected token t, one CTA per token: each X row
 // is read once (an expert-major gather, row by row of H, would read it once per selecting
 // expert, mostly from DRAM), and written to its rows in ascending expert order.
+//
+// Variable-row expert regions (count [E] and tiles [E+1] in 256-row blocks, device arrays): CTAs
+// from N on zero the padding rows count[e] .. 256 (tiles[e+1] - tiles[e]) - 1 of each region,
+// kPadCtas CTAs per expert.
+constexpr int kPadCtas = 8;
+
 template <typename T>
 __global__ void scatter_rows_kernel(const T* __restrict__ X, const int* __restrict__ slot,
+                                    const int* __restrict__ count, const int* __restrict__ tiles,
                                     T* __restrict__ H, int N, int E, int M, int d) {
-  pdl_begin(X, slot);
+  pdl_begin(X, slot, count, tiles);
+  if ((int)blockIdx.x >= N) {
+    const int e = ((int)blockIdx.x - N) / kPadCtas, part = ((int)blockIdx.x - N) % kPadCtas;
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int64_t end = (int64_t)tiles[e + 1] * 256;
+    const int units = d * (int)sizeof(T) / 16;
+    for (int64_t row = (int64_t)tiles[e] * 256 + count[e] + part * nw + (threadIdx.x >> 5); row < end;
+         row += kPadCtas * nw) {
+      uint4* dst = reinterpret_cast<uint4*>(H + row * d);
+      for (int v = lane; v < units; v += 32) dst[v] = make_uint4(0, 0, 0, 0);
+    }
+    return;
+  }
   extern __shared__ int sh[];
   int* s_e = sh;
   int* s_m = sh + E;
@@ -156,35 +175,11 @@ __global__ void scatter_rows_kernel(const T* __restrict__ X, const int* __restri
 
 template <typename T>
 cudaError_t launch_scatter_rows(const T* X, const int* slot, T* H, int N, int E, int M, int d,
-                                LaunchStream st) {
+                                LaunchStream st, const int* count, const int* tiles) {
   if (N == 0) return cudaSuccess;
   const size_t smem = (size_t)2 * E * sizeof(int);
-  return launch_kernel(scatter_rows_kernel<T>, N, 128, smem, st, 1, X, slot, H, N, E, M, d);
-}
-
-// Zero the padding rows of variable-row expert regions: rows count[e] .. 256*(tiles[e+1] -
-// tiles[e]) - 1 of expert e's region (one warp per possible padding row).
-template <typename T>
-__global__ void zero_pad_rows_kernel(const int* __restrict__ count, const int* __restrict__ tiles,
-                                     T* __restrict__ H, int E, int d) {
-  pdl_begin(count, tiles);
-  const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  const int e = (int)(w / 256);
-  if (e >= E) return;
-  const int64_t row = (int64_t)tiles[e] * 256 + count[e] + (w % 256);
-  if (row >= (int64_t)tiles[e + 1] * 256) return;
-  uint4* dst = reinterpret_cast<uint4*>(H + row * d);
-  const int nv = d * (int)sizeof(T) / 16;
-  for (int v = lane; v < nv; v += 32) dst[v] = make_uint4(0, 0, 0, 0);
-}
-
-template <typename T>
-cudaError_t launch_zero_pad_rows(const int* count, const int* tiles, T* H, int E, int d,
-                                 LaunchStream st) {
-  const int64_t warps = (int64_t)E * 256;
-  return launch_kernel(zero_pad_rows_kernel<T>, (unsigned)((warps + 7) / 8), 256, 0, st, 1, count,
-                       tiles, H, E, d);
+  return launch_kernel(scatter_rows_kernel<T>, N + (count ? E * kPadCtas : 0), 128, smem, st, 1, X,
+                       slot, count, tiles, H, N, E, M, d);
 }
 
 // ------------------------------------------------------------------ backward: dO = g dY_t, dgate = <dY_t, O>
@@ -725,9 +720,7 @@ ECMOE_INST(bf16)
 // the fp32 path gathers rows inside its GEMMs; the bf16 path takes the gate and its gradient
 // into the expert GEMMs' epilogues
 template cudaError_t launch_scatter_rows<bf16>(const bf16*, const int*, bf16*, int, int, int, int,
-                                               LaunchStream);
-template cudaError_t launch_zero_pad_rows<bf16>(const int*, const int*, bf16*, int, int,
-                                                LaunchStream);
+                                               LaunchStream, const int*, const int*);
 template cudaError_t launch_bwd_gather_scale<float>(const float*, const float*, const int*,
                                                     const float*, float*, float*, int64_t, int,
                                                     LaunchStream);

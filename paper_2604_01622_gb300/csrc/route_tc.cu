@@ -54,10 +54,10 @@ __device__ __forceinline__ uint32_t score_key(float v) {
 // One warp per token, lane l holding experts l, l+32, ... (E <= 256) in registers: k rounds
 // of a warp argmax (largest key by a max-reduction, then the lowest expert index holding
 // it by a min-reduction). Writes the choices best first, the normalised gates and their
-// sum Z (summed in choice order).
+// sum Z (summed in choice order), and sets the token's row of the slot map to -1.
 __global__ void tc_topk_rows_kernel(const float* __restrict__ S, int N, int E, int k,
                                     int* __restrict__ choice, float* __restrict__ tgate,
-                                    float* __restrict__ Z) {
+                                    float* __restrict__ Z, int* __restrict__ slot) {
   pdl_begin(S);
   constexpr int MAXC = 8;
   const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -71,6 +71,7 @@ __global__ void tc_topk_rows_kernel(const float* __restrict__ S, int N, int E, i
     const int e = lane + 32 * i;
     val[i] = e < E ? row[e] : 0.f;
     key[i] = e < E ? score_key(val[i]) : 0u;
+    if (e < E) slot[(size_t)t * E + e] = -1;
   }
   float sum = 0.f, my_v = 0.f;
   int my_e = 0;   // lane r keeps the r-th choice
@@ -265,70 +266,52 @@ __global__ void tc_block_scan_kernel(const int* __restrict__ hist, int nblk, int
   if (threadIdx.x == 0) total[e] = carry;
 }
 
-// One CTA (E <= blockDim): kept rows per expert count[e] = min(total, cap) (cap < 0: no cap),
-// padded regions tiles[e] (cumulative 256-row blocks, tiles[E] the total) and in count[E]
-// the padded rows in use.
-__global__ void tc_offsets_kernel(int E, int cap, const int* __restrict__ total,
-                                  int* __restrict__ count, int* __restrict__ tiles) {
-  pdl_begin(total);
-  __shared__ int s_warp[33];
-  const int e = threadIdx.x;
-  int c = e < E ? total[e] : 0;
+// One thread per (token, choice) pair: absolute position, keep/drop and the row of each kept
+// pair. Every CTA first makes the expert table from the totals (kept rows per expert
+// min(total, cap), cap < 0: no cap, and padded regions of whole 256-row blocks), a scan of at most
+// 256 counts that is cheaper than a launch of its own; the first CTA writes it out: count[e],
+// tiles[e] (cumulative blocks, tiles[E] their sum) and in count[E] the padded rows in use.
+__global__ void __launch_bounds__(kMaxE)
+tc_fill_kernel(const int* __restrict__ choice, const float* __restrict__ tgate, int N, int E, int k,
+               int cap, const int* __restrict__ boff, const int* __restrict__ total,
+               int* __restrict__ count, int* __restrict__ tiles, float* __restrict__ row_gate,
+               int* __restrict__ slot, int* __restrict__ kept) {
+  pdl_begin(choice, tgate, boff, total);
+  __shared__ int s_warp[33], s_count[kMaxE], s_row0[kMaxE];
+  const int ex = threadIdx.x;
+  int c = ex < E ? total[ex] : 0;
   if (cap >= 0 && c > cap) c = cap;
-  const int nb = (c + kPadRows - 1) / kPadRows;
   int all;
-  const int off = block_scan_excl(nb, s_warp, &all);
-  if (e < E) {
-    count[e] = c;
-    tiles[e] = off;
-  }
-  if (threadIdx.x == 0) {
-    tiles[E] = all;
-    count[E] = all * kPadRows;
-  }
-}
-
-// One thread per (token, choice) pair: absolute position, keep/drop, row maps; then one
-// thread per possible padding row of each expert: row_token -1, gate 0.
-__global__ void tc_fill_kernel(const int* __restrict__ choice, const float* __restrict__ tgate,
-                               int N, int E, int k, const int* __restrict__ boff,
-                               const int* __restrict__ count, const int* __restrict__ tiles,
-                               int* __restrict__ row_token, float* __restrict__ row_gate,
-                               int* __restrict__ slot, int* __restrict__ kept) {
-  pdl_begin(choice, tgate, boff, count, tiles);
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t NK = (int64_t)N * k;
-  if (j < NK) {
-    const int t = (int)(j / k);
-    const int e = choice[j];
-    int* sl = slot + (size_t)t * E + e;
-    const int pos = boff[(size_t)(t / kRankBlock) * E + e] + *sl;
-    const bool keep = pos < count[e];
-    kept[j] = keep;
-    if (keep) {
-      const int row = tiles[e] * kPadRows + pos;
-      *sl = row;
-      row_token[row] = t;
-      row_gate[row] = tgate[j];
-    } else {
-      *sl = -1;
+  const int off = block_scan_excl((c + kPadRows - 1) / kPadRows, s_warp, &all);
+  s_count[ex] = c;
+  s_row0[ex] = off * kPadRows;
+  if (blockIdx.x == 0) {
+    if (ex < E) {
+      count[ex] = c;
+      tiles[ex] = off;
     }
-    return;
+    if (ex == 0) {
+      tiles[E] = all;
+      count[E] = all * kPadRows;
+    }
   }
-  const int64_t q = j - NK;
-  const int e = (int)(q / kPadRows);
-  if (e >= E) return;
-  const int row = tiles[e] * kPadRows + count[e] + (int)(q % kPadRows);
-  if (row < tiles[e + 1] * kPadRows) {
-    row_token[row] = -1;
-    row_gate[row] = 0.f;
-  }
+  __syncthreads();
+  const int64_t j = (int64_t)blockIdx.x * kMaxE + threadIdx.x;
+  if (j >= (int64_t)N * k) return;
+  const int t = (int)(j / k);
+  const int e = choice[j];
+  int* sl = slot + (size_t)t * E + e;
+  const int pos = boff[(size_t)(t / kRankBlock) * E + e] + *sl;
+  const bool keep = pos < s_count[e];
+  kept[j] = keep;
+  const int row = keep ? s_row0[e] + pos : -1;
+  *sl = row;
+  if (keep) row_gate[row] = tgate[j];
 }
 
 cudaError_t launch_tc_route(const float* S, int N, int E, int k, int cap, int* choice,
-                            float* tgate, float* Z, int* count, int* tiles, int* row_token,
-                            float* row_gate, int* slot, int* kept, int* scratch,
-                            LaunchStream st) {
+                            float* tgate, float* Z, int* count, int* tiles, float* row_gate,
+                            int* slot, int* kept, int* scratch, LaunchStream st) {
   if (N == 0) return cudaSuccess;
   if (E > kMaxE || k > 32 || k > E) return cudaErrorInvalidValue;
   const int nblk = (N + kRankBlock - 1) / kRankBlock;
@@ -336,25 +319,20 @@ cudaError_t launch_tc_route(const float* S, int N, int E, int k, int cap, int* c
   int* boff = scratch + (size_t)nblk * E;       // [nblk][E]
   int* total = boff + (size_t)nblk * E;         // [E]
   cudaError_t err;
-  if (E % 4 == 0 && E <= kTopkFastE && k <= kTopkFastK) {
-    // four threads per token; the slot map's -1 rows are written there too
+  if (E % 4 == 0 && E <= kTopkFastE && k <= kTopkFastK)   // four threads per token
     err = launch_kernel(tc_topk_rows4_kernel, (unsigned)(((int64_t)N * 4 + 255) / 256), 256, 0, st, 1,
                         S, N, E, k, choice, tgate, Z, slot);
-  } else {
-    err = cudaMemsetAsync(slot, 0xFF, (size_t)N * E * sizeof(int), st);   // -1
-    if (err != cudaSuccess) return err;
-    err = launch_kernel(tc_topk_rows_kernel, (N + 7) / 8, 256, 0, st, 1, S, N, E, k, choice, tgate, Z);
-  }
+  else
+    err = launch_kernel(tc_topk_rows_kernel, (N + 7) / 8, 256, 0, st, 1, S, N, E, k, choice, tgate, Z,
+                        slot);
   if (err != cudaSuccess) return err;
   err = launch_kernel(tc_rank_kernel, nblk, kRankBlock, 0, st, 1, choice, N, E, k, slot, hist);
   if (err != cudaSuccess) return err;
   err = launch_kernel(tc_block_scan_kernel, E, 256, 0, st, 1, hist, nblk, E, boff, total);
   if (err != cudaSuccess) return err;
-  err = launch_kernel(tc_offsets_kernel, 1, kMaxE, 0, st, 1, E, cap, total, count, tiles);
-  if (err != cudaSuccess) return err;
-  const int64_t threads = (int64_t)N * k + (int64_t)E * kPadRows;
-  return launch_kernel(tc_fill_kernel, (unsigned)((threads + 255) / 256), 256, 0, st, 1, choice, tgate,
-                       N, E, k, boff, count, tiles, row_token, row_gate, slot, kept);
+  return launch_kernel(tc_fill_kernel, (unsigned)(((int64_t)N * k + kMaxE - 1) / kMaxE), kMaxE, 0, st,
+                       1, choice, tgate, N, E, k, cap, boff, total, count, tiles, row_gate, slot,
+                       kept);
 }
 
 // Scratch ints launch_tc_route needs for N tokens and E experts.
@@ -365,13 +343,14 @@ int64_t tc_route_scratch_ints(int N, int E) {
 
 // Gradient through the normalised gates and the softmax, one warp per token:
 // dS_tj = (dg_tj - sum_{j' kept} dg_tj' g_tj') / Z_t for the k chosen j (dg = 0 if dropped),
-// dZ = S * (dS - <dS, S>). dg comes from the per-row gate gradients through the slot map;
-// lane r < k holds the token's r-th choice.
+// dZ = S * (dS - <dS, S>). dg is the sum of the pair's gate-gradient partials [parts][P], in part
+// order, found through the slot map; lane r < k holds the token's r-th choice.
 __global__ void tc_softmax_bwd_kernel(const float* __restrict__ S, const int* __restrict__ choice,
                                       const float* __restrict__ tgate, const float* __restrict__ Z,
                                       const int* __restrict__ slot,
-                                      const float* __restrict__ row_dgate, float* __restrict__ dZ,
-                                      bf16* __restrict__ dZb, int N, int E, int Ep, int k) {
+                                      const float* __restrict__ row_dgate, int parts, int64_t P,
+                                      float* __restrict__ dZ, bf16* __restrict__ dZb, int N, int E,
+                                      int Ep, int k) {
   pdl_begin(S, choice, tgate, Z, slot, row_dgate);
   const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -381,7 +360,8 @@ __global__ void tc_softmax_bwd_kernel(const float* __restrict__ S, const int* __
   if (lane < k) {
     my_e = choice[(size_t)t * k + lane];
     const int row = slot[(size_t)t * E + my_e];
-    dg = row >= 0 ? row_dgate[row] : 0.f;
+    if (row >= 0)
+      for (int j = 0; j < parts; ++j) dg += row_dgate[(size_t)j * P + row];
     g = tgate[(size_t)t * k + lane];
     s_e = S[(size_t)t * E + my_e];
   }
@@ -409,13 +389,13 @@ __global__ void tc_softmax_bwd_kernel(const float* __restrict__ S, const int* __
 }
 
 cudaError_t launch_tc_softmax_bwd(const float* S, const int* choice, const float* tgate,
-                                  const float* Z, const int* slot, const float* row_dgate,
-                                  float* dZ, bf16* dZb, int N, int E, int Ep, int k,
+                                  const float* Z, const int* slot, const float* row_dgate, int parts,
+                                  int64_t P, float* dZ, bf16* dZb, int N, int E, int Ep, int k,
                                   LaunchStream st) {
   if (N == 0) return cudaSuccess;
   if (k > 32 || Ep % 32) return cudaErrorInvalidValue;
   return launch_kernel(tc_softmax_bwd_kernel, (N + 7) / 8, 256, 0, st, 1, S, choice, tgate, Z, slot,
-                       row_dgate, dZ, dZb, N, E, Ep, k);
+                       row_dgate, parts, P, dZ, dZb, N, E, Ep, k);
 }
 
 }  // namespace ecmoe
