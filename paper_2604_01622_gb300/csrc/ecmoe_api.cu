@@ -190,8 +190,9 @@ void layout(ec_ctx* c) {
     c->wr_splits = router_wgrad_splits((int)N, (int)d, c->Ep);
     c->o_part = take((size_t)c->wr_splits * d * c->Ep * 4);
   } else {
-    // one split per 64 tokens (at most 64): X^T dZ has only d*E outputs for the whole GPU
-    c->wr_splits = (int)std::max<size_t>(1, std::min<size_t>(64, N / 64));
+    // one split per 64 tokens (at most 64): X^T dZ has only d*E outputs for the whole GPU. Up to
+    // 256 tokens a single chain takes less than summing the splits in another launch.
+    c->wr_splits = N <= 256 ? 1 : (int)std::min<size_t>(64, N / 64);
     c->o_part = take((size_t)c->wr_splits * d * E * 4);
   }
   c->total = o;
@@ -456,14 +457,15 @@ ec_status ffn_backward(ec_ctx* c, const FfnNames& nm, const T* dO, const T* H, c
     SimtGemmArgs dh = sg(dA, fs, F, true, f32p(Wg), wgs, F, true, dH, hs, d, M, d, F, E);
     dh.segs = 2; dh.A2 = dB; dh.B2 = f32p(Wu);
     EC_KERNEL(nm.dgrad_h, 1, launch_simt_gemm(dh, st));
-    // dWd = U^T dO ; dWg = H^T dA ; dWu = H^T dB   (A[m][k] = U[k][m])
-    EC_KERNEL(nm.wgrad, 1,
-              launch_simt_gemm(sg(U, fs, F, false, dO, hs, d, false, dWd, wgs, d, F, d, M, E),
-                               st));
+    // dWg = H^T dA, dWu = H^T dB and dWd = U^T dO (A[m][k] = U[k][m]), the columns of dWd in two
+    // parts of whole 16-byte units
     SimtGemmArgs dw = sg(H, idx ? 0 : hs, d, false, dA, fs, F, false, dWg, wgs, F, d, F, M, E);
     dw.idx = idx; dw.idx_bs = M;
     dw.B2 = dB; dw.C2 = dWu;
-    EC_KERNEL(nm.wgrad, 1, launch_simt_gemm(dw, st));
+    const int h = (d / 2 + 3) / 4 * 4;
+    SimtGemmArgs dd = sg(U, fs, F, false, dO, hs, d, false, dWd, wgs, d, F, h, M, E);
+    dd.B2 = dO + h; dd.C2 = dWd + h; dd.N2 = d - h;
+    EC_KERNEL(nm.wgrad, 1, launch_simt_gemm_pair(dw, dd, st));
   }
   return EC_OK;
 }
@@ -618,13 +620,15 @@ ec_status run_backward(ec_ctx* c, const void* dY, void* dX, float* dWr, float* d
                                st));
     EC_KERNEL("dx_combine", nz,
               launch_dx_combine<T>(dH, slot, dXr, res, dHsh, static_cast<T*>(dX), N, E, M, d, st));
-    float* part = at<float>(c, c->o_part);
+    const bool one = c->wr_splits == 1;
+    float* part = one ? dWr : at<float>(c, c->o_part);
     SimtGemmArgs a = sg(f32p(c->X), 0, d, false, dZ, 0, E, false, part, 0, E, d, E, N, 1);
     a.splits = c->wr_splits;
     a.c_split = (int64_t)d * E;
     EC_KERNEL("router_wgrad_gemm", 1, launch_simt_gemm(a, st));
-    EC_KERNEL("router_wgrad_reduce", 1,
-              launch_reduce_splits(part, dWr, (int64_t)d * E, c->wr_splits, st));
+    if (!one)
+      EC_KERNEL("router_wgrad_reduce", 1,
+                launch_reduce_splits(part, dWr, (int64_t)d * E, c->wr_splits, st));
   }
   if (dbr && !fused) EC_KERNEL("router_dbias", 2, launch_colsum(dZ, dbr, N, E, colsum, st));
   return EC_OK;

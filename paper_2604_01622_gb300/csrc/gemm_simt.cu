@@ -74,7 +74,8 @@ __device__ __forceinline__ void store_group(float* dst, const float* v, int n, i
 // groups of RW and columns in CG groups of CW, spread evenly over the tile (so with two B
 // operands, each half of the tile's columns, it holds the same columns of both products).
 template <int BM, int BN, int BK, int TM, int TN, int MINB, bool A_K, bool B_K, int EPI>
-__global__ void __launch_bounds__(BM / TM * (BN / TN), MINB) simt_gemm_kernel(const SimtGemmArgs p) {
+__global__ void __launch_bounds__(BM / TM * (BN / TN), MINB)
+simt_gemm_kernel(const SimtGemmArgs p0, const SimtGemmArgs p1, int z1) {
   constexpr int TX = BN / TN, TY = BM / TM, NT = TX * TY;
   constexpr bool DUAL = EPI == SIMT_DUAL || EPI == SIMT_SWIGLU_FWD;
   constexpr int RW = TM >= 4 ? 4 : 2, RG = TM / RW;   // rows per group, groups per thread
@@ -91,9 +92,14 @@ __global__ void __launch_bounds__(BM / TM * (BN / TN), MINB) simt_gemm_kernel(co
   // and those of As four addresses
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ty = warp / (TX / 8) * 4 + (lane >> 3), tx = warp % (TX / 8) * 8 + (lane & 7);
-  const int b = blockIdx.z / p.splits, sp = blockIdx.z % p.splits;
+  // SIMT_DUAL: a second problem of the same form from grid layer z1 on
+  const bool other = EPI == SIMT_DUAL && (int)blockIdx.z >= z1;
+  const SimtGemmArgs p = other ? p1 : p0;
+  const int z = (int)blockIdx.z - (other ? z1 : 0);
+  const int b = z / p.splits, sp = z % p.splits;
   const int m0 = blockIdx.y * BM;
   const int n0 = blockIdx.x * (DUAL ? BN / 2 : BN);
+  if (EPI == SIMT_DUAL && (m0 >= p.M || n0 >= p.N)) return;   // the grid covers both problems
   const int kb = sp * p.kchunk, ke = min(p.K, kb + p.kchunk);
   const int ksl = (ke - kb + BK - 1) / BK;            // k-slices of one product
   const int nsl = p.segs * ksl;
@@ -145,13 +151,14 @@ __global__ void __launch_bounds__(BM / TM * (BN / TN), MINB) simt_gemm_kernel(co
       const int nn = B_K ? cm(c) : (c % (BN / 4)) * 4;   // column of the tile
       const bool h1 = DUAL && nn >= BN / 2;
       const float* Bp = h1 ? B1 : Bb;
+      const int N = h1 ? p.N2 : p.N;
       const int gn = n0 + (h1 ? nn - BN / 2 : nn);
       if constexpr (B_K) {
         const int gk = k0 + ck(c);
-        load4(rb[i], Bp + (int64_t)gn * p.b_ld + gk, gn < p.N ? gk : ke, ke, vb);
+        load4(rb[i], Bp + (int64_t)gn * p.b_ld + gk, gn < N ? gk : ke, ke, vb);
       } else {
         const int gk = k0 + c / (BN / 4);
-        load4(rb[i], Bp + (int64_t)gk * p.b_ld + gn, gk < ke ? gn : p.N, p.N, vb);
+        load4(rb[i], Bp + (int64_t)gk * p.b_ld + gn, gk < ke ? gn : N, N, vb);
       }
     }
   };
@@ -283,7 +290,7 @@ __global__ void __launch_bounds__(BM / TM * (BN / TN), MINB) simt_gemm_kernel(co
         const float* x = v + h * CW;
         const float* y = v + (CG / 2 + h) * CW;
         store_group<CW>(C + ro + n, x, n, p.N, p.vec_c);
-        store_group<CW>(C2 + ro + n, y, n, p.N, p.vec_c);
+        store_group<CW>(C2 + ro + n, y, n, p.N2, p.vec_c);
         if constexpr (EPI == SIMT_SWIGLU_FWD) {
           float u[CW];
 #pragma unroll
@@ -325,12 +332,15 @@ int simt_sms() {
 }
 
 template <int BM, int BN, int BK, int TM, int TN, int MINB, bool A_K, bool B_K, int EPI>
-cudaError_t go(const SimtGemmArgs& a, LaunchStream st) {
+cudaError_t go(const SimtGemmArgs& a, const SimtGemmArgs* a2, LaunchStream st) {
   constexpr bool DUAL = EPI == SIMT_DUAL || EPI == SIMT_SWIGLU_FWD;
   constexpr int cols = DUAL ? BN / 2 : BN;
-  const dim3 grid((a.N + cols - 1) / cols, (a.M + BM - 1) / BM, a.batch * a.splits);
+  const SimtGemmArgs& o = a2 ? *a2 : a;
+  const int N = a.N > o.N ? a.N : o.N, M = a.M > o.M ? a.M : o.M;
+  const int z1 = a.batch * a.splits;
+  const dim3 grid((N + cols - 1) / cols, (M + BM - 1) / BM, z1 + (a2 ? a2->batch * a2->splits : 0));
   return launch_kernel(simt_gemm_kernel<BM, BN, BK, TM, TN, MINB, A_K, B_K, EPI>, grid,
-                       BM / TM * (BN / TN), 0, st, 1, a);
+                       BM / TM * (BN / TN), 0, st, 1, a, o, z1);
 }
 
 // Tile shape: the one whose busiest SM has the least work, tiles per SM (rounded up) times the
@@ -342,13 +352,15 @@ cudaError_t go(const SimtGemmArgs& a, LaunchStream st) {
 // 279 us, down 123 against 140, dH 254 against 281), wide ones for the weight gradients (dWd 160
 // against 193) and dU; the small tiles for a few rows per expert (96 x 500 x 364: 27 against 43).
 template <bool A_K, bool B_K, int EPI>
-cudaError_t pick(const SimtGemmArgs& a, LaunchStream st) {
+cudaError_t pick(const SimtGemmArgs& a, const SimtGemmArgs* a2, LaunchStream st) {
   constexpr int half = (EPI == SIMT_DUAL || EPI == SIMT_SWIGLU_FWD) ? 2 : 1;
   constexpr bool TALL = A_K && EPI != SIMT_SWIGLU_BWD;
   const int64_t sms = simt_sms();
+  auto tiles_of = [&](const SimtGemmArgs& p, int bm, int bn) {
+    return (int64_t)((p.M + bm - 1) / bm) * (((int64_t)p.N * half + bn - 1) / bn) * p.batch * p.splits;
+  };
   auto cost = [&](int bm, int bn, double per_output) {
-    const int64_t tiles = (int64_t)((a.M + bm - 1) / bm) * (((int64_t)a.N * half + bn - 1) / bn) *
-                          a.batch * a.splits;
+    const int64_t tiles = tiles_of(a, bm, bn) + (a2 ? tiles_of(*a2, bm, bn) : 0);
     return (double)((tiles + sms - 1) / sms) * bm * bn * per_output;
   };
   const double c[4] = {cost(128, 128, 1.0), TALL ? cost(128, 64, 1.02) : cost(64, 128, 1.06),
@@ -357,15 +369,15 @@ cudaError_t pick(const SimtGemmArgs& a, LaunchStream st) {
   for (int i = 1; i < 4; ++i)
     if (c[i] < c[best]) best = i;
   switch (best) {
-    case 0: return go<128, 128, 16, 8, 8, 2, A_K, B_K, EPI>(a, st);
+    case 0: return go<128, 128, 16, 8, 8, 2, A_K, B_K, EPI>(a, a2, st);
     case 1:
       if constexpr (TALL)
-        return go<128, 64, 16, 8, 8, EPI == SIMT_SWIGLU_FWD ? 3 : 4, A_K, B_K, EPI>(a, st);
+        return go<128, 64, 16, 8, 8, EPI == SIMT_SWIGLU_FWD ? 3 : 4, A_K, B_K, EPI>(a, a2, st);
       else
-        return go<64, 128, 16, 8, 8, 4, A_K, B_K, EPI>(a, st);
-    case 2: return go<64, 64, 16, 8, 4, 4, A_K, B_K, EPI>(a, st);
+        return go<64, 128, 16, 8, 8, 4, A_K, B_K, EPI>(a, a2, st);
+    case 2: return go<64, 64, 16, 8, 4, 4, A_K, B_K, EPI>(a, a2, st);
   }
-  return go<32, 32, 32, 2, 4, 4, A_K, B_K, EPI>(a, st);
+  return go<32, 32, 32, 2, 4, 4, A_K, B_K, EPI>(a, a2, st);
 }
 
 bool vec_ok(const void* p, int64_t bs, int64_t ld, int contiguous) {
@@ -375,26 +387,37 @@ bool vec_ok(const void* p, int64_t bs, int64_t ld, int contiguous) {
 
 }  // namespace
 
-cudaError_t launch_simt_gemm(SimtGemmArgs a, LaunchStream st) {
-  if (a.M == 0 || a.N == 0 || a.batch == 0) return cudaSuccess;
+static void prepare(SimtGemmArgs& a) {
   const bool second_a = a.segs == 2;
   if (!a.A2) a.A2 = a.A;
   if (!a.B2) a.B2 = a.B;
+  if (a.N2 < 0) a.N2 = a.N;
   // split boundaries are multiples of 4, so a chunk of four k never crosses one
   a.kchunk = a.splits > 1 ? ((a.K + a.splits - 1) / a.splits + 3) / 4 * 4 : a.K;
   a.vec_a = vec_ok(a.A, a.a_bs, a.a_ld, a.a_kfast ? a.K : a.M) &&
             (!second_a || vec_ok(a.A2, a.a_bs, a.a_ld, a.a_kfast ? a.K : a.M));
   a.vec_b = vec_ok(a.B, a.b_bs, a.b_ld, a.b_kfast ? a.K : a.N) &&
-            vec_ok(a.B2, a.b_bs, a.b_ld, a.b_kfast ? a.K : a.N);
+            vec_ok(a.B2, a.b_bs, a.b_ld, a.b_kfast ? a.K : a.N2);
   a.vec_c = vec_ok(a.C, a.c_bs, a.c_ld, a.N) && a.c_split % 4 == 0 &&
-            (!a.C2 || vec_ok(a.C2, a.c_bs, a.c_ld, a.N)) &&
+            (!a.C2 || vec_ok(a.C2, a.c_bs, a.c_ld, a.N2)) &&
             (!a.C3 || vec_ok(a.C3, a.c_bs, a.c_ld, a.N));
-  if (a.C3) return pick<true, false, SIMT_SWIGLU_FWD>(a, st);
-  if (a.E1) return pick<true, true, SIMT_SWIGLU_BWD>(a, st);
-  if (a.C2) return pick<false, false, SIMT_DUAL>(a, st);
+}
+
+cudaError_t launch_simt_gemm(SimtGemmArgs a, LaunchStream st) {
+  if (a.M == 0 || a.N == 0 || a.batch == 0) return cudaSuccess;
+  prepare(a);
+  if (a.C3) return pick<true, false, SIMT_SWIGLU_FWD>(a, nullptr, st);
+  if (a.E1) return pick<true, true, SIMT_SWIGLU_BWD>(a, nullptr, st);
   if (a.a_kfast)
-    return a.b_kfast ? pick<true, true, SIMT_PLAIN>(a, st) : pick<true, false, SIMT_PLAIN>(a, st);
-  return pick<false, false, SIMT_PLAIN>(a, st);
+    return a.b_kfast ? pick<true, true, SIMT_PLAIN>(a, nullptr, st)
+                     : pick<true, false, SIMT_PLAIN>(a, nullptr, st);
+  return pick<false, false, SIMT_PLAIN>(a, nullptr, st);
+}
+
+cudaError_t launch_simt_gemm_pair(SimtGemmArgs a, SimtGemmArgs b, LaunchStream st) {
+  prepare(a);
+  prepare(b);
+  return pick<false, false, SIMT_DUAL>(a, &b, st);
 }
 
 // ------------------------------------------------------------------ router

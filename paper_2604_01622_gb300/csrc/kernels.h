@@ -109,7 +109,7 @@ cudaError_t launch_reduce_splits(const float* part, float* out, int64_t n, int s
 // dimension (k rows `ld` apart). With idx, A's rows (kfast) or k rows (else) are gathered:
 // row i is row idx[b*idx_bs + i] of A. Forms, by the pointers given:
 //   segs == 2       C = A.B + A2.B2 (two K loops, each rounded as its own sum)
-//   C2 (no C3, E1)  C = A.B, C2 = A.B2
+//   C2 (no C3, E1)  C = A.B (N columns), C2 = A.B2 (N2 <= N columns, N by default); pairs only
 //   C3              a = A.B, b = A.B2: C = a, C2 = b, C3 = silu(a) b
 //   E1              dU = A.B with a = E1, b = E2 (layout of C): C = dU b silu'(a), C2 = dU silu(a)
 //   splits > 1      (plain) split s of K writes C + s * c_split
@@ -123,12 +123,15 @@ struct SimtGemmArgs {
   float *C = nullptr, *C2 = nullptr, *C3 = nullptr;
   const float *E1 = nullptr, *E2 = nullptr;
   int64_t c_bs = 0, c_ld = 0, c_split = 0;
-  int M = 0, N = 0, K = 0, batch = 1, splits = 1, segs = 1;
+  int M = 0, N = 0, N2 = -1, K = 0, batch = 1, splits = 1, segs = 1;
   bool a_kfast = true, b_kfast = false;
   // set by the launcher
   int kchunk = 0;
   bool vec_a = false, vec_b = false, vec_c = false;
 };
 cudaError_t launch_simt_gemm(SimtGemmArgs a, LaunchStream st);
+// Two problems of the C2 form with both operands contiguous off K (the weight gradients), one
+// launch.
+cudaError_t launch_simt_gemm_pair(SimtGemmArgs a, SimtGemmArgs b, LaunchStream st);
 
 }  // namespace ecmoe

@@ -18,6 +18,7 @@ pytestmark = pytest.mark.gpu
     (900, 132, 14, 132, 130),     # 64 x 64, 14 experts
     (130, 68, 6, 36, 33),         # 32 x 32: one row past a tile
     (1000, 36, 70, 20, 40),       # 70 experts: two column tiles of the router
+    (60, 4, 3, 8, 9),             # the smallest width: the second half of dWd has no columns
     (40, 516, 5, 4, 7),           # 40 tokens, k loop of 516 = 8 slices and 4; d_ff one chunk
 ])
 def test_f32_layer_tile_edges(L, d, E, d_ff, k):
