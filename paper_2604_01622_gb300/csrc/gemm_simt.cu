@@ -13,8 +13,8 @@
 // 4 x 4 kernel with 4-byte loads before it ran 22 TFLOP/s on the same shapes (16 experts of 1000
 // rows, d 500, d_ff 364). The row gather of H = X[idx], the SwiGLU and its derivative, and the
 // second product of dH are part of the same launches, so no intermediate is written that a
-// later kernel only reads back: that layer's step 2820 -> 1387 us, a 256-token layer's (24
-// kernels, now 15) 195 -> 64-69 us, most of it host time by now.
+// later kernel only reads back: that layer's step 2820 -> 1304 us, a 256-token layer's (24
+// kernels, now 13) 195 -> 62-64 us, most of it host time by now.
 #include "common.cuh"
 #include "kernels.h"
 

@@ -45,6 +45,109 @@ __device__ __forceinline__ int token_pairs(const int* __restrict__ slot, const f
   return *s_cnt;
 }
 
+// ------------------------------------------------------------------ narrow rows
+// Rows of at most 32 16-byte units: a warp per token, four tokens per CTA, each warp listing its
+// token's rows for itself (a CTA per token would keep 8 of 128 threads busy at d 64). The sums
+// take up to eight rows at a time, in the order of the wide kernels.
+constexpr int kNarrow = 32, kNarrowWarps = 4;
+
+__device__ __forceinline__ int list_rows(const int* __restrict__ slot, const float* __restrict__ gate,
+                                         int t, int E, int M, int64_t* rows, float* gates) {
+  const int lane = threadIdx.x & 31;
+  int cnt = 0;
+  for (int e0 = 0; e0 < E; e0 += 32) {
+    const int e = e0 + lane;
+    const int m = e < E ? slot[(size_t)t * E + e] : -1;
+    const unsigned ball = __ballot_sync(0xffffffffu, m >= 0);
+    if (m >= 0) {
+      const int p = cnt + __popc(ball & ((1u << lane) - 1u));
+      const int64_t row = (int64_t)e * M + m;
+      rows[p] = row;
+      if (gates) gates[p] = __ldg(gate + row);
+    }
+    cnt += __popc(ball);
+  }
+  __syncwarp();
+  return cnt;
+}
+
+// out_t = b0_t + b1_t + b2_t (each if given, in this order) + sum of gate * row (gate NULL: 1).
+template <typename T>
+__global__ void __launch_bounds__(kNarrowWarps * 32)
+narrow_sum_kernel(const T* __restrict__ rows, const float* __restrict__ gate,
+                  const int* __restrict__ slot, const T* __restrict__ b0, const T* __restrict__ b1,
+                  const T* __restrict__ b2, T* __restrict__ out, int N, int E, int M, int nv) {
+  pdl_begin(rows, gate, slot, b0, b1, b2);
+  extern __shared__ int64_t sh_rows[];
+  const int warp = threadIdx.x >> 5, v = threadIdx.x & 31;
+  int64_t* s_row = sh_rows + (size_t)warp * E;
+  float* s_gate =
+      gate ? reinterpret_cast<float*>(sh_rows + (size_t)kNarrowWarps * E) + warp * E : nullptr;
+  const int t = blockIdx.x * kNarrowWarps + warp;
+  if (t >= N) return;
+  const int cnt = list_rows(slot, gate, t, E, M, s_row, s_gate);
+  if (v >= nv) return;
+  constexpr int VN = 16 / sizeof(T), PB = 8;
+  const uint4* ob = reinterpret_cast<const uint4*>(rows);
+  const int64_t base = (int64_t)t * nv + v;
+  float acc[VN], r[VN];
+  bool first = true;
+#pragma unroll
+  for (int j = 0; j < VN; ++j) acc[j] = 0.f;
+  auto add = [&](const T* b) {
+    if (!b) return;
+    unpack16(__ldg(reinterpret_cast<const uint4*>(b) + base), r, T());
+#pragma unroll
+    for (int j = 0; j < VN; ++j) acc[j] = first ? r[j] : acc[j] + r[j];
+    first = false;
+  };
+  add(b0);
+  add(b1);
+  add(b2);
+  for (int p = 0; p < cnt; p += PB) {
+    uint4 u[PB];
+#pragma unroll
+    for (int q = 0; q < PB; ++q)
+      u[q] = p + q < cnt ? __ldg(ob + s_row[p + q] * nv + v) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int q = 0; q < PB; ++q)
+      if (p + q < cnt) {
+        const float g = s_gate ? s_gate[p + q] : 1.0f;
+        unpack16(u[q], r, T());
+#pragma unroll
+        for (int j = 0; j < VN; ++j) acc[j] = fmaf(g, r[j], acc[j]);
+      }
+  }
+  reinterpret_cast<uint4*>(out)[base] = pack16(acc, T());
+}
+
+template <typename T>
+static cudaError_t launch_narrow_sum(const T* rows, const float* gate, const int* slot, const T* b0,
+                                     const T* b1, const T* b2, T* out, int N, int E, int M, int nv,
+                                     LaunchStream st) {
+  const size_t smem = (size_t)kNarrowWarps * E * (sizeof(int64_t) + (gate ? sizeof(float) : 0));
+  return launch_kernel(narrow_sum_kernel<T>, (N + kNarrowWarps - 1) / kNarrowWarps,
+                       kNarrowWarps * 32, smem, st, 1, rows, gate, slot, b0, b1, b2, out, N, E, M, nv);
+}
+
+// H[row] = X[t] for every row of token t (the token-major scatter below).
+template <typename T>
+__global__ void __launch_bounds__(kNarrowWarps * 32)
+narrow_scatter_kernel(const T* __restrict__ X, const int* __restrict__ slot, T* __restrict__ H, int N,
+                      int E, int M, int nv) {
+  pdl_begin(X, slot);
+  extern __shared__ int64_t sh_rows[];
+  const int warp = threadIdx.x >> 5, v = threadIdx.x & 31;
+  int64_t* s_row = sh_rows + (size_t)warp * E;
+  const int t = blockIdx.x * kNarrowWarps + warp;
+  if (t >= N) return;
+  const uint4 u = v < nv ? __ldg(reinterpret_cast<const uint4*>(X) + (int64_t)t * nv + v)
+                         : make_uint4(0, 0, 0, 0);
+  const int cnt = list_rows(slot, nullptr, t, E, M, s_row, nullptr);
+  if (v < nv)
+    for (int p = 0; p < cnt; ++p) reinterpret_cast<uint4*>(H)[s_row[p] * nv + v] = u;
+}
+
 // ------------------------------------------------------------------ combine Y_t = sum g * O
 template <typename T>
 __global__ void combine_kernel(const T* __restrict__ O, const float* __restrict__ gate,
@@ -122,6 +225,8 @@ template <typename T>
 cudaError_t launch_combine(const T* O, const float* gate, const int* slot, const T* R, const T* R2,
                            T* Y, int N, int E, int M, int d, LaunchStream st) {
   if (N == 0) return cudaSuccess;
+  if (d * (int)sizeof(T) / 16 <= kNarrow)
+    return launch_narrow_sum<T>(O, gate, slot, R, R2, nullptr, Y, N, E, M, d * (int)sizeof(T) / 16, st);
   const size_t smem = (size_t)3 * E * sizeof(int);
   // two 16-byte column groups per thread: half a row's groups per CTA, 32 to 128 threads
   const int nv = d * (int)sizeof(T) / 16;
@@ -177,6 +282,11 @@ template <typename T>
 cudaError_t launch_scatter_rows(const T* X, const int* slot, T* H, int N, int E, int M, int d,
                                 LaunchStream st, const int* count, const int* tiles) {
   if (N == 0) return cudaSuccess;
+  const int nv = d * (int)sizeof(T) / 16;
+  if (nv <= kNarrow && !count)
+    return launch_kernel(narrow_scatter_kernel<T>, (N + kNarrowWarps - 1) / kNarrowWarps,
+                         kNarrowWarps * 32, (size_t)kNarrowWarps * E * sizeof(int64_t), st, 1, X, slot,
+                         H, N, E, M, nv);
   const size_t smem = (size_t)2 * E * sizeof(int);
   return launch_kernel(scatter_rows_kernel<T>, N + (count ? E * kPadCtas : 0), 128, smem, st, 1, X,
                        slot, count, tiles, H, N, E, M, d);
@@ -627,6 +737,8 @@ cudaError_t launch_dx_combine(const T* dH, const int* slot, const T* dXr, const 
   if (N == 0) return cudaSuccess;
   const size_t smem = (size_t)2 * E * sizeof(int);
   const int nv = d * (int)sizeof(T) / 16;
+  if (nv <= kNarrow)
+    return launch_narrow_sum<T>(dH, nullptr, slot, dXr, R, R2, dX, N, E, M, nv, st);
   const int threads = std::min(128, std::max(32, (nv / 2 + 31) / 32 * 32));
   return launch_kernel(dx_combine_kernel<T>, N, threads, smem, st, 1, dH, slot, dXr, R, R2, dX, N, E,
                        M, d);
