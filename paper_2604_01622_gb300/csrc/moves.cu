@@ -46,10 +46,15 @@ __device__ __forceinline__ int token_pairs(const int* __restrict__ slot, const f
 }
 
 // ------------------------------------------------------------------ narrow rows
-// Rows of at most 32 16-byte units: a warp per token, four tokens per CTA, each warp listing its
-// token's rows for itself (a CTA per token would keep 8 of 128 threads busy at d 64). The sums
-// take up to eight rows at a time, in the order of the wide kernels.
-constexpr int kNarrow = 32, kNarrowWarps = 4;
+// Short rows take a warp per token, four tokens per CTA, each warp listing its token's rows for
+// itself: a CTA per token kept 8 of 128 threads busy at d 64 and paid a block barrier between the
+// slot map and the row loads. The sums take up to eight rows at a time, in the order of the wide
+// kernels. Limits in 16-byte units, measured both ways (bf16, us a launch): gather d 128 33 -> 12,
+// d 512 14 -> 10, d 768 22.5 -> 20.5, d 1024 27 -> 28.7; sums d 128 34 -> 23, d 384 equal, d 512
+// 14.3 -> 16.4 (fp32 d 256 10 -> 8).
+constexpr int kNarrowScatter = 96, kNarrowWarps = 4;
+template <typename T>
+constexpr int kNarrowSum = sizeof(T) == 4 ? 64 : 48;
 
 __device__ __forceinline__ int list_rows(const int* __restrict__ slot, const float* __restrict__ gate,
                                          int t, int E, int M, int64_t* rows, float* gates) {
@@ -79,46 +84,47 @@ narrow_sum_kernel(const T* __restrict__ rows, const float* __restrict__ gate,
                   const T* __restrict__ b2, T* __restrict__ out, int N, int E, int M, int nv) {
   pdl_begin(rows, gate, slot, b0, b1, b2);
   extern __shared__ int64_t sh_rows[];
-  const int warp = threadIdx.x >> 5, v = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int64_t* s_row = sh_rows + (size_t)warp * E;
   float* s_gate =
       gate ? reinterpret_cast<float*>(sh_rows + (size_t)kNarrowWarps * E) + warp * E : nullptr;
   const int t = blockIdx.x * kNarrowWarps + warp;
   if (t >= N) return;
   const int cnt = list_rows(slot, gate, t, E, M, s_row, s_gate);
-  if (v >= nv) return;
   constexpr int VN = 16 / sizeof(T), PB = 8;
   const uint4* ob = reinterpret_cast<const uint4*>(rows);
-  const int64_t base = (int64_t)t * nv + v;
-  float acc[VN], r[VN];
-  bool first = true;
+  for (int v = lane; v < nv; v += 32) {
+    const int64_t base = (int64_t)t * nv + v;
+    float acc[VN], r[VN];
+    bool first = true;
 #pragma unroll
-  for (int j = 0; j < VN; ++j) acc[j] = 0.f;
-  auto add = [&](const T* b) {
-    if (!b) return;
-    unpack16(__ldg(reinterpret_cast<const uint4*>(b) + base), r, T());
+    for (int j = 0; j < VN; ++j) acc[j] = 0.f;
+    auto add = [&](const T* b) {
+      if (!b) return;
+      unpack16(__ldg(reinterpret_cast<const uint4*>(b) + base), r, T());
 #pragma unroll
-    for (int j = 0; j < VN; ++j) acc[j] = first ? r[j] : acc[j] + r[j];
-    first = false;
-  };
-  add(b0);
-  add(b1);
-  add(b2);
-  for (int p = 0; p < cnt; p += PB) {
-    uint4 u[PB];
+      for (int j = 0; j < VN; ++j) acc[j] = first ? r[j] : acc[j] + r[j];
+      first = false;
+    };
+    add(b0);
+    add(b1);
+    add(b2);
+    for (int p = 0; p < cnt; p += PB) {
+      uint4 u[PB];
 #pragma unroll
-    for (int q = 0; q < PB; ++q)
-      u[q] = p + q < cnt ? __ldg(ob + s_row[p + q] * nv + v) : make_uint4(0, 0, 0, 0);
+      for (int q = 0; q < PB; ++q)
+        u[q] = p + q < cnt ? __ldg(ob + s_row[p + q] * nv + v) : make_uint4(0, 0, 0, 0);
 #pragma unroll
-    for (int q = 0; q < PB; ++q)
-      if (p + q < cnt) {
-        const float g = s_gate ? s_gate[p + q] : 1.0f;
-        unpack16(u[q], r, T());
+      for (int q = 0; q < PB; ++q)
+        if (p + q < cnt) {
+          const float g = s_gate ? s_gate[p + q] : 1.0f;
+          unpack16(u[q], r, T());
 #pragma unroll
-        for (int j = 0; j < VN; ++j) acc[j] = fmaf(g, r[j], acc[j]);
-      }
+          for (int j = 0; j < VN; ++j) acc[j] = fmaf(g, r[j], acc[j]);
+        }
+    }
+    reinterpret_cast<uint4*>(out)[base] = pack16(acc, T());
   }
-  reinterpret_cast<uint4*>(out)[base] = pack16(acc, T());
 }
 
 template <typename T>
@@ -137,15 +143,19 @@ narrow_scatter_kernel(const T* __restrict__ X, const int* __restrict__ slot, T* 
                       int E, int M, int nv) {
   pdl_begin(X, slot);
   extern __shared__ int64_t sh_rows[];
-  const int warp = threadIdx.x >> 5, v = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int64_t* s_row = sh_rows + (size_t)warp * E;
   const int t = blockIdx.x * kNarrowWarps + warp;
   if (t >= N) return;
-  const uint4 u = v < nv ? __ldg(reinterpret_cast<const uint4*>(X) + (int64_t)t * nv + v)
-                         : make_uint4(0, 0, 0, 0);
+  const uint4* src = reinterpret_cast<const uint4*>(X) + (int64_t)t * nv;
+  uint4* dst = reinterpret_cast<uint4*>(H);
+  uint4 u = lane < nv ? __ldg(src + lane) : make_uint4(0, 0, 0, 0);   // while the rows are listed
   const int cnt = list_rows(slot, nullptr, t, E, M, s_row, nullptr);
-  if (v < nv)
-    for (int p = 0; p < cnt; ++p) reinterpret_cast<uint4*>(H)[s_row[p] * nv + v] = u;
+  for (int v = lane; v < nv; v += 32) {
+    const uint4 next = v + 32 < nv && cnt ? __ldg(src + v + 32) : make_uint4(0, 0, 0, 0);
+    for (int p = 0; p < cnt; ++p) dst[s_row[p] * nv + v] = u;
+    u = next;
+  }
 }
 
 // ------------------------------------------------------------------ combine Y_t = sum g * O
@@ -225,7 +235,7 @@ template <typename T>
 cudaError_t launch_combine(const T* O, const float* gate, const int* slot, const T* R, const T* R2,
                            T* Y, int N, int E, int M, int d, LaunchStream st) {
   if (N == 0) return cudaSuccess;
-  if (d * (int)sizeof(T) / 16 <= kNarrow)
+  if (d * (int)sizeof(T) / 16 <= kNarrowSum<T>)
     return launch_narrow_sum<T>(O, gate, slot, R, R2, nullptr, Y, N, E, M, d * (int)sizeof(T) / 16, st);
   const size_t smem = (size_t)3 * E * sizeof(int);
   // two 16-byte column groups per thread: half a row's groups per CTA, 32 to 128 threads
@@ -283,7 +293,7 @@ cudaError_t launch_scatter_rows(const T* X, const int* slot, T* H, int N, int E,
                                 LaunchStream st, const int* count, const int* tiles) {
   if (N == 0) return cudaSuccess;
   const int nv = d * (int)sizeof(T) / 16;
-  if (nv <= kNarrow && !count)
+  if (nv <= kNarrowScatter && !count)
     return launch_kernel(narrow_scatter_kernel<T>, (N + kNarrowWarps - 1) / kNarrowWarps,
                          kNarrowWarps * 32, (size_t)kNarrowWarps * E * sizeof(int64_t), st, 1, X, slot,
                          H, N, E, M, nv);
@@ -737,7 +747,7 @@ cudaError_t launch_dx_combine(const T* dH, const int* slot, const T* dXr, const 
   if (N == 0) return cudaSuccess;
   const size_t smem = (size_t)2 * E * sizeof(int);
   const int nv = d * (int)sizeof(T) / 16;
-  if (nv <= kNarrow)
+  if (nv <= kNarrowSum<T>)
     return launch_narrow_sum<T>(dH, nullptr, slot, dXr, R, R2, dX, N, E, M, nv, st);
   const int threads = std::min(128, std::max(32, (nv / 2 + 31) / 32 * 32));
   return launch_kernel(dx_combine_kernel<T>, N, threads, smem, st, 1, dH, slot, dXr, R, R2, dX, N, E,
