@@ -421,13 +421,15 @@ cudaError_t launch_simt_gemm_pair(SimtGemmArgs a, SimtGemmArgs b, LaunchStream s
 }
 
 // ------------------------------------------------------------------ router
-// Scores of 32 tokens per CTA: logits X.Wr as one FMA chain per (token, expert) in ascending
+// Scores of RBM tokens per CTA: logits X.Wr as one FMA chain per (token, expert) in ascending
 // k, kept in shared memory (never written to global), then the row softmax, S, S^T and the
-// slot map's -1.
+// slot map's -1. Neither the chain nor the softmax depends on the tile: every variant gives the
+// same bits. A CTA is bound by its shared-memory reads (3 wavefronts per k and warp), so few tokens
+// want small tiles on many SMs and many tokens the larger tiles' reuse.
 namespace {
-constexpr int RBM = 32, RBK = 64;
+constexpr int RBK = 64;
 
-template <int BN, int TM, int TN>
+template <int RBM, int BN, int TM, int TN>
 __global__ void __launch_bounds__(RBM / TM * (BN / TN))
 router_f32_kernel(const float* __restrict__ X, const float* __restrict__ Wr,
                   const float* __restrict__ br, float* __restrict__ S, float* __restrict__ ST,
@@ -537,16 +539,16 @@ router_f32_kernel(const float* __restrict__ X, const float* __restrict__ Wr,
     }
   }
   __syncthreads();
-  for (int e = warp; e < E; e += nw) {
-    const int t = t0 + lane;
-    if (t < N) ST[(size_t)e * N + t] = tile[lane * (E + 1) + e];
+  for (int i = tid; i < E * RBM; i += NT) {
+    const int e = i / RBM, r = i % RBM;
+    if (t0 + r < N) ST[(size_t)e * N + t0 + r] = tile[r * (E + 1) + e];
   }
 }
 
-template <int BN, int TM, int TN>
+template <int RBM, int BN, int TM, int TN>
 cudaError_t router_go(const float* X, const float* Wr, const float* br, float* S, float* ST,
                       int* slot, int N, int d, int E, LaunchStream st) {
-  auto kern = router_f32_kernel<BN, TM, TN>;
+  auto kern = router_f32_kernel<RBM, BN, TM, TN>;
   const size_t smem =
       ((size_t)2 * RBK * (RBM + 4 + BN + 4) + (size_t)RBM * (E + 1)) * sizeof(float);
   if (smem > 48 * 1024) {
@@ -562,8 +564,21 @@ cudaError_t router_go(const float* X, const float* Wr, const float* br, float* S
 cudaError_t launch_router_f32(const float* X, const float* Wr, const float* br, float* S,
                               float* ST, int* slot, int N, int d, int E, LaunchStream st) {
   if (N == 0) return cudaSuccess;
-  if (E <= 16) return router_go<16, 2, 2>(X, Wr, br, S, ST, slot, N, d, E, st);
-  return router_go<64, 2, 4>(X, Wr, br, S, ST, slot, N, d, E, st);
+  // Tokens per CTA by how many 152 SMs get (1216 = 8 x 152 tokens, 4864 = 16 x 2 x 152, 9728 = 16
+  // x 4 x 152); one pass over X up to 128 experts. d 656, from 32 tokens x 64 experts (x 16 for
+  // E <= 16) per CTA for every size: 16 experts, 858 tokens 31 -> 19 us (16000: 47.5, and 48.5
+  // with 16 tokens); 30 experts, 858 36 -> 22, 16000 97 -> 65; 64 experts, 858 36 -> 24, 3000
+  // 50 -> 44, 16000 98 -> 71; 128 experts, 858 60 -> 32, 3000 89 -> 62, 16000 180 -> 120.
+  if (E <= 16)
+    return N <= 9728 ? router_go<16, 16, 2, 1>(X, Wr, br, S, ST, slot, N, d, E, st)
+                     : router_go<32, 16, 2, 2>(X, Wr, br, S, ST, slot, N, d, E, st);
+  if (E <= 32) return router_go<16, 32, 2, 2>(X, Wr, br, S, ST, slot, N, d, E, st);
+  if (E <= 64)
+    return N <= 1216   ? router_go<8, 64, 1, 4>(X, Wr, br, S, ST, slot, N, d, E, st)
+           : N <= 4864 ? router_go<16, 64, 2, 4>(X, Wr, br, S, ST, slot, N, d, E, st)
+                       : router_go<64, 64, 4, 4>(X, Wr, br, S, ST, slot, N, d, E, st);
+  return N <= 1216 ? router_go<16, 128, 2, 4>(X, Wr, br, S, ST, slot, N, d, E, st)
+                   : router_go<32, 128, 4, 4>(X, Wr, br, S, ST, slot, N, d, E, st);
 }
 
 }  // namespace ecmoe

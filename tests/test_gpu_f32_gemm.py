@@ -2,8 +2,7 @@
 oracle (relative max-norm 1e-4, the fp32 parity bound of the other tests): one shape per tile
 (128 x 128, 128 x 64 and 64 x 128, 64 x 64, 32 x 32), each with ragged row, column and k edges, an expert
 count that is not a multiple of 4 (scalar loads and stores in the router products), more than 64
-experts (several column tiles of the router kernel) and fewer than 64 tokens (one split of
-X^T dZ)."""
+experts (the router's widest tile) and fewer than 64 tokens (one split of X^T dZ)."""
 import pytest
 
 from paper_2604_01622_gb300 import inputs as I
@@ -17,7 +16,7 @@ pytestmark = pytest.mark.gpu
     (2000, 260, 16, 132, 260),    # half tiles
     (900, 132, 14, 132, 130),     # 64 x 64, 14 experts
     (130, 68, 6, 36, 33),         # 32 x 32: one row past a tile
-    (1000, 36, 70, 20, 40),       # 70 experts: two column tiles of the router
+    (1000, 36, 70, 20, 40),       # 70 experts: one 128-column tile of the router
     (60, 4, 3, 8, 9),             # the smallest width: the second half of dWd has no columns
     (40, 516, 5, 4, 7),           # 40 tokens, k loop of 516 = 8 slices and 4; d_ff one chunk
 ])
