@@ -652,7 +652,7 @@ def measure(w, args, device, ws, local, headline):
         per.setdefault(name, []).append(t)
     gemm = {k: v for k, v in per.items() if k.startswith("gemm_")}
     shared_ms = sum(sum(v) for k, v in per.items() if k.startswith("shared_")) / args.steps
-    gemm_launches = sum(len(v) for v in gemm.values())
+    gemm_launches = sum(len(v) for v in gemm.values()) + len(per.get("gemm_wgrad", []))
     gemm_ms_step = sum(sum(v) for v in gemm.values()) / args.steps
     P = sum(rows) / len(rows)
     flops_step = 18.0 * sum(rows) * w.d * w.d_ff

@@ -45,7 +45,7 @@ struct ec_ctx {
   // state saved by the forward pass
   bool residual = false;   // Y = X + EC(X), dX = dY + EC input gradient
   int Fs = 0;              // shared experts: total hidden width (0 = none)
-  size_t o_Ash = 0, o_Bsh = 0, o_Ush = 0, o_Osh = 0, o_dAsh = 0, o_dBsh = 0;
+  size_t o_Ash = 0, o_Bsh = 0, o_Ush = 0, o_Osh = 0, o_dAsh = 0, o_dBsh = 0, o_shpart = 0;
   const void *Wgs = nullptr, *Wus = nullptr, *Wds = nullptr;
   float *dWgs = nullptr, *dWus = nullptr, *dWds = nullptr;
   bool have_fwd = false;
@@ -182,6 +182,8 @@ void layout(ec_ctx* c) {
   c->o_Osh = take(Fs ? N * d * es : 0);
   c->o_dAsh = take(N * Fs * es);
   c->o_dBsh = take(N * Fs * es);
+  // two summands of the shared FFN's dWd (tensor cores, where its tiles fill the GPU badly)
+  c->o_shpart = take(use_tc(c) ? 2 * Fs * d * 4 : 0);
   c->o_dXr = take(N * d * es);   // the router's part of dX, in the layer dtype
   c->o_colsum = take((size_t)std::max(colsum_scratch_floats((int)N, (int)E),
                                        router_bwd_scratch_floats((int)N, (int)E)) * 4);
@@ -426,7 +428,8 @@ ec_status ffn_backward(ec_ctx* c, const FfnNames& nm, const T* dO, const T* H, c
                        const T* A, const T* B, const T* U, const void* Wg, const void* Wu,
                        const void* Wd,
                        T* dA, T* dB, T* dH, float* dWg, float* dWu, float* dWd, int E, int M, int F,
-                       LaunchStream st, const float* gate = nullptr, float* dgate_part = nullptr) {
+                       LaunchStream st, const float* gate = nullptr, float* dgate_part = nullptr,
+                       float* dwd_half = nullptr) {
   const int d = c->d;
   const int64_t P = (int64_t)E * M;
   if (P == 0) {
@@ -443,10 +446,13 @@ ec_status ffn_backward(ec_ctx* c, const FfnNames& nm, const T* dO, const T* H, c
     EC_KERNEL(nm.dgrad_h, 1,
               tc_expert_dgrad_h(dA, dB, Wg, Wu, dH, E, M, d, F, status, st, nullptr, c->tiles));
     int launched = 0;
+    bool halves = false;
     EC_KERNEL(nm.wgrad, 0,
               tc_expert_wgrad(H, U, dO, dA, dB, dWg, dWu, dWd, E, M, d, F, status, st, &launched,
-                              nullptr, c->tiles));
+                              nullptr, c->tiles, dwd_half, &halves));
     c->launches += launched;
+    if (halves)
+      EC_KERNEL(nm.wgrad, 1, launch_reduce_splits(dwd_half, dWd, (int64_t)F * d, 2, st));
   } else {
     const int64_t hs = (int64_t)M * d, fs = (int64_t)M * F, wgs = (int64_t)d * F;
     // dU = dO . Wd^T (B[k=i][n=j] = Wd[j][i]), its SwiGLU backward in the epilogue
@@ -578,7 +584,8 @@ ec_status run_backward(ec_ctx* c, const void* dY, void* dX, float* dWr, float* d
     EC_TRY(ffn_backward<T>(c, kShared, dYt, static_cast<const T*>(c->X), nullptr, at<T>(c, c->o_Ash),
                            at<T>(c, c->o_Bsh), at<T>(c, c->o_Ush), c->Wgs, c->Wus, c->Wds,
                            at<T>(c, c->o_dAsh), at<T>(c, c->o_dBsh), dh, dWgs, dWus, dWds, 1, N,
-                           Fs, st));
+                           Fs, st, nullptr, nullptr,
+                           use_tc(c) ? at<float>(c, c->o_shpart) : nullptr));
     dHsh = dh;
   }
   // router: dZ = S (dS - <dS,S>), dX = dZ Wr^T + sum dH, dWr = X^T dZ, dbr = sum dZ

@@ -1697,12 +1697,19 @@ cudaError_t tc_expert_dgrad_h(const void* dA, const void* dB, const void* Wg, co
 // [dWg | dWu][e] [d][F] = H[e]^T . [dA | dB][e] and dWd[e] [F][d] = U[e]^T . dO[e] (A[m][k=t] = H[t][m]
 // and U[t][m], MN-major). Up to 16 waves of tiles they are one tile list, so a launch, its ramp
 // and a partly empty last wave fall away: small ragged step 83 -> 76 us, 4096 tokens with 32
-// experts of d_ff 512 252 -> 246 us, and the shared experts' d_ff x d gradient needs no split over
-// K and no sum of its halves.
+// experts of d_ff 512 252 -> 246 us.
+//
+// One FFN over all tokens (the shared experts) has few tiles with a long K loop, and its last wave
+// can be nearly empty. With `half` (2 d_ff d floats) the down gradient may run as two halves of
+// the tokens, summed in order by launch_reduce_splits, where that fills the waves better. *halves
+// says so. A wide wave costs 1.83 narrow ones (1.78 where its launch holds one problem), the sum and
+// the extra launches about 30 k-slices of one and the time of the sum's bytes: 32768 tokens,
+// d = d_ff = 2048: one list 553 us, halves 516; d 1024 502 -> 328 the other way. Two launches of
+// whole problems where they take no more waves than one wide list: d 4096, d_ff 2048 1010 -> 992.
 cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const void* dA,
                             const void* dB, float* dWg, float* dWu, float* dWd, int E, int M,
                             int d, int F, int* status, LaunchStream st, int* launches,
-                            const VarRows* vr, int tiles) {
+                            const VarRows* vr, int tiles, float* half, bool* halves) {
   // Variable rows: the K loop of expert e runs over its own padded region (count rows,
   // rounded up to the 64-row k-step, the rest of which is zero in both operands).
   CUtensorMap ma0, ma1, mb0, mb1, mb2, mo0, mo1, mo2;
@@ -1714,9 +1721,10 @@ cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const 
   TC_TRY(make_out_map(&mo0, dWg, true, F, d, E));
   TC_TRY(make_out_map(&mo1, dWu, true, F, d, E));
   TC_TRY(make_out_map(&mo2, dWd, true, d, F, E));
-  // which: bit 0 the gate/up gradients, bit 1 the down gradient
-  auto go = [&](int which, bool wide) -> cudaError_t {
-    Args p = base_args(E, which & 1 ? d : 0, F, vr ? vr->P : M, wide ? 256 : 128, status);
+  // which: bit 0 the gate/up gradients, bit 1 the down gradient (batches: E, or 2 halves of one)
+  auto go = [&](int which, bool wide, int batches) -> cudaError_t {
+    Args p = base_args(batches, which & 1 ? d : 0, F, vr ? vr->P : batches > E ? M / 2 : M,
+                       wide ? 256 : 128, status);
     if (vr) {
       p.vm_tiles = vr->tiles;
       p.vm_count = vr->count;
@@ -1744,20 +1752,40 @@ cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const 
   const int pairs = sm_count() / 2 > 0 ? sm_count() / 2 : 1;
   const int64_t mt = (d + 255) / 256, mt2 = (F + 255) / 256;   // row tiles of the two problems
   const int64_t narrow = E * (mt * ((F + 127) / 128) + mt2 * ((d + 255) / 256));
+  const int64_t waves = (narrow + pairs - 1) / pairs;
   // Many tiles: two launches, down first (one list of both cost the 32768-token step of d 2048
-  // 1.6%, 7340 -> 7460 us). Two as well where only one problem has columns for wide tiles.
-  if (narrow > 16 * (int64_t)pairs || w0 != w1) {
-    TC_TRY(go(2, w1));
-    return go(1, w0);
+  // 1.6%, 7340 -> 7460 us). Two as well where only one problem has columns for wide tiles, unless
+  // the narrow ones are few (d = d_ff = 256, 32768 tokens: 502 -> 184 us).
+  bool wide = w0 && w1;
+  const int64_t wt0 = E * mt * (F / 256), wt1 = E * mt2 * (d / 512);   // wide tiles
+  const int64_t wide_waves = (wt0 + wt1 + pairs - 1) / pairs;
+  const int64_t wide_apart = (wt0 + pairs - 1) / pairs + (wt1 + pairs - 1) / pairs;
+  if (waves > 16 || (w0 != w1 && waves > 4) || (wide && wide_apart == wide_waves && wide_waves > 2 &&
+                                                2 * wide_waves <= waves)) {
+    TC_TRY(go(2, w1, E));
+    return go(1, w0, E);
   }
-  bool wide = w0;
-  if (wide && tiles == 0) {
+  if (wide && tiles == 0)
     // half as wide tiles where their last wave leaves less idle; one takes more than half of a
     // wide one's time (its MMAs wait longer for operands: 7% on the large shapes)
-    const int64_t nw = E * (mt * (F / 256) + mt2 * (d / 512));
-    wide = 2.0 * ((nw + pairs - 1) / pairs) <= 1.07 * ((narrow + pairs - 1) / pairs);
+    wide = 2.0 * wide_waves <= 1.07 * waves;
+  if (half && E == 1 && M % 2 == 0 && M >= 2048) {
+    const bool h1 = wide_cols(tiles, d, M / 2);
+    const int64_t t0 = w0 ? wt0 : mt * ((F + 127) / 128);
+    const int64_t t1 = 2 * (h1 ? mt2 * (d / 512) : mt2 * ((d + 255) / 256));
+    const double apart = (w0 ? 1.78 : 1.0) * ((t0 + pairs - 1) / pairs) +
+                         (h1 ? 0.89 : 0.5) * ((t1 + pairs - 1) / pairs) +
+                         (30.0 + 5e-6 * F * d) * BK / M;
+    if (apart < (wide ? 1.83 * wide_waves : 1.0 * waves)) {
+      TC_TRY(go(1, w0, 1));
+      TC_TRY(act_map(&ma1, U, F, 2, M / 2, nullptr, 64));
+      TC_TRY(act_map(&mb2, dO, d, 2, M / 2, nullptr, 64));
+      TC_TRY(make_out_map(&mo2, half, true, d, F, 2));
+      *halves = true;
+      return go(2, h1, 2);
+    }
   }
-  return go(3, wide);
+  return go(3, wide, E);
 }
 
 cudaError_t tc_router_dgrad(const void* dZb, const void* Wr, void* dXr, int N, int d, int E,

@@ -1,0 +1,46 @@
+"""The shared experts' weight gradients on each side of their tile rules: one list of tiles, the
+down gradient as two halves of the tokens (narrow and wide tiles, token counts whose half is and is
+not a multiple of the 64-row k-step), and one list of narrow tiles where only one of the two
+problems has columns for wide ones. Against the SwiGLU FFN in 64 bits, 2e-2 relative max-norm (the
+bf16 parity bound of the other tests)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2604_01622_gb300.layer import ECMoELayer
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("N,d,Fs", [
+    (8192, 832, 1600),     # halves, narrow tiles
+    (8196, 1600, 832),     # halves of 4098 tokens
+    (8193, 1600, 832),     # an odd count has no halves: one list
+    (16384, 4096, 1024),   # halves, wide tiles
+    (4096, 256, 256),      # wide columns for the gate/up gradients alone: one narrow list
+    (5000, 1024, 192),     # ... and for the down gradient alone
+])
+def test_shared_weight_gradients(N, d, Fs):
+    E, F = 4, 64
+    g = torch.Generator(device="cuda").manual_seed(N + d)
+
+    def r(*s, scale=1.0):
+        return (torch.randn(*s, device="cuda", generator=g) * scale).to(torch.bfloat16)
+
+    X, dY = r(N, d), r(N, d)
+    Wr, Wg, Wu, Wd = r(d, E, scale=.1), r(E, d, F), r(E, d, F), r(E, F, d)
+    sh = (r(d, Fs, scale=d ** -.5), r(d, Fs, scale=d ** -.5), r(Fs, d, scale=Fs ** -.5))
+    layer = ECMoELayer(N, d, E, F, np.array([0, N], np.int32), np.array([8], np.int32),
+                       d_ff_shared=Fs)
+    layer.forward(X, Wr, None, Wg, Wu, Wd, shared=sh)
+    got = layer.backward(dY)
+    layer.check()
+    x, dy, wg, wu, wd = (t.double() for t in (X, dY, *sh))
+    a, b = x @ wg, x @ wu
+    s = torch.sigmoid(a)
+    du = dy @ wd.T
+    ref = {"dWg_s": x.T @ (du * b * s * (1 + a * (1 - s))), "dWu_s": x.T @ (du * a * s),
+           "dWd_s": (a * s * b).T @ dy}
+    for k, want in ref.items():
+        err = ((got[k].double() - want).abs().max() / want.abs().max()).item()
+        assert err <= 2e-2, (k, err)
