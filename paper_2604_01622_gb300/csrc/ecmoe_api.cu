@@ -182,8 +182,8 @@ void layout(ec_ctx* c) {
   c->o_Osh = take(Fs ? N * d * es : 0);
   c->o_dAsh = take(N * Fs * es);
   c->o_dBsh = take(N * Fs * es);
-  // two summands of the shared FFN's dWd (tensor cores, where its tiles fill the GPU badly)
-  c->o_shpart = take(use_tc(c) ? 2 * Fs * d * 4 : 0);
+  // summands of the shared FFN's weight gradients (tensor cores, where its tiles fill the GPU badly)
+  c->o_shpart = take(use_tc(c) && Fs ? one_ffn_wgrad_scratch((int)N, (int)d, (int)Fs) * 4 : 0);
   c->o_dXr = take(N * d * es);   // the router's part of dX, in the layer dtype
   c->o_colsum = take((size_t)std::max(colsum_scratch_floats((int)N, (int)E),
                                        router_bwd_scratch_floats((int)N, (int)E)) * 4);
@@ -429,7 +429,7 @@ ec_status ffn_backward(ec_ctx* c, const FfnNames& nm, const T* dO, const T* H, c
                        const void* Wd,
                        T* dA, T* dB, T* dH, float* dWg, float* dWu, float* dWd, int E, int M, int F,
                        LaunchStream st, const float* gate = nullptr, float* dgate_part = nullptr,
-                       float* dwd_half = nullptr) {
+                       float* dw_scratch = nullptr) {
   const int d = c->d;
   const int64_t P = (int64_t)E * M;
   if (P == 0) {
@@ -446,13 +446,16 @@ ec_status ffn_backward(ec_ctx* c, const FfnNames& nm, const T* dO, const T* H, c
     EC_KERNEL(nm.dgrad_h, 1,
               tc_expert_dgrad_h(dA, dB, Wg, Wu, dH, E, M, d, F, status, st, nullptr, c->tiles));
     int launched = 0;
-    bool halves = false;
+    WgradParts parts;
     EC_KERNEL(nm.wgrad, 0,
               tc_expert_wgrad(H, U, dO, dA, dB, dWg, dWu, dWd, E, M, d, F, status, st, &launched,
-                              nullptr, c->tiles, dwd_half, &halves));
+                              nullptr, c->tiles, dw_scratch, &parts));
     c->launches += launched;
-    if (halves)
-      EC_KERNEL(nm.wgrad, 1, launch_reduce_splits(dwd_half, dWd, (int64_t)F * d, 2, st));
+    if (parts.splits)
+      EC_KERNEL(nm.wgrad, 1,
+                parts.all ? launch_reduce_splits(dw_scratch, dWg, (int64_t)F * d, parts.splits, st,
+                                                 dWu, dWd)
+                          : launch_reduce_splits(dw_scratch, dWd, (int64_t)F * d, parts.splits, st));
   } else {
     const int64_t hs = (int64_t)M * d, fs = (int64_t)M * F, wgs = (int64_t)d * F;
     // dU = dO . Wd^T (B[k=i][n=j] = Wd[j][i]), its SwiGLU backward in the epilogue

@@ -18,6 +18,7 @@
 // Operands may be K-major or MN-major in global memory (tensor-core transpose bits), so
 // no operand is ever repacked. Every mbarrier wait is bounded in time: on expiry the CTA
 // records DEV_TIMEOUT in the status word, all roles leave their loops, and TMEM is freed.
+#include <algorithm>
 #include <cuda.h>
 #include <cstdio>
 #include "common.cuh"
@@ -403,7 +404,7 @@ struct Tile {
 
 template <int VARM, int TM, bool TWO>
 __device__ __forceinline__ Tile tile_at(const Args& p, int tile, int tiles_per_b, uint32_t rank) {
-  static_assert(!TWO || VARM == 0 || VARM == 2, "two problems: batches over the experts");
+  static_assert(!TWO || VARM == 0 || VARM == 2 || VARM == 4, "two problems: batches of both");
   static_assert(VARM != 1 || TM == PADR, "variable-row tiles are one padding unit high");
   static_assert(VARM != 3 || TM == BM, "row-split tiles are one CTA high");
   Tile t;
@@ -1699,17 +1700,34 @@ cudaError_t tc_expert_dgrad_h(const void* dA, const void* dB, const void* Wg, co
 // and a partly empty last wave fall away: small ragged step 83 -> 76 us, 4096 tokens with 32
 // experts of d_ff 512 252 -> 246 us.
 //
-// One FFN over all tokens (the shared experts) has few tiles with a long K loop, and its last wave
-// can be nearly empty. With `half` (2 d_ff d floats) the down gradient may run as two halves of
-// the tokens, summed in order by launch_reduce_splits, where that fills the waves better. *halves
-// says so. A wide wave costs 1.83 narrow ones (1.78 where its launch holds one problem), the sum and
-// the extra launches about 30 k-slices of one and the time of the sum's bytes: 32768 tokens,
-// d = d_ff = 2048: one list 553 us, halves 516; d 1024 502 -> 328 the other way. Two launches of
-// whole problems where they take no more waves than one wide list: d 4096, d_ff 2048 1010 -> 992.
+// One FFN over all tokens (the shared experts) has few tiles with a long K loop. Tiles for half the
+// GPU or less run as several blocks of whole 64-token k-slices, at most a wave of them, summed in
+// order by launch_reduce_splits (32768 tokens, d = d_ff = 512: 184 -> 57 us; 6158 tokens, d 64,
+// d_ff 192: 43 -> 18). With more tiles the last wave can be nearly empty: there the down gradient
+// alone may run as two halves of the tokens, where that fills the waves better. A wide wave costs
+// 1.83 narrow ones (1.78 where its launch holds one problem), the sum and the extra launches about
+// 30 k-slices of one and the time of the sum's bytes: 32768 tokens, d = d_ff = 2048: one list 553
+// us, halves 516; d 1024 502 -> 328 the other way. Two launches of whole problems where they take
+// no more waves than one wide list: d 4096, d_ff 2048 1010 -> 992.
+static int one_ffn_wgrad_splits(int M, int d, int F) {
+  const int64_t tiles = (int64_t)((d + 255) / 256) * ((F + 127) / 128) +
+                        (int64_t)((F + 255) / 256) * ((d + 255) / 256);
+  const int blocks = (M + BK - 1) / BK;
+  const int s = (int)std::min<int64_t>(76 / std::max<int64_t>(tiles, 1), blocks / 8);
+  // the sum and its launch take about 30 k-slices
+  if (s < 2 || blocks - blocks / s <= 30) return 1;
+  const int per = (blocks + s - 1) / s;
+  return (blocks + per - 1) / per;
+}
+
+size_t one_ffn_wgrad_scratch(int M, int d, int F) {
+  return (size_t)std::max(2, 3 * one_ffn_wgrad_splits(M, d, F)) * d * F;
+}
+
 cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const void* dA,
                             const void* dB, float* dWg, float* dWu, float* dWd, int E, int M,
                             int d, int F, int* status, LaunchStream st, int* launches,
-                            const VarRows* vr, int tiles, float* half, bool* halves) {
+                            const VarRows* vr, int tiles, float* scratch, WgradParts* parts) {
   // Variable rows: the K loop of expert e runs over its own padded region (count rows,
   // rounded up to the 64-row k-step, the rest of which is zero in both operands).
   CUtensorMap ma0, ma1, mb0, mb1, mb2, mo0, mo1, mo2;
@@ -1746,6 +1764,22 @@ cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const 
     return launch<256, true, true, true, false, EPI_WGRAD, 6, 8, true>(ma0, ma1, mb0, mb1, mo0, mo1,
                                                                        mo2, p, st, &mb2);
   };
+  const int splits = scratch && E == 1 && !vr && tiles == 0 ? one_ffn_wgrad_splits(M, d, F) : 1;
+  if (splits > 1) {
+    const size_t n = (size_t)splits * d * F;
+    TC_TRY(make_out_map(&mo0, scratch, true, F, d, splits));
+    TC_TRY(make_out_map(&mo1, scratch + n, true, F, d, splits));
+    TC_TRY(make_out_map(&mo2, scratch + 2 * n, true, d, F, splits));
+    Args p = base_args(splits, d, F, M, 128, status);
+    p.k_blocks = (p.k_blocks + splits - 1) / splits;
+    p.M2 = F;
+    p.N2 = d;
+    p.n_tiles2 = (d + 255) / 256;
+    *parts = {splits, true};
+    ++*launches;
+    return launch<256, true, true, true, false, EPI_WGRAD, 6, 8, true, 4>(ma0, ma1, mb0, mb1, mo0, mo1,
+                                                                          mo2, p, st, &mb2);
+  }
   // K rows per expert (variable rows: on average)
   const int rows = vr ? vr->P / (E > 0 ? E : 1) : M;
   const bool w0 = wide_cols(tiles, 2 * F, rows), w1 = wide_cols(tiles, d, rows);
@@ -1769,7 +1803,7 @@ cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const 
     // half as wide tiles where their last wave leaves less idle; one takes more than half of a
     // wide one's time (its MMAs wait longer for operands: 7% on the large shapes)
     wide = 2.0 * wide_waves <= 1.07 * waves;
-  if (half && E == 1 && M % 2 == 0 && M >= 2048) {
+  if (scratch && E == 1 && M % 2 == 0 && M >= 2048) {
     const bool h1 = wide_cols(tiles, d, M / 2);
     const int64_t t0 = w0 ? wt0 : mt * ((F + 127) / 128);
     const int64_t t1 = 2 * (h1 ? mt2 * (d / 512) : mt2 * ((d + 255) / 256));
@@ -1780,8 +1814,8 @@ cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const 
       TC_TRY(go(1, w0, 1));
       TC_TRY(act_map(&ma1, U, F, 2, M / 2, nullptr, 64));
       TC_TRY(act_map(&mb2, dO, d, 2, M / 2, nullptr, 64));
-      TC_TRY(make_out_map(&mo2, half, true, d, F, 2));
-      *halves = true;
+      TC_TRY(make_out_map(&mo2, scratch, true, d, F, 2));
+      *parts = {2, false};
       return go(2, h1, 2);
     }
   }

@@ -69,13 +69,19 @@ cudaError_t tc_expert_dgrad_h(const void* dA, const void* dB, const void* Wg, co
 
 // Weight gradients per expert, fp32: dWd = U^T.dO, dWg = H^T.dA, dWu = H^T.dB, one kernel for
 // few tiles, else two; *launches counts them. With `vr`, each expert sums over its own rows (an
-// expert with none gets zeros). E = 1 with `half` (2 d_ff d floats): dWd may be left there as two
-// summands (*halves set), for the caller to add up.
+// expert with none gets zeros). E = 1 with `scratch` (one_ffn_wgrad_scratch floats): summands may be
+// left there, for the caller to add up: *parts says how many, of dWd [parts.splits][d_ff d] or,
+// with parts.all, of dWg, dWu and dWd in turn.
+struct WgradParts {
+  int splits = 0;
+  bool all = false;
+};
+size_t one_ffn_wgrad_scratch(int M, int d, int F);
 cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const void* dA,
                             const void* dB, float* dWg, float* dWu, float* dWd, int E, int M,
                             int d, int F, int* status, LaunchStream st, int* launches,
-                            const VarRows* vr = nullptr, int tiles = 0, float* half = nullptr,
-                            bool* halves = nullptr);
+                            const VarRows* vr = nullptr, int tiles = 0, float* scratch = nullptr,
+                            WgradParts* parts = nullptr);
 
 // Router backward on the tensor cores. dZb [2][N][Ep] bf16: hi and lo planes of the
 // zero-padded softmax gradient (dZ ~ hi + lo); Wr: the router weights as the forward pass read

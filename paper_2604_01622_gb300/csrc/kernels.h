@@ -100,8 +100,10 @@ cudaError_t launch_dx_combine(const T* dH, const int* slot, const T* dXr, const 
 cudaError_t launch_colsum(const float* Z, float* out, int N, int E, float* scratch,
                           LaunchStream st);
 int64_t colsum_scratch_floats(int N, int E);
+// out = sum of part [splits][n] in order; with out1 and out2 (both) three such arrays after one
+// another.
 cudaError_t launch_reduce_splits(const float* part, float* out, int64_t n, int splits,
-                                 LaunchStream st);
+                                 LaunchStream st, float* out1 = nullptr, float* out2 = nullptr);
 
 // ---------------------------------------------------------------- fp32 SIMT GEMM
 // C[b] = A[b].B[b], A logical [M][K], B logical [K][N], C [M][N] (row stride c_ld). Each operand

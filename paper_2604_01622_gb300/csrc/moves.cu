@@ -814,8 +814,11 @@ cudaError_t launch_colsum(const float* Z, float* out, int N, int E, float* scrat
 }
 
 __global__ void reduce_splits_kernel(const float* __restrict__ part, float* __restrict__ out,
-                                     int64_t n, int splits) {
+                                     float* __restrict__ out1, float* __restrict__ out2, int64_t n,
+                                     int splits) {
   pdl_begin(part);
+  part += blockIdx.y * splits * n;
+  if (blockIdx.y) out = blockIdx.y == 1 ? out1 : out2;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     // split order, eight loads in flight before they are added
@@ -834,10 +837,11 @@ __global__ void reduce_splits_kernel(const float* __restrict__ part, float* __re
 }
 
 cudaError_t launch_reduce_splits(const float* part, float* out, int64_t n, int splits,
-                                 LaunchStream st) {
+                                 LaunchStream st, float* out1, float* out2) {
   if (n == 0) return cudaSuccess;
   const unsigned blocks = grid_for(n, 152 * 16);
-  return launch_kernel(reduce_splits_kernel, blocks, 256, 0, st, 1, part, out, n, splits);
+  return launch_kernel(reduce_splits_kernel, dim3(blocks, out1 ? 3 : 1), 256, 0, st, 1, part, out,
+                       out1, out2, n, splits);
 }
 
 #define ECMOE_INST(T)                                                                            \

@@ -1,7 +1,7 @@
-"""The shared experts' weight gradients on each side of their tile rules: one list of tiles, the
-down gradient as two halves of the tokens (narrow and wide tiles, token counts whose half is and is
-not a multiple of the 64-row k-step), and one list of narrow tiles where only one of the two
-problems has columns for wide ones. Against the SwiGLU FFN in 64 bits, 2e-2 relative max-norm (the
+"""The shared experts' weight gradients on each side of their tile rules: few tiles as blocks of the
+tokens (the most and the fewest blocks, a short last one), one list of tiles, the down gradient as two
+halves of the tokens (narrow and wide tiles, token counts whose half is and is not a multiple of
+the 64-row k-step), and one list where only one of the two problems has columns for wide ones. Against the SwiGLU FFN in 64 bits, 2e-2 relative max-norm (the
 bf16 parity bound of the other tests)."""
 import numpy as np
 import pytest
@@ -17,8 +17,11 @@ pytestmark = pytest.mark.gpu
     (8196, 1600, 832),     # halves of 4098 tokens
     (8193, 1600, 832),     # an odd count has no halves: one list
     (16384, 4096, 1024),   # halves, wide tiles
-    (4096, 256, 256),      # wide columns for the gate/up gradients alone: one narrow list
-    (5000, 1024, 192),     # ... and for the down gradient alone
+    (13000, 64, 64),       # 2 tiles: 23 blocks of 9 k-slices, the last of 6
+    (4097, 256, 256),      # blocks, one token in the last slice
+    (3900, 1536, 384),     # 30 tiles: two blocks
+    (3840, 1536, 384),     # ... of 30 slices each, one list
+    (8192, 2048, 896),     # wide columns for the down gradient alone, few tiles
 ])
 def test_shared_weight_gradients(N, d, Fs):
     E, F = 4, 64
