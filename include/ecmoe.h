@@ -105,9 +105,9 @@ ec_status ec_ctx_set_residual(ec_ctx* ctx, int32_t on);
  * accumulator halves, else 256 x 256; with at most 128 rows per expert, 128-row tiles on single
  * SMs. EC_TILES_256 always takes 256 x 256; EC_TILES_512 takes 256 x 512 wherever the columns
  * fill it. All three give bit-identical results (every output is accumulated over K in the same
- * order, with the same epilogue arithmetic; only the tiling of the output differs). Takes effect
- * from the next call on the context; returns EC_ERR_INVALID_ARG for any other value (the context
- * keeps its policy). */
+ * order and the same partial sums, with the same epilogue arithmetic; only the tiling of the
+ * output differs). Takes effect from the next call on the context; returns EC_ERR_INVALID_ARG for
+ * any other value (the context keeps its policy). */
 enum { EC_TILES_AUTO = 0, EC_TILES_256 = 1, EC_TILES_512 = 2 };
 ec_status ec_ctx_set_tiles(ec_ctx* ctx, int32_t policy);
 

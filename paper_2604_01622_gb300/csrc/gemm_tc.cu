@@ -1724,6 +1724,56 @@ size_t one_ffn_wgrad_scratch(int M, int d, int F) {
   return (size_t)std::max(2, 3 * one_ffn_wgrad_splits(M, d, F)) * d * F;
 }
 
+// Tile widths and launches of the weight gradients under a tile policy; rows: K per expert (variable
+// rows: on average).
+struct WgradRule {
+  bool wide0, wide1;   // wide tiles for the gate/up and the down gradient, where they run apart
+  bool apart;          // two launches
+  bool wide;           // tiles of the one list
+  double waves;        // length of the one list, in waves of narrow tiles
+};
+
+static WgradRule wgrad_rule(int tiles, int E, int rows, int d, int F) {
+  WgradRule r{wide_cols(tiles, 2 * F, rows), wide_cols(tiles, d, rows), false, false, 0.0};
+  const int pairs = sm_count() / 2 > 0 ? sm_count() / 2 : 1;
+  const int64_t mt = (d + 255) / 256, mt2 = (F + 255) / 256;   // row tiles of the two problems
+  const int64_t narrow = E * (mt * ((F + 127) / 128) + mt2 * ((d + 255) / 256));
+  const int64_t waves = (narrow + pairs - 1) / pairs;
+  // Many tiles: two launches, down first (one list of both cost the 32768-token step of d 2048
+  // 1.6%, 7340 -> 7460 us). Two as well where only one problem has columns for wide tiles, unless
+  // the narrow ones are few (d = d_ff = 256, 32768 tokens: 502 -> 184 us).
+  r.wide = r.wide0 && r.wide1;
+  const int64_t wt0 = E * mt * (F / 256), wt1 = E * mt2 * (d / 512);   // wide tiles
+  const int64_t wide_waves = (wt0 + wt1 + pairs - 1) / pairs;
+  const int64_t wide_apart = (wt0 + pairs - 1) / pairs + (wt1 + pairs - 1) / pairs;
+  r.apart = waves > 16 || (r.wide0 != r.wide1 && waves > 4) ||
+            (r.wide && wide_apart == wide_waves && wide_waves > 2 && 2 * wide_waves <= waves);
+  if (r.wide && tiles == 0)
+    // half as wide tiles where their last wave leaves less idle; one takes more than half of a
+    // wide one's time (its MMAs wait longer for operands: 7% on the large shapes)
+    r.wide = 2.0 * wide_waves <= 1.07 * waves;
+  r.waves = r.wide ? 1.83 * wide_waves : 1.0 * waves;
+  return r;
+}
+
+// Whether the down gradient of one FFN over M tokens runs as two halves of them. The partial sums
+// show in the result's last bits, so this, like the number of blocks, is a rule on the sizes alone:
+// the tiles that EC_TILES_AUTO takes for them, whatever the policy of the call.
+static bool one_ffn_wgrad_halves(int M, int d, int F) {
+  if (M % 2 != 0 || M < 2048) return false;
+  const WgradRule r = wgrad_rule(0, 1, M, d, F);
+  if (r.apart) return false;
+  const int pairs = sm_count() / 2 > 0 ? sm_count() / 2 : 1;
+  const int64_t mt = (d + 255) / 256, mt2 = (F + 255) / 256;
+  const bool h1 = wide_cols(0, d, M / 2);
+  const int64_t t0 = r.wide0 ? mt * (F / 256) : mt * ((F + 127) / 128);
+  const int64_t t1 = 2 * mt2 * (h1 ? d / 512 : (d + 255) / 256);
+  const double apart = (r.wide0 ? 1.78 : 1.0) * ((t0 + pairs - 1) / pairs) +
+                       (h1 ? 0.89 : 0.5) * ((t1 + pairs - 1) / pairs) +
+                       (30.0 + 5e-6 * F * d) * BK / M;
+  return apart < r.waves;
+}
+
 cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const void* dA,
                             const void* dB, float* dWg, float* dWu, float* dWd, int E, int M,
                             int d, int F, int* status, LaunchStream st, int* launches,
@@ -1739,87 +1789,64 @@ cudaError_t tc_expert_wgrad(const void* H, const void* U, const void* dO, const 
   TC_TRY(make_out_map(&mo0, dWg, true, F, d, E));
   TC_TRY(make_out_map(&mo1, dWu, true, F, d, E));
   TC_TRY(make_out_map(&mo2, dWd, true, d, F, E));
-  // which: bit 0 the gate/up gradients, bit 1 the down gradient (batches: E, or 2 halves of one)
+  const bool one_ffn = scratch && E == 1 && !vr;
+  const int splits = one_ffn ? one_ffn_wgrad_splits(M, d, F) : 1;
+  // which: bit 0 the gate/up gradients, bit 1 the down gradient (batches: E, the token blocks of
+  // one FFN, or its 2 halves)
   auto go = [&](int which, bool wide, int batches) -> cudaError_t {
-    Args p = base_args(batches, which & 1 ? d : 0, F, vr ? vr->P : batches > E ? M / 2 : M,
-                       wide ? 256 : 128, status);
+    const bool blocks = splits > 1;
+    Args p = base_args(batches, which & 1 ? d : 0, F,
+                       vr ? vr->P : batches > E && !blocks ? M / 2 : M, wide ? 256 : 128, status);
     if (vr) {
       p.vm_tiles = vr->tiles;
       p.vm_count = vr->count;
       p.vm_E = E;
     }
+    if (blocks) p.k_blocks = (p.k_blocks + splits - 1) / splits;
     p.M2 = which & 2 ? F : 0;
     p.N2 = d;
     p.n_tiles2 = (d + (wide ? 511 : 255)) / (wide ? 512 : 256);
     ++*launches;
-    if (wide && vr)
-      return launch<512, true, true, true, false, EPI_WGRAD, kWideStages, 8, true, 2>(
-          ma0, ma1, mb0, mb1, mo0, mo1, mo2, p, st, &mb2);
     if (wide)
-      return launch<512, true, true, true, false, EPI_WGRAD, kWideStages, 8, true>(
-          ma0, ma1, mb0, mb1, mo0, mo1, mo2, p, st, &mb2);
-    if (vr)
-      return launch<256, true, true, true, false, EPI_WGRAD, 6, 8, true, 2>(
-          ma0, ma1, mb0, mb1, mo0, mo1, mo2, p, st, &mb2);
-    return launch<256, true, true, true, false, EPI_WGRAD, 6, 8, true>(ma0, ma1, mb0, mb1, mo0, mo1,
-                                                                       mo2, p, st, &mb2);
+      return vr ? launch<512, true, true, true, false, EPI_WGRAD, kWideStages, 8, true, 2>(
+                      ma0, ma1, mb0, mb1, mo0, mo1, mo2, p, st, &mb2)
+             : blocks ? launch<512, true, true, true, false, EPI_WGRAD, kWideStages, 8, true, 4>(
+                            ma0, ma1, mb0, mb1, mo0, mo1, mo2, p, st, &mb2)
+                      : launch<512, true, true, true, false, EPI_WGRAD, kWideStages, 8, true>(
+                            ma0, ma1, mb0, mb1, mo0, mo1, mo2, p, st, &mb2);
+    return vr ? launch<256, true, true, true, false, EPI_WGRAD, 6, 8, true, 2>(
+                    ma0, ma1, mb0, mb1, mo0, mo1, mo2, p, st, &mb2)
+           : blocks ? launch<256, true, true, true, false, EPI_WGRAD, 6, 8, true, 4>(
+                          ma0, ma1, mb0, mb1, mo0, mo1, mo2, p, st, &mb2)
+                    : launch<256, true, true, true, false, EPI_WGRAD, 6, 8, true>(
+                          ma0, ma1, mb0, mb1, mo0, mo1, mo2, p, st, &mb2);
   };
-  const int splits = scratch && E == 1 && !vr && tiles == 0 ? one_ffn_wgrad_splits(M, d, F) : 1;
   if (splits > 1) {
     const size_t n = (size_t)splits * d * F;
     TC_TRY(make_out_map(&mo0, scratch, true, F, d, splits));
     TC_TRY(make_out_map(&mo1, scratch + n, true, F, d, splits));
     TC_TRY(make_out_map(&mo2, scratch + 2 * n, true, d, F, splits));
-    Args p = base_args(splits, d, F, M, 128, status);
-    p.k_blocks = (p.k_blocks + splits - 1) / splits;
-    p.M2 = F;
-    p.N2 = d;
-    p.n_tiles2 = (d + 255) / 256;
     *parts = {splits, true};
-    ++*launches;
-    return launch<256, true, true, true, false, EPI_WGRAD, 6, 8, true, 4>(ma0, ma1, mb0, mb1, mo0, mo1,
-                                                                          mo2, p, st, &mb2);
+    // at most a wave of narrow tiles: wide ones only where the policy asks for them
+    const bool w0 = tiles == 2 && wide_cols(tiles, 2 * F, M), w1 = tiles == 2 && wide_cols(tiles, d, M);
+    if (w0 == w1) return go(3, w0, splits);
+    TC_TRY(go(2, w1, splits));
+    return go(1, w0, splits);
   }
-  // K rows per expert (variable rows: on average)
-  const int rows = vr ? vr->P / (E > 0 ? E : 1) : M;
-  const bool w0 = wide_cols(tiles, 2 * F, rows), w1 = wide_cols(tiles, d, rows);
-  const int pairs = sm_count() / 2 > 0 ? sm_count() / 2 : 1;
-  const int64_t mt = (d + 255) / 256, mt2 = (F + 255) / 256;   // row tiles of the two problems
-  const int64_t narrow = E * (mt * ((F + 127) / 128) + mt2 * ((d + 255) / 256));
-  const int64_t waves = (narrow + pairs - 1) / pairs;
-  // Many tiles: two launches, down first (one list of both cost the 32768-token step of d 2048
-  // 1.6%, 7340 -> 7460 us). Two as well where only one problem has columns for wide tiles, unless
-  // the narrow ones are few (d = d_ff = 256, 32768 tokens: 502 -> 184 us).
-  bool wide = w0 && w1;
-  const int64_t wt0 = E * mt * (F / 256), wt1 = E * mt2 * (d / 512);   // wide tiles
-  const int64_t wide_waves = (wt0 + wt1 + pairs - 1) / pairs;
-  const int64_t wide_apart = (wt0 + pairs - 1) / pairs + (wt1 + pairs - 1) / pairs;
-  if (waves > 16 || (w0 != w1 && waves > 4) || (wide && wide_apart == wide_waves && wide_waves > 2 &&
-                                                2 * wide_waves <= waves)) {
-    TC_TRY(go(2, w1, E));
-    return go(1, w0, E);
+  const WgradRule r = wgrad_rule(tiles, E, vr ? vr->P / (E > 0 ? E : 1) : M, d, F);
+  if (one_ffn && one_ffn_wgrad_halves(M, d, F)) {
+    TC_TRY(go(1, r.wide0, 1));
+    TC_TRY(act_map(&ma1, U, F, 2, M / 2, nullptr, 64));
+    TC_TRY(act_map(&mb2, dO, d, 2, M / 2, nullptr, 64));
+    TC_TRY(make_out_map(&mo2, scratch, true, d, F, 2));
+    *parts = {2, false};
+    return go(2, wide_cols(tiles, d, M / 2), 2);
   }
-  if (wide && tiles == 0)
-    // half as wide tiles where their last wave leaves less idle; one takes more than half of a
-    // wide one's time (its MMAs wait longer for operands: 7% on the large shapes)
-    wide = 2.0 * wide_waves <= 1.07 * waves;
-  if (scratch && E == 1 && M % 2 == 0 && M >= 2048) {
-    const bool h1 = wide_cols(tiles, d, M / 2);
-    const int64_t t0 = w0 ? wt0 : mt * ((F + 127) / 128);
-    const int64_t t1 = 2 * (h1 ? mt2 * (d / 512) : mt2 * ((d + 255) / 256));
-    const double apart = (w0 ? 1.78 : 1.0) * ((t0 + pairs - 1) / pairs) +
-                         (h1 ? 0.89 : 0.5) * ((t1 + pairs - 1) / pairs) +
-                         (30.0 + 5e-6 * F * d) * BK / M;
-    if (apart < (wide ? 1.83 * wide_waves : 1.0 * waves)) {
-      TC_TRY(go(1, w0, 1));
-      TC_TRY(act_map(&ma1, U, F, 2, M / 2, nullptr, 64));
-      TC_TRY(act_map(&mb2, dO, d, 2, M / 2, nullptr, 64));
-      TC_TRY(make_out_map(&mo2, scratch, true, d, F, 2));
-      *parts = {2, false};
-      return go(2, h1, 2);
-    }
+  if (r.apart) {
+    TC_TRY(go(2, r.wide1, E));
+    return go(1, r.wide0, E);
   }
-  return go(3, wide, E);
+  return go(3, r.wide, E);
 }
 
 cudaError_t tc_router_dgrad(const void* dZb, const void* Wr, void* dXr, int N, int d, int E,

@@ -7,6 +7,7 @@ import numpy as np
 import pytest
 import torch
 
+from paper_2604_01622_gb300 import EC_TILES_256, EC_TILES_512, EC_TILES_AUTO
 from paper_2604_01622_gb300.layer import ECMoELayer
 
 pytestmark = pytest.mark.gpu
@@ -47,3 +48,42 @@ def test_shared_weight_gradients(N, d, Fs):
     for k, want in ref.items():
         err = ((got[k].double() - want).abs().max() / want.abs().max()).item()
         assert err <= 2e-2, (k, err)
+
+
+def _shared_grads(N, d, Fs, policy):
+    """Gradients of a layer with shared experts under one tile policy."""
+    E, F = 4, 64
+    g = torch.Generator(device="cuda").manual_seed(N + d + Fs)
+
+    def r(*s, scale=1.0):
+        return (torch.randn(*s, device="cuda", generator=g) * scale).to(torch.bfloat16)
+
+    layer = ECMoELayer(N, d, E, F, np.array([0, N], np.int32), np.array([200], np.int32),
+                       d_ff_shared=Fs)
+    layer.set_tiles(policy)
+    layer.forward(r(N, d), r(d, E, scale=.1), None, r(E, d, F), r(E, d, F), r(E, F, d),
+                  shared=(r(d, Fs, scale=d ** -.5), r(d, Fs, scale=d ** -.5),
+                          r(Fs, d, scale=Fs ** -.5)))
+    got = layer.backward(r(N, d))
+    layer.check()
+    layer.close()
+    return got
+
+
+@pytest.mark.parametrize("N,d,Fs", [
+    (4097, 256, 256),      # blocks of the tokens, wide columns for the gate/up gradients
+    (13000, 512, 512),     # blocks, wide columns for all three
+    (3900, 512, 320),      # blocks, wide columns for the down gradient alone
+    (8192, 832, 1600),     # halves, no wide columns
+    (16384, 4096, 1024),   # halves, wide columns for all three
+    (8192, 2048, 896),     # one list, wide columns for the down gradient alone
+])
+def test_tile_policies_agree_with_shared_experts(N, d, Fs):
+    """The number of partial sums over the tokens follows from the sizes, not from the tile policy:
+    every gradient has the same bits under the three policies."""
+    want = _shared_grads(N, d, Fs, EC_TILES_AUTO)
+    for policy in (EC_TILES_256, EC_TILES_512):
+        got = _shared_grads(N, d, Fs, policy)
+        for k, t in want.items():
+            if t is not None:
+                assert torch.equal(got[k], t), (policy, k)
