@@ -1741,12 +1741,12 @@ static WgradRule wgrad_rule(int tiles, int E, int rows, int d, int F) {
   const int64_t waves = (narrow + pairs - 1) / pairs;
   // Many tiles: two launches, down first (one list of both cost the 32768-token step of d 2048
   // 1.6%, 7340 -> 7460 us). Two as well where only one problem has columns for wide tiles, unless
-  // the narrow ones are few (d = d_ff = 256, 32768 tokens: 502 -> 184 us).
+  // the narrow ones are few (d = d_ff = 256, 32768 tokens: 502 -> 184 us) and may be taken.
   r.wide = r.wide0 && r.wide1;
   const int64_t wt0 = E * mt * (F / 256), wt1 = E * mt2 * (d / 512);   // wide tiles
   const int64_t wide_waves = (wt0 + wt1 + pairs - 1) / pairs;
   const int64_t wide_apart = (wt0 + pairs - 1) / pairs + (wt1 + pairs - 1) / pairs;
-  r.apart = waves > 16 || (r.wide0 != r.wide1 && waves > 4) ||
+  r.apart = waves > 16 || (r.wide0 != r.wide1 && (waves > 4 || tiles == 2)) ||
             (r.wide && wide_apart == wide_waves && wide_waves > 2 && 2 * wide_waves <= waves);
   if (r.wide && tiles == 0)
     // half as wide tiles where their last wave leaves less idle; one takes more than half of a

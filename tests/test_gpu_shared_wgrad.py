@@ -51,7 +51,8 @@ def test_shared_weight_gradients(N, d, Fs):
 
 
 def _shared_grads(N, d, Fs, policy):
-    """Gradients of a layer with shared experts under one tile policy."""
+    """Gradients of a layer with shared experts under one tile policy, and the launches of its
+    backward pass."""
     E, F = 4, 64
     g = torch.Generator(device="cuda").manual_seed(N + d + Fs)
 
@@ -64,10 +65,12 @@ def _shared_grads(N, d, Fs, policy):
     layer.forward(r(N, d), r(d, E, scale=.1), None, r(E, d, F), r(E, d, F), r(E, F, d),
                   shared=(r(d, Fs, scale=d ** -.5), r(d, Fs, scale=d ** -.5),
                           r(Fs, d, scale=Fs ** -.5)))
+    before = layer.launches
     got = layer.backward(r(N, d))
+    launches = layer.launches - before
     layer.check()
     layer.close()
-    return got
+    return got, launches
 
 
 @pytest.mark.parametrize("N,d,Fs", [
@@ -81,9 +84,17 @@ def _shared_grads(N, d, Fs, policy):
 def test_tile_policies_agree_with_shared_experts(N, d, Fs):
     """The number of partial sums over the tokens follows from the sizes, not from the tile policy:
     every gradient has the same bits under the three policies."""
-    want = _shared_grads(N, d, Fs, EC_TILES_AUTO)
+    want, _ = _shared_grads(N, d, Fs, EC_TILES_AUTO)
     for policy in (EC_TILES_256, EC_TILES_512):
-        got = _shared_grads(N, d, Fs, policy)
+        got, _ = _shared_grads(N, d, Fs, policy)
         for k, t in want.items():
             if t is not None:
                 assert torch.equal(got[k], t), (policy, k)
+
+
+def test_wide_tiles_where_one_of_the_two_problems_fills_them():
+    """d 2048 fills wide tiles of the down gradient, the gate/up columns of d_ff 896 (shared) and 64
+    (routed) do not: EC_TILES_512 runs the two apart, each with its own tiles, where EC_TILES_256
+    has one list of narrow ones."""
+    narrow = _shared_grads(8192, 2048, 896, EC_TILES_256)[1]
+    assert _shared_grads(8192, 2048, 896, EC_TILES_512)[1] == narrow + 2
