@@ -549,11 +549,16 @@ template <int RBM, int BN, int TM, int TN>
 cudaError_t router_go(const float* X, const float* Wr, const float* br, float* S, float* ST,
                       int* slot, int N, int d, int E, LaunchStream st) {
   auto kern = router_f32_kernel<RBM, BN, TM, TN>;
-  const size_t smem =
-      ((size_t)2 * RBK * (RBM + 4 + BN + 4) + (size_t)RBM * (E + 1)) * sizeof(float);
-  if (smem > 48 * 1024) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto bytes = [](int experts) {
+    return ((size_t)2 * RBK * (RBM + 4 + BN + 4) + (size_t)RBM * (experts + 1)) * sizeof(float);
+  };
+  // narrow tiles are for up to BN experts; the limit, one for the process, covers every call's need
+  // (a call on another thread may come between this one's setting and its launch)
+  constexpr int most = BN < 128 ? BN : 512;
+  const size_t smem = bytes(E);
+  if (bytes(most) > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)bytes(most));
     if (e != cudaSuccess) return e;
   }
   return launch_kernel(kern, (N + RBM - 1) / RBM, RBM / TM * (BN / TN), smem, st, 1, X, Wr, br, S,

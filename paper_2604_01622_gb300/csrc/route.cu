@@ -621,6 +621,7 @@ __global__ void __launch_bounds__(NT, NT <= 512 ? 2 : 1) topk_block_kernel(TopkA
 // barriers (1-1.4 k cycles each with the search behind them); 64 columns of 131072 scores take
 // 52 us.
 constexpr int kTail = 512;
+constexpr int kClusterKeys = 49152;   // 192 KB of keys per CTA
 
 template <int CL>
 __global__ void __launch_bounds__(256, 4) topk_cluster_kernel(TopkArgs p, int chunk) {
@@ -989,32 +990,31 @@ __global__ void __launch_bounds__(512) topk_long_kernel(TopkArgs p) {
   }
 }
 
+// The limit on a kernel's shared memory is one for the process, so every call sets it to the most
+// that any call needs: a call on another thread may come between this one's setting and its launch.
 template <int CL>
 static cudaError_t topk_cluster(const TopkArgs& p, int G, int span, LaunchStream st) {
   auto kern = topk_cluster_kernel<CL>;
   const int chunk = ((span + CL - 1) / CL + 8 * kStep - 1) / (8 * kStep) * (8 * kStep);
-  const size_t smem = (size_t)chunk * 4;
-  if (smem > 40 * 1024) {   // with the static part above the 48 KB default
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  return launch_kernel(kern, dim3((unsigned)(p.E * CL), (unsigned)G), 256, smem, st, CL, p, chunk);
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kClusterKeys * 4);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(kern, dim3((unsigned)(p.E * CL), (unsigned)G), 256, (size_t)chunk * 4, st, CL,
+                       p, chunk);
 }
 
-template <int NT>
+// Columns of at most MAXK scores (with the places before the first one).
+template <int NT, int MAXK>
 static cudaError_t topk_block(const TopkArgs& p, int G, int span, LaunchStream st) {
   auto kern = topk_block_kernel<NT>;
   constexpr int unit = kStep * NT / 32;
+  static_assert(MAXK % unit == 0, "the longest column fills its places");
   const int chunk = (span + unit - 1) / unit * unit;
-  const size_t smem = ((size_t)chunk + kList) * 4;
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+                                             (MAXK + kList) * 4);
   if (e != cudaSuccess) return e;
-  return launch_kernel(kern, dim3(p.E, G), NT, smem, st, 1, p, chunk);
+  return launch_kernel(kern, dim3(p.E, G), NT, ((size_t)chunk + kList) * 4, st, 1, p, chunk);
 }
-
-constexpr int kClusterKeys = 49152;   // 192 KB of keys per CTA
 
 cudaError_t launch_topk(const TopkArgs& p, int G, int max_group, bool aligned, LaunchStream st) {
   if (G == 0 || p.E == 0) return cudaSuccess;
@@ -1029,8 +1029,8 @@ cudaError_t launch_topk(const TopkArgs& p, int G, int max_group, bool aligned, L
   if (span <= 2048) return launch_kernel(topk_reg_kernel<16, 128, 8>, grid, 128, 0, st, 1, p);
   if (span <= 4096) return launch_kernel(topk_reg_kernel<16, 256, 4>, grid, 256, 0, st, 1, p);
   if (span <= 8192) return launch_kernel(topk_reg_kernel<16, 512, 2>, grid, 512, 0, st, 1, p);
-  if (span <= 16384) return topk_block<512>(p, G, span, st);
-  if (span <= 49152) return topk_block<1024>(p, G, span, st);
+  if (span <= 16384) return topk_block<512, 16384>(p, G, span, st);
+  if (span <= 49152) return topk_block<1024, 49152>(p, G, span, st);
   if (span <= 8 * kClusterKeys) return topk_cluster<8>(p, G, span, st);
   return launch_kernel(topk_long_kernel, grid, 512, 0, st, 1, p);
 }
