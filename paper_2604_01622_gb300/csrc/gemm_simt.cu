@@ -15,6 +15,8 @@
 // second product of dH are part of the same launches, so no intermediate is written that a
 // later kernel only reads back: that layer's step 2820 -> 1304 us, a 256-token layer's (24
 // kernels, now 13) 195 -> 62-64 us, most of it host time by now.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -351,6 +353,7 @@ cudaError_t go(const SimtGemmArgs& a, const SimtGemmArgs* a2, LaunchStream st) {
 // leaves a nearly empty last wave, tall ones where A's rows are contiguous (gate/up 260 against
 // 279 us, down 123 against 140, dH 254 against 281), wide ones for the weight gradients (dWd 160
 // against 193) and dU; the small tiles for a few rows per expert (96 x 500 x 364: 27 against 43).
+// A grid has at most 65535 rows of tiles, which rules the small ones out from 2.1 million rows on.
 template <bool A_K, bool B_K, int EPI>
 cudaError_t pick(const SimtGemmArgs& a, const SimtGemmArgs* a2, LaunchStream st) {
   constexpr int half = (EPI == SIMT_DUAL || EPI == SIMT_SWIGLU_FWD) ? 2 : 1;
@@ -359,8 +362,9 @@ cudaError_t pick(const SimtGemmArgs& a, const SimtGemmArgs* a2, LaunchStream st)
   auto tiles_of = [&](const SimtGemmArgs& p, int bm, int bn) {
     return (int64_t)((p.M + bm - 1) / bm) * (((int64_t)p.N * half + bn - 1) / bn) * p.batch * p.splits;
   };
-  auto cost = [&](int bm, int bn, double per_output) {
+  auto cost = [&](int bm, int bn, double per_output) -> double {
     const int64_t tiles = tiles_of(a, bm, bn) + (a2 ? tiles_of(*a2, bm, bn) : 0);
+    if ((std::max(a.M, a2 ? a2->M : 0) - 1) / bm >= 65535) return INFINITY;
     return (double)((tiles + sms - 1) / sms) * bm * bn * per_output;
   };
   const double c[4] = {cost(128, 128, 1.0), TALL ? cost(128, 64, 1.02) : cost(64, 128, 1.06),

@@ -3,9 +3,12 @@ oracle (relative max-norm 1e-4, the fp32 parity bound of the other tests): one s
 (128 x 128, 128 x 64 and 64 x 128, 64 x 64, 32 x 32), each with ragged row, column and k edges, an expert
 count that is not a multiple of 4 (scalar loads and stores in the router products), more than 64
 experts (the router's widest tile) and fewer than 64 tokens (one split of X^T dZ)."""
+import numpy as np
 import pytest
+import torch
 
 from paper_2604_01622_gb300 import inputs as I
+from paper_2604_01622_gb300.layer import ECMoELayer
 from tests.test_gpu_parity import _check_layer
 
 pytestmark = pytest.mark.gpu
@@ -24,3 +27,32 @@ def test_f32_layer_tile_edges(L, d, E, d_ff, k):
     w = I.scaled(I.WORKLOADS["tiny_f32"], G=1, L=L, d=d, E=E, d_ff=d_ff, k_base=k, seed=31,
                  router_bias=True)
     _check_layer(I.make_inputs(w))
+
+
+def test_more_rows_than_a_grid_of_the_smallest_tiles():
+    """2.1 million rows per expert and d_ff 4: the smallest tile (32 rows) would need more than the
+    65535 tile rows a launch can have. Against the layer in 64 bits on the same selection."""
+    N, M, d, E, F = 2_100_200, 2_100_100, 4, 2, 4
+    g = torch.Generator(device="cuda").manual_seed(5)
+    X, dY, Wr, Wg, Wu, Wd = (torch.randn(s, device="cuda", generator=g) for s in
+                             ((N, d), (N, d), (d, E), (E, d, F), (E, d, F), (E, F, d)))
+    lay = ECMoELayer(N, d, E, F, np.array([0, N], np.int32), np.array([M], np.int32), dtype="f32")
+    Y, idx, gate, S = lay.forward(X, Wr, None, Wg, Wu, Wd)
+    got = lay.backward(dY)
+    lay.check()
+    x, dy, wg, wu, wd = (t.double() for t in (X, dY, Wg, Wu, Wd))
+    y = torch.zeros_like(x)
+    for e in range(E):
+        rows = idx[e].long()
+        h, do, gt = x[rows], dy[rows], gate[e].double()[:, None]
+        a, b = h @ wg[e], h @ wu[e]
+        s = torch.sigmoid(a)
+        u = a * s * b
+        y.index_add_(0, rows, gt * (u @ wd[e]))
+        du = (gt * do) @ wd[e].T
+        ref = {"dWg": h.T @ (du * b * s * (1 + a * (1 - s))), "dWu": h.T @ (du * a * s),
+               "dWd": u.T @ (gt * do)}
+        for k, want in ref.items():
+            err = ((got[k][e].double() - want).abs().max() / want.abs().max()).item()
+            assert err <= 1e-4, (k, e, err)
+    assert ((Y.double() - y).abs().max() / y.abs().max()).item() <= 1e-4
