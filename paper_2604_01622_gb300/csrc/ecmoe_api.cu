@@ -182,8 +182,6 @@ void layout(ec_ctx* c) {
   c->o_Osh = take(Fs ? N * d * es : 0);
   c->o_dAsh = take(N * Fs * es);
   c->o_dBsh = take(N * Fs * es);
-  // summands of the shared FFN's weight gradients (tensor cores, where its tiles fill the GPU badly)
-  c->o_shpart = take(use_tc(c) && Fs ? one_ffn_wgrad_scratch((int)N, (int)d, (int)Fs) * 4 : 0);
   c->o_dXr = take(N * d * es);   // the router's part of dX, in the layer dtype
   c->o_colsum = take((size_t)std::max(colsum_scratch_floats((int)N, (int)E),
                                        router_bwd_scratch_floats((int)N, (int)E)) * 4);
@@ -197,6 +195,9 @@ void layout(ec_ctx* c) {
     c->wr_splits = N <= 256 ? 1 : (int)std::min<size_t>(64, N / 64);
     c->o_part = take((size_t)c->wr_splits * d * E * 4);
   }
+  // summands of the shared FFN's weight gradients (tensor cores, where its tiles fill the GPU
+  // badly); last and in whole 256-byte units, so a write past them is one past the workspace
+  c->o_shpart = take(use_tc(c) && Fs ? one_ffn_wgrad_scratch((int)N, (int)d, (int)Fs) * 4 : 0);
   c->total = o;
 }
 

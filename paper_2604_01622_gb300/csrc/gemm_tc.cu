@@ -1721,7 +1721,8 @@ static int one_ffn_wgrad_splits(int M, int d, int F) {
 }
 
 size_t one_ffn_wgrad_scratch(int M, int d, int F) {
-  return (size_t)std::max(2, 3 * one_ffn_wgrad_splits(M, d, F)) * d * F;
+  const int splits = one_ffn_wgrad_splits(M, d, F);
+  return (size_t)(splits > 1 ? 3 * splits : 2) * d * F;   // three gradients, or dWd in halves
 }
 
 // Tile widths and launches of the weight gradients under a tile policy; rows: K per expert (variable

@@ -15,7 +15,7 @@ from tests._util import dev
 
 pytestmark = pytest.mark.gpu
 
-G = 1 << 16
+GUARD = 1 << 16
 PAT = 0xA5
 
 
@@ -23,12 +23,12 @@ class Guarded:
     def __init__(self, shape, dtype):
         n = int(np.prod(shape)) * torch.empty((), dtype=dtype).element_size()
         self.n = n
-        self.raw = torch.full((n + 2 * G,), PAT, dtype=torch.uint8, device="cuda")
-        self.t = self.raw[G:G + n].view(dtype).view(*shape) if n else torch.empty(
+        self.raw = torch.full((n + 2 * GUARD,), PAT, dtype=torch.uint8, device="cuda")
+        self.t = self.raw[GUARD:GUARD + n].view(dtype).view(*shape) if n else torch.empty(
             shape, dtype=dtype, device="cuda")
 
     def intact(self):
-        return bool((self.raw[:G] == PAT).all()) and bool((self.raw[G + self.n:] == PAT).all())
+        return bool((self.raw[:GUARD] == PAT).all()) and bool((self.raw[GUARD + self.n:] == PAT).all())
 
     @property
     def ptr(self):
@@ -57,12 +57,14 @@ def _check(bufs):
             assert torch.isfinite(b.t.float()).all(), name
 
 
-# (dtype, d, d_ff, tile policy): fp32 SIMT path; bf16 with 256-column tiles (d = 192 leaves a
-# ragged column tile); bf16 with 256 x 512 tiles (d and 2 d_ff multiples of 512)
-EC_SHAPES = [("f32", 68, 36, 0), ("bf16", 192, 128, 1), ("bf16", 512, 256, 2)]
+# (dtype, d, d_ff, tile policy), 110 rows per expert: fp32 SIMT path; bf16 with 256-column tiles
+# (d = 192 leaves a ragged column tile); bf16 with 256 x 512 tiles (d and 2 d_ff multiples of 512);
+# bf16 with the one-CTA tiles for at most 128 rows (ragged row and column tiles)
+EC_SHAPES = [("f32", 68, 36, 0), ("bf16", 192, 128, 1), ("bf16", 512, 256, 2), ("bf16", 192, 320, 0)]
 
 
-@pytest.mark.parametrize("dtype,d,d_ff,tiles", EC_SHAPES, ids=["f32", "bf16", "bf16_wide"])
+@pytest.mark.parametrize("dtype,d,d_ff,tiles", EC_SHAPES,
+                         ids=["f32", "bf16", "bf16_wide", "bf16_short_rows"])
 def test_expert_choice_writes_stay_inside_buffers(dtype, d, d_ff, tiles):
     from paper_2604_01622_gb300.layer import ECMoELayer
     base = I.WORKLOADS["tiny_f32"] if dtype == "f32" else I.WORKLOADS["ec_d2048_e64"]
@@ -123,20 +125,28 @@ def test_token_choice_writes_stay_inside_buffers(d, d_ff, tiles):
     lay.close()
 
 
-def test_shared_experts_writes_stay_inside_buffers():
-    """Shared experts over 2048 tokens: their FFN buffers and the two split-K halves of their
-    dWd (summed afterwards) stay inside the workspace; the shared gradients inside theirs."""
+@pytest.mark.parametrize("G,L,d,d_ff,Fs,tiles", [
+    (2, 1024, 512, 256, 512, 0),   # one list
+    (1, 4097, 256, 64, 256, 0),    # eight blocks of the tokens
+    (1, 13000, 512, 64, 512, 2),   # six blocks in 256 x 512 tiles
+    (1, 8192, 832, 64, 1600, 0),   # two halves of the tokens for the down gradient
+], ids=["list", "blocks", "blocks_wide", "halves"])
+def test_shared_experts_writes_stay_inside_buffers(G, L, d, d_ff, Fs, tiles):
+    """Shared experts: their FFN buffers stay inside the workspace, the shared gradients inside
+    theirs, and the summands of their weight gradients inside the scratch at the end of the
+    workspace, which the guard follows without a gap."""
     from paper_2604_01622_gb300.layer import ECMoELayer
-    w = I.scaled(I.WORKLOADS["ec_d2048_e64"], G=2, L=1024, d=512, E=6, d_ff=256, k_base=96,
+    w = I.scaled(I.WORKLOADS["ec_d2048_e64"], G=G, L=L, d=d, E=6, d_ff=d_ff, k_base=96,
                  router_bias=True, layers=1)
-    n_sh, f_sh = 2, 256
+    n_sh, f_sh = 2, Fs // 2
     inp = I.make_inputs(w)
     L = inp.layers[0]
     sh = I.make_shared(w, 0, n_sh, f_sh)
     lay = ECMoELayer(w.N, w.d, w.E, w.d_ff, inp.group_off, inp.k_g, dtype="bf16",
-                     d_ff_shared=n_sh * f_sh)
+                     d_ff_shared=Fs)
+    lay.set_tiles(tiles)
     ws = _guard_workspace(lay)
-    M, Fs = lay.M, n_sh * f_sh
+    M = lay.M
     out = {"Y": Guarded((w.N, w.d), torch.bfloat16), "idx": Guarded((w.E, M), torch.int32),
            "gate": Guarded((w.E, M), torch.float32), "S": Guarded((w.E, w.N), torch.float32)}
     X, Wr, Wg, Wu, Wd = dev(inp.X), dev(L.Wr), dev(L.Wg), dev(L.Wu), dev(L.Wd)
