@@ -1,8 +1,9 @@
 """The fp32 path's GEMMs at the sizes where a tile shape or a load form changes, against the
-oracle (relative max-norm 1e-4, the fp32 parity bound of the other tests): one shape per tile
-(128 x 128, 128 x 64 and 64 x 128, 64 x 64, 32 x 32), each with ragged row, column and k edges, an expert
-count that is not a multiple of 4 (scalar loads and stores in the router products), more than 64
-experts (the router's widest tile) and fewer than 64 tokens (one split of X^T dZ)."""
+oracle (relative max-norm 1e-4, the fp32 parity bound of the other tests). Every tile that a product
+can take runs with ragged row, column and k edges; the comments say which the choice by the busiest
+of 152 SMs gives. Also an expert count that is not a multiple of 4 (scalar loads and stores in the
+router products), more than 64 experts (the router's widest tile), fewer than 64 tokens (one split
+of X^T dZ) and more rows than a grid of the smallest tiles can have."""
 import numpy as np
 import pytest
 import torch
@@ -15,13 +16,18 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("L,d,E,d_ff,k", [
-    (3000, 260, 24, 132, 700),    # 128 x 128: a 60-row tail, 4 columns past a tile
-    (2000, 260, 16, 132, 260),    # half tiles
-    (900, 132, 14, 132, 130),     # 64 x 64, 14 experts
+    (337, 252, 65, 124, 117),     # 128 x 128 (gate/up, down, dH, weight gradients), 64 x 128 (dU)
+    (1421, 196, 7, 116, 1029),    # the same with 5 rows past a tile; 64 x 128 weight gradients
+    (406, 100, 16, 332, 262),     # 128 x 128 (dU, weight gradients), 64 x 64 (gate/up)
+    (4100, 252, 124, 4, 30),      # X^T dZ 128 x 128
+    (867, 360, 67, 4, 469),       # X^T dZ 64 x 128
+    (3000, 260, 24, 132, 700),    # 128 x 64 (gate/up, down, dH, dZ Wr^T): a 60-row tail
+    (2000, 260, 16, 132, 260),    # 64 x 64, 4 columns past a tile
+    (900, 132, 14, 132, 130),     # 128 x 64 (gate/up) and 64 x 64, 14 experts
     (130, 68, 6, 36, 33),         # 32 x 32: one row past a tile
     (1000, 36, 70, 20, 40),       # 70 experts: one 128-column tile of the router
     (60, 4, 3, 8, 9),             # the smallest width: the second half of dWd has no columns
-    (40, 516, 5, 4, 7),           # 40 tokens, k loop of 516 = 8 slices and 4; d_ff one chunk
+    (40, 516, 5, 4, 7),           # 40 tokens, k loop of 516 = 32 slices and 4; d_ff one chunk
 ])
 def test_f32_layer_tile_edges(L, d, E, d_ff, k):
     w = I.scaled(I.WORKLOADS["tiny_f32"], G=1, L=L, d=d, E=E, d_ff=d_ff, k_base=k, seed=31,

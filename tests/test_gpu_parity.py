@@ -111,7 +111,7 @@ def test_selection_degenerate_columns():
 
 
 def test_selection_long_groups_beyond_shared_memory():
-    """Groups longer than the shared-memory key buffer take the global-memory path."""
+    """Groups longer than one CTA's shared memory spread their keys over a cluster."""
     from paper_2604_01622_gb300.layer import ECMoELayer
     rng = np.random.default_rng(8)
     N, E = 60000, 3
