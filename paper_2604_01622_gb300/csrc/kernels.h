@@ -67,8 +67,8 @@ cudaError_t launch_scatter_rows(const T* X, const int* slot, T* H, int N, int E,
 template <typename T>
 cudaError_t launch_combine(const T* O, const float* gate, const int* slot, const T* R, const T* R2,
                            T* Y, int N, int E, int M, int d, LaunchStream st);
-// dO row r = gate[r] dY row idx[r], dgate[r] = <dY row idx[r], O row r> (zero rows where
-// idx[r] < 0), for the P rows (fp32 path).
+// dO row r = gate[r] dY row idx[r], dgate[r] = <dY row idx[r], O row r>, for the P rows (fp32
+// path).
 template <typename T>
 cudaError_t launch_bwd_gather_scale(const T* dY, const T* O, const int* idx, const float* gate,
                                     T* dO, float* dgate, int64_t P, int d, LaunchStream st);

@@ -324,12 +324,6 @@ __global__ void bwd_gather_scale_kernel(const T* __restrict__ dY, const T* __res
   const float g = gate[row];
   constexpr int VN = 16 / sizeof(T);
   const int nv = d / VN;
-  if (t < 0) {   // padding row: zero gradient row, zero gate gradient
-    uint4* out = reinterpret_cast<uint4*>(dO + (size_t)row * d);
-    for (int v = lane; v < nv; v += 32) out[v] = make_uint4(0, 0, 0, 0);
-    if (lane == 0) dgate[row] = 0.f;
-    return;
-  }
   const uint4* dy = reinterpret_cast<const uint4*>(dY + (size_t)t * d);
   const uint4* o = reinterpret_cast<const uint4*>(O + (size_t)row * d);
   uint4* out = reinterpret_cast<uint4*>(dO + (size_t)row * d);

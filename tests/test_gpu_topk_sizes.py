@@ -1,8 +1,8 @@
 """Selection at the column lengths where the top-k kernel changes form (scores per thread,
 threads, keys in shared memory from 8193 scores, over a cluster of eight CTAs from 49153, and the
-scan over global memory above 393216), on columns that
-start on and off the 16-byte grid, and the output forms of ec_route: scores returned in place,
-to an array that the kernels cannot write directly, and not at all. Exact against the oracle."""
+scan over global memory above 393216), on columns that start on and off the 16-byte grid, and the
+output forms of ec_route: scores returned in place, to an array that the kernels cannot write
+directly, and not at all. Exact against the oracle."""
 import numpy as np
 import pytest
 import torch
