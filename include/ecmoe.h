@@ -23,7 +23,7 @@
  *     M = sum_g k_g: row e holds expert e's tokens, group g at offsets
  *     k_off[g] .. k_off[g+1]-1 where k_off is the prefix sum of k_g.
  *   - Device pointers must be 16-byte aligned. On the bf16 path d and d_ff must be
- *     multiples of 64.
+ *     multiples of 64, on the fp32 path of 4.
  *   - Every compute call is asynchronous on `stream` (a cudaStream_t, NULL for the
  *     legacy default stream) and does no host synchronisation. Argument errors are
  *     returned before anything is launched. A kernel that gives up on a bounded
@@ -133,9 +133,10 @@ ec_status ec_route(ec_ctx* ctx, const void* X, const void* Wr, const float* br,
                    const float* S_in, float* S_out, int32_t* idx, float* gate, void* stream);
 
 /* Whole-layer forward (Sec. 2.2): Y [N][d] in the context's dtype. idx, gate, S_out as in
- * ec_route (each may be NULL). Saves what ec_moe_backward needs in the workspace, and
- * remembers the weight pointers, which must stay valid and unchanged until the backward
- * call. Wg, Wu [E][d][d_ff]; Wd [E][d_ff][d]. */
+ * ec_route (each may be NULL). Saves activations and selection for ec_moe_backward in the
+ * workspace, and remembers the pointers of X, Wr and the expert weights, which must stay valid
+ * and unchanged until the backward call (so Y may not overwrite X if one follows). Wg, Wu
+ * [E][d][d_ff]; Wd [E][d_ff][d]. */
 ec_status ec_moe_forward(ec_ctx* ctx, const void* X, const void* Wr, const float* br,
                          const void* Wg, const void* Wu, const void* Wd, void* Y,
                          int32_t* idx, float* gate, float* S_out, void* stream);
