@@ -86,10 +86,14 @@ ec_status cuda_fail(ec_ctx* c, cudaError_t e, const char* where) {
   } while (0)
 
 // Small calls overlap each kernel's start with the end of the one before it; large ones do not.
-// Measured (forward + backward, expert rows x d x d_ff): 0.09 G 123 -> 93 us, 8.6 G 290 -> 259
-// us; at 137 G 32768 tokens with 128 experts lost 2% (2360 -> 2410 us: near the power limit the
-// gaps between kernels are not idle time lost) and 8192 tokens with 64 experts gained 1%. Forward
-// alone: 4.3 G 200 -> 187 us, 21 G 222 -> 210 us.
+// Measured without and with it (us, forward | forward + backward; product = expert rows x d x
+// d_ff): 0.09 G | 123 -> 93; 17 G, 32768 rows 139 -> 128 | 402 -> 382; 34 G, 32768 rows 261 -> 252 |
+// 750 -> 733, 65536 rows 271 -> 260 | 794 -> 779; 48 G, 22912 rows 334 -> 324 | 1008 -> 1000. The
+// product does not decide alone. Where the rows are many and short the gaps between kernels are
+// a small part of the time: 524288 rows of d 256, 17 G 342 -> 347 | 915 -> 908 and 34 G 459 -> 454 |
+// 1280 -> 1313. Past the limit few rows still gain (69 G, 32768 rows 369 -> 362 | 1170 -> 1162; 103 G,
+// 49152 rows 541 -> 534 | 1653 -> 1652) and many lose in the step (69 G, 131072 rows 434 -> 434 | 1268
+// -> 1281, 262144 rows 483 -> 480 | 1393 -> 1431; 137 G, 262144 rows | 2360 -> 2410).
 constexpr double kOverlapMax = 5e10;
 LaunchStream launch_stream(const ec_ctx* c, void* stream) {
   const double rows = c->tc_k ? (double)c->N * c->tc_k : (double)c->E * c->M;

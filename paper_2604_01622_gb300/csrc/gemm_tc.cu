@@ -1713,7 +1713,7 @@ static int one_ffn_wgrad_splits(int M, int d, int F) {
   const int64_t tiles = (int64_t)((d + 255) / 256) * ((F + 127) / 128) +
                         (int64_t)((F + 255) / 256) * ((d + 255) / 256);
   const int blocks = (M + BK - 1) / BK;
-  const int s = (int)std::min<int64_t>(76 / std::max<int64_t>(tiles, 1), blocks / 8);
+  const int s = (int)std::min<int64_t>(kSms / 2 / std::max<int64_t>(tiles, 1), blocks / 8);
   // the sum and its launch take about 30 k-slices
   if (s < 2 || blocks - blocks / s <= 30) return 1;
   const int per = (blocks + s - 1) / s;
@@ -1878,7 +1878,7 @@ cudaError_t tc_router_dgrad(const void* dZb, const void* Wr, void* dXr, int N, i
 // back.
 int router_wgrad_splits(int N, int d, int Ep) {
   const int tiles = ((d + BM - 1) / BM) * ((Ep + 127) / 128), blocks = (N + BK - 1) / BK;
-  const int want = tiles < 152 ? 152 / tiles : 1;
+  const int want = tiles < kSms ? kSms / tiles : 1;
   const int most = blocks / 2 > 0 ? blocks / 2 : 1;
   const int s = want < most ? want : most;
   const int per = (blocks + s - 1) / s;

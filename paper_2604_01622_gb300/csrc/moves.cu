@@ -662,10 +662,10 @@ cudaError_t launch_reduce_partials(const float* part, float* out, int rows, int 
                   (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
   const int64_t n = (int64_t)rows * cols / (v4 ? 4 : 1);
   // few outputs: 64-thread CTAs spread them over more SMs
-  const int nt = n < 152 * 256 ? 64 : 256;
+  const int nt = n < kSms * 256 ? 64 : 256;
   const int64_t blocks = (n + nt - 1) / nt;
   return launch_kernel(v4 ? reduce_partials_kernel<4> : reduce_partials_kernel<1>,
-                       (unsigned)(blocks < 152 * 16 ? blocks : 152 * 16), nt, 0, st, 1, part, out,
+                       (unsigned)(blocks < kSms * 16 ? blocks : kSms * 16), nt, 0, st, 1, part, out,
                        rows, cols, ld, splits);
 }
 
@@ -833,7 +833,7 @@ __global__ void reduce_splits_kernel(const float* __restrict__ part, float* __re
 cudaError_t launch_reduce_splits(const float* part, float* out, int64_t n, int splits,
                                  LaunchStream st, float* out1, float* out2) {
   if (n == 0) return cudaSuccess;
-  const unsigned blocks = grid_for(n, 152 * 16);
+  const unsigned blocks = grid_for(n, kSms * 16);
   return launch_kernel(reduce_splits_kernel, dim3(blocks, out1 ? 3 : 1), 256, 0, st, 1, part, out,
                        out1, out2, n, splits);
 }
