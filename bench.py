@@ -42,7 +42,7 @@ UNIT = "tokens/s"
 # counters were taken on 1, 2 and 4 of the workload's 8 sequences (captures of a few GB); each
 # launch's traffic is affine in the sequences (within 1.4%) and is extrapolated to 8.
 TILE_POLICY = {"auto": 0, "256": 1, "512": 2}   # EC_TILES_AUTO / EC_TILES_256 / EC_TILES_512
-TRAFFIC = {"d35aded7c71d": 2865896485}
+TRAFFIC = {"778f6190cc7e": 2843681871}
 
 
 def _peaks():
@@ -715,7 +715,9 @@ def run_ours(args):
     hbm, bf16_burst, bf16_sust, peak_src = _peaks()
     gemm_tflops = res["gemm_tflops"]
     src = os.path.join(ROOT, "paper_2604_01622_gb300", "csrc", "gemm_tc.cu")
-    tr = TRAFFIC.get(_src_hash(src))
+    # captured on the default workload's expert-choice step
+    tr = (TRAFFIC.get(_src_hash(src)) if w is I.WORKLOADS["ec_d2048_e64"] and not tc
+          and args.tiles == "auto" else None)
     roofline = {
         "kernel": "tc_gemm_kernel (tcgen05 grouped expert GEMMs: gate/up, down, dU, dH, dW)",
         "bound": "tensor", "achieved": round(gemm_tflops, 1),
